@@ -243,7 +243,6 @@ int run_evaluate(const gp_node *progs, const int32_t *offsets, int n_progs, cons
                  int32_t *out_status, cudaStream_t st, int64_t ld = -1) {
     if (ld < 0) ld = n_rows;
     const bool mom = metric == GP_PEARSON;
-    GP_CUDA(cudaMemsetAsync(W.counters, 0, 8 * sizeof(unsigned long long), st));
     CompileArgs ca{progs, offsets, n_progs, n_feat, W.code, W.meta,
                    c->status, nullptr};
     if (mom) {
@@ -253,9 +252,11 @@ int run_evaluate(const gp_node *progs, const int32_t *offsets, int n_progs, cons
     }
     GP_CUDA(launch_compile(ca, st));
     const bool split = pl.o.long_edge > 0;
-    GP_CUDA(launch_order(W.meta, n_progs, W.order, W.class_count, st, 0, split ? pl.o.long_edge : 0));
-    GP_CUDA(launch_sumw(w, n_rows, W.sumw_part, W.sumw, st));
-    if (mom) GP_CUDA(launch_ystats(y, w, n_rows, W.sumw, W.ystat_part, W.ystat, st));
+    GP_CUDA(launch_order(W.meta, n_progs, W.order, W.class_count, st, W.counters, 0,
+                         split ? pl.o.long_edge : 0, w ? nullptr : W.sumw, n_rows));
+    if (w) GP_CUDA(launch_sumw(w, n_rows, W.sumw_part, W.sumw, W.counters + kTicket, st));
+    if (mom)
+        GP_CUDA(launch_ystats(y, w, n_rows, W.sumw, W.ystat_part, W.ystat, W.counters + kTicket, st));
     const int fmode = (n_feat <= 2) ? 2 : 0;
     // the moment epilogue has instances for 4 and 8 rows per thread
     const int rpt = (mom && pl.o.rows_per_thread == 16) ? 8 : pl.o.rows_per_thread;
@@ -356,8 +357,7 @@ int run_predict_compiled(const Workspace &W, int p0, int b, const float *X, int6
                          int n_feat, float *out_pred, DevCtx *c, cudaStream_t st, int rpt = 4) {
     const int64_t chunk = std::min<int64_t>(round_up(n_rows, 256), 4096);
     const int n_chunks = (int)((n_rows + chunk - 1) / chunk);
-    GP_CUDA(cudaMemsetAsync(W.counters, 0, 8 * sizeof(unsigned long long), st));
-    GP_CUDA(launch_order(W.meta + p0, b, W.order, W.class_count, st));
+    GP_CUDA(launch_order(W.meta + p0, b, W.order, W.class_count, st, W.counters));
     const bool vec = aligned16(X) && (n_rows % 4 == 0);
     const int fmode = (n_feat <= 2) ? 2 : 0;
     for (int cls = 0; cls < kNumClasses; ++cls) {
@@ -574,7 +574,10 @@ int gp_evaluate_plain(const gp_node *progs, const int32_t *offsets, int n_progs,
     CompileArgs ca{progs, offsets, n_progs, n_feat, W.code, W.meta,
                    c->status, nullptr};
     GP_CUDA(launch_compile(ca, st));
-    GP_CUDA(launch_sumw(w, n_rows, W.sumw_part, W.sumw, st));
+    // (no program reads the order here)
+    GP_CUDA(launch_order(W.meta, n_progs, W.order, W.class_count, st, W.counters, 0, 0,
+                         w ? nullptr : W.sumw, n_rows));
+    if (w) GP_CUDA(launch_sumw(w, n_rows, W.sumw_part, W.sumw, W.counters + kTicket, st));
     PlainArgs pa{progs, offsets, W.meta, X, n_rows, n_rows, y, w, metric, n_blocks, W.part};
     for (int p = 0; p < n_progs; ++p) GP_CUDA(launch_plain(pa, p, st));
     FinalizeArgs fa{};
@@ -714,13 +717,13 @@ int gp_const_grad(const gp_node *progs, const int32_t *offsets, int n_progs, con
     }
     Workspace W = carve(c->ws, L, true);
     cudaStream_t st = S(stream);
-    GP_CUDA(cudaMemsetAsync(W.counters, 0, 8 * sizeof(unsigned long long), st));
     CompileArgs ca{progs, offsets, n_progs, n_feat, W.code, W.meta,
                    c->status, nullptr};
     ca.grad = 1;  // the gradient form: no constant folding, marker words
     GP_CUDA(launch_compile(ca, st));
-    GP_CUDA(launch_order(W.meta, n_progs, W.order, W.class_count, st, 1));
-    GP_CUDA(launch_sumw(w, n_rows, W.sumw_part, W.sumw, st));
+    GP_CUDA(launch_order(W.meta, n_progs, W.order, W.class_count, st, W.counters, 1, 0,
+                         w ? nullptr : W.sumw, n_rows));
+    if (w) GP_CUDA(launch_sumw(w, n_rows, W.sumw_part, W.sumw, W.counters + kTicket, st));
     // one launch per bucket (constants, stack depth) of the compiled programs
     const bool vec = aligned16(X) && aligned16(y) && (!w || aligned16(w)) && (n_rows % 4 == 0) &&
                      (chunk % 4 == 0);

@@ -149,7 +149,7 @@ constexpr int kOrderClasses = 5;
 
 // Workspace carved out of one device allocation (all offsets 256-aligned).
 struct Workspace {
-    unsigned long long *counters;  // [8] work-queue counters
+    unsigned long long *counters;  // [8] work-queue counters; [kTicket] grid sums' ticket
     double *sumw;                  // [1] total weight
     double *sumw_part;             // [kSumwBlocks]
     uint2 *code;                   // [P][kCodeStride], the gradient form [P][kGradCodeStride]
@@ -168,6 +168,7 @@ struct Workspace {
 };
 
 constexpr int kSumwBlocks = 512;
+constexpr int kTicket = 7;  // counters[kTicket]
 
 struct Layout {
     size_t counters, sumw, sumw_part, code, meta, order, class_count, part;
@@ -209,16 +210,20 @@ struct CompileArgs {
 };
 cudaError_t launch_compile(const CompileArgs &a, cudaStream_t st);
 // weighted mean of y and the moments of yc = fl(y - fl(ybar)) (FP64,
-// fixed partition); needs the total weight already in *sumw
+// fixed partition); needs the total weight already in *sumw.  ticket: a
+// zeroed word, zero again afterwards
 cudaError_t launch_ystats(const float *y, const float *w, int64_t n_rows, const double *sumw,
-                          double *part, double *ystat, cudaStream_t st);
-// mode 0 with edge > 0 also writes to class_count[kOrderClasses] how many
-// class-0 programs have more than `edge` compiled words (the long bucket,
-// which the order puts first)
-cudaError_t launch_order(const ProgMeta *meta, int n_progs, int32_t *order,
-                         int32_t *class_count, cudaStream_t st, int mode = 0, int edge = 0);
-cudaError_t launch_sumw(const float *w, int64_t n_rows, double *part,
-                        double *sumw, cudaStream_t st);
+                          double *part, double *ystat, unsigned long long *ticket, cudaStream_t st);
+// the program order; clears the workspace's counters.  mode 0 with edge > 0
+// also writes to class_count[kOrderClasses] how many class-0 programs have
+// more than `edge` compiled words (the long bucket, which the order puts
+// first); with sumw it writes n_rows there (the total weight without weights)
+cudaError_t launch_order(const ProgMeta *meta, int n_progs, int32_t *order, int32_t *class_count,
+                         cudaStream_t st, unsigned long long *counters, int mode = 0, int edge = 0,
+                         double *sumw = nullptr, int64_t n_rows = 0);
+// the total of the weights w (not null); ticket as above
+cudaError_t launch_sumw(const float *w, int64_t n_rows, double *part, double *sumw,
+                        unsigned long long *ticket, cudaStream_t st);
 
 struct EvalArgs {
     const uint2 *code;
