@@ -17,7 +17,9 @@ same bits; the constants are written here as the bit patterns that
 gp_math.cuh's static_asserts pin.  Code size matters as much as
 instruction count (at 8 rows per lane an unrolled body per operation
 overflowed the instruction cache: ncu's no_instruction stall rose to 4 per
-issue), so the division forms share one body (the divisor staged in U;
+issue; the same bodies as scalar FFMA, a packed one costing two issue slots
+anyway, took a third more code and Pagie-1 16M x 4096 from 301 to 398 ms),
+so the division forms share one body (the divisor staged in U;
 the reversed forms swap the rows into U first), sin and cos share one,
 and tan goes to the C++ switch.
 
@@ -46,7 +48,7 @@ OPS = dict(PUSH_X=0, PUSH_C=1, PUSH_X_SP=2, PUSH_C_SP=3, ADD_S=4, SUB_S=5, MUL_S
 COL1 = 32
 
 # float bit patterns (pinned by static_asserts in gp_math.cuh)
-K = dict(inv_pi=0x3EA2F983, magic=0x4B400000, pi_hi=0x40490FDB, pi_mid=0xB3BBBD2E,
+K = dict(inv_pi=0x3EA2F983, magic=0x4B400000, magic1=0x4B400001, pi_hi=0x40490FDB, pi_mid=0xB3BBBD2E,
          pi_lo=0xA7772CED, q0=0xBE2AAAA6, q1=0x3C088769, q2=0xB94FB7D4, q3=0x362EDC67,
          trig_fast=0x47800000,
          lp0=0xBEFFFFFD, lp1=0x3EAAAB7A, lp2=0xBE80024D, lp3=0x3E4C6960, lp4=0xBE29AE98,
@@ -208,7 +210,9 @@ class Gen:
     # sin or cos of every row (the steps of sincos_fast): one body for
     # both, the kind (0 sin, 1 cos) from the dispatch index.  j = the
     # integer nearest x/pi - kind/2, r = x - (j + kind/2) pi, then one odd
-    # polynomial, negated when j + kind is odd (a sign-bit flip)
+    # polynomial, negated when j + kind is odd.  The rounding constant of cos
+    # is one more than that of sin, so that in both the low bit of the rounded
+    # sum says whether to negate
     def trig(self, src=None, dst=None, kind=None):
         """sin/cos of the pairs src(i) into dst(i) (default: the rows, in
         place, after the range test, the kind from the dispatch index); a
@@ -221,16 +225,15 @@ class Gen:
             self.e("setp.ne.u32 %%p, %%kd, 0;")
             self.e("selp.b64 %%KM, 0xBF000000BF000000, 0x8000000080000000, %%p;")  # -kind/2
             self.e("selp.b64 %%F, 0x3F0000003F000000, 0x0000000000000000, %%p;")   # +kind/2
-            self.e("shl.b32 %%kd, %%kd, 31;")
+            self.e(f"selp.b64 %%K1, {kp('magic1')}, {kp('magic')}, %%p;")
         else:
             self.e("mov.b64 %%KM, " + ("0xBF000000BF000000;" if kind else "0x8000000080000000;"))
             self.e("mov.b64 %%F, " + ("0x3F0000003F000000;" if kind else "0x0000000000000000;"))
-            self.e(f"mov.b32 %%kd, {0x80000000 if kind else 0};")
+            self.e(f"mov.b64 %%K1, {kp('magic1' if kind else 'magic')};")
         for i in range(self.np):
             t = src(i)
             self.e(f"mov.b64 %%K0, {kp('inv_pi')};")
             self.e(f"fma.rn.f32x2 %%JM, {t}, %%K0, %%KM;")
-            self.e(f"mov.b64 %%K1, {kp('magic')};")
             self.e("add.rn.f32x2 %%JM, %%JM, %%K1;")
             self.e("sub.rn.f32x2 %%JJ, %%JM, %%K1;")
             self.e("add.rn.f32x2 %%JJ, %%JJ, %%F;")
@@ -244,23 +247,22 @@ class Gen:
             self.e("mul.rn.f32x2 %%S, %%R, %%R;")
             # sin r = r + (s r)(Q0 + s (Q1 + s (Q2 + s Q3)))
             self.e(f"mov.b64 %%K0, {kp('q3')};")
-            self.e(f"mov.b64 %%K1, {kp('q2')};")
-            self.e("fma.rn.f32x2 %%P, %%K0, %%S, %%K1;")
+            self.e(f"mov.b64 %%P, {kp('q2')};")
+            self.e("fma.rn.f32x2 %%P, %%K0, %%S, %%P;")
             for c in ("q1", "q0"):
                 self.e(f"mov.b64 %%K0, {kp(c)};")
                 self.e("fma.rn.f32x2 %%P, %%P, %%S, %%K0;")
             self.e("mul.rn.f32x2 %%Q, %%S, %%R;")
             self.e("fma.rn.f32x2 %%P, %%P, %%Q, %%R;")
-            self.unpack(i, "%%n0", "%%n1", "%%JM")   # bit 0: parity of j
-            self.unpack(i, "%%v0", "%%v1", "%%P")
+            # bit 0 of the sum: negate.  Times 2^31 plus the result's bits
+            # flips its sign in one instruction (with the scaling of exp and
+            # -b shared by the quotient's steps: sin 94 -> 85 instructions a
+            # word of 8 rows, div 94 -> 90; 10M x 28 type tables 1.7% faster)
+            self.unpack(i, "%%n0", "%%n1", "%%JM")
+            self.e("mov.b64 {%%m0, %%m1}, %%P;")
             for r in (0, 1):
-                n, v = f"%%n{r}", f"%%v{r}"
-                self.e(f"shl.b32 {n}, {n}, 31;")
-                self.e(f"xor.b32 {n}, {n}, %%kd;")
-                self.e(f"mov.b32 %%a, {v};")
-                self.e(f"xor.b32 %%a, %%a, {n};")
-                self.e(f"mov.b32 {v}, %%a;")
-            self.pack(i, "%%v0", "%%v1", dst(i) if dst else None)
+                self.e(f"mad.lo.u32 %%m{r}, %%n{r}, 0x80000000, %%m{r};")
+            self.e(f"mov.b64 {dst(i) if dst else self.T[i]}, {{%%m0, %%m1}};")
 
     # log of every row (f_log: the logarithm of max(|t|, thr), 0 below the
     # threshold, inf and NaN passed through)
@@ -343,11 +345,12 @@ class Gen:
             self.e("fma.rn.f32x2 %%P, %%P, %%R, %%K0;")
         self.unpack(i, "%%n0", "%%n1", "%%JM")
         if not wide:
+            # times 2^j: the low bits of the rounded sum are j, added to the
+            # exponent (the product is normal for |x| < 87)
+            self.e("mov.b64 {%%m0, %%m1}, %%P;")
             for r in (0, 1):
-                # 2^j: the low bits of the rounded sum are j, shifted into the exponent
-                self.e(f"mad.lo.u32 %%n{r}, %%n{r}, 8388608, 0x3F800000;")
-            self.e("mov.b64 %%S, {%%n0, %%n1};")
-            self.e(f"mul.rn.f32x2 {t}, %%P, %%S;")
+                self.e(f"mad.lo.u32 %%m{r}, %%n{r}, 8388608, %%m{r};")
+            self.e(f"mov.b64 {t}, {{%%m0, %%m1}};")
             return
         for r in (0, 1):
             # j = the sum's bits - the magic's; 2^(j >> 1) into n, the rest into m
@@ -377,15 +380,16 @@ class Gen:
     # root and 1.2e9 quotients.  Outside those ranges the word is handed
     # back, and the switch uses the IEEE operations themselves.
     def rcp_pair(self, src, dst):
-        """dst = 1 / src for one pair, its rows in the reciprocal's range"""
+        """dst = 1 / src for one pair, its rows in the reciprocal's range;
+        leaves -src in F"""
         self.e(f"mov.b64 {{%%v0, %%v1}}, {src};")
         self.e("rcp.approx.ftz.f32 %%u0, %%v0;")
         self.e("rcp.approx.ftz.f32 %%u1, %%v1;")
         self.e("mov.b64 %%P, {%%u0, %%u1};")
         self.e(f"mov.b64 %%K0, {kp('mone')};")
-        self.e("mul.rn.f32x2 %%Q, %%P, %%K0;")           # -e
+        self.e(f"mul.rn.f32x2 %%F, {src}, %%K0;")         # -b
         self.e(f"mov.b64 %%K1, {kp('one')};")
-        self.e(f"fma.rn.f32x2 %%Q, {src}, %%Q, %%K1;")    # 1 - b e
+        self.e("fma.rn.f32x2 %%Q, %%F, %%P, %%K1;")       # 1 - b e
         self.e(f"fma.rn.f32x2 {dst}, %%P, %%Q, %%P;")     # e + e (1 - b e)
 
     def inv(self):
@@ -507,9 +511,7 @@ class Gen:
             # y = 1 / b, q = a y, then q + (a - b q) y
             self.rcp_pair(den(i), "%%JJ")
             self.e(f"mul.rn.f32x2 %%JM, {num(i)}, %%JJ;")
-            self.e(f"mov.b64 %%K0, {kp('mone')};")
-            self.e(f"mul.rn.f32x2 %%R, {den(i)}, %%K0;")     # -b
-            self.e(f"fma.rn.f32x2 %%R, %%R, %%JM, {num(i)};")  # a - b q
+            self.e(f"fma.rn.f32x2 %%R, %%F, %%JM, {num(i)};")  # a - b q
             self.e("fma.rn.f32x2 %%JM, %%R, %%JJ, %%JM;")
             self.e(f"mov.b64 {{%%s0, %%s1}}, {den(i)};")
             self.e("mov.b64 {%%c0, %%c1}, %%JM;")

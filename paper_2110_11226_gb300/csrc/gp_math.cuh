@@ -69,6 +69,7 @@ constexpr float kC0 = 0.0416666679f, kC1 = -0.00138888834f, kC2 = 2.47994594e-05
 // 1.5 * 2^23 rounds to an integer in the FMA pipe, and for |j| < 2^22 the
 // two's-complement low bits of that sum's encoding are j's low bits.
 constexpr float kRoundMagic = 12582912.0f;  // 1.5 * 2^23
+constexpr float kRoundMagic1 = 12582913.0f;
 
 // The evaluator's fast loop (inline PTX) spells these constants as float
 // bit patterns; the checks keep the two spellings the same numbers.
@@ -93,6 +94,7 @@ static_assert(__builtin_bit_cast(uint32_t, kC1) == 0xBAB60B5Cu, "trig constant")
 static_assert(__builtin_bit_cast(uint32_t, kC2) == 0x37D0086Fu, "trig constant");
 static_assert(__builtin_bit_cast(uint32_t, kC3) == 0xB4920F4Eu, "trig constant");
 static_assert(__builtin_bit_cast(uint32_t, kRoundMagic) == 0x4B400000u, "trig constant");
+static_assert(__builtin_bit_cast(uint32_t, kRoundMagic1) == 0x4B400001u, "trig constant");
 static_assert(__builtin_bit_cast(uint32_t, kTrigFast) == 0x47800000u, "trig constant");
 // log: the bit pattern of sqrt(1/2) splits x into 2^k m; log(1 + f) ~
 // f + f^2 (P0 + f (P1 + ... + f P7)); ln2 = LN2_HI (16 significant bits,
@@ -192,10 +194,11 @@ __device__ __forceinline__ float exp_wide(float x) {
 // x/pi - kind/2, r = x - (j + kind/2) pi in [-pi/2, pi/2] (plus rounding
 // slack), and the result is sin r, negated when j + kind is odd
 __device__ __forceinline__ float sincos_fast(float x, int kind) {
-    const float half = kind ? 0.5f : 0.0f;
-    const float t1 = __fmaf_rn(x, kInvPi, -half);
-    const float jm = __fadd_rn(t1, kRoundMagic);
-    const float jh = __fadd_rn(__fsub_rn(jm, kRoundMagic), half);
+    // cos rounds with 1.5 * 2^23 + 1, so that in both the sum's low bit is
+    // the parity of j + kind
+    const float jm = kind ? __fadd_rn(__fmaf_rn(x, kInvPi, -0.5f), kRoundMagic1)
+                          : __fmaf_rn(x, kInvPi, kRoundMagic);
+    const float jh = kind ? __fadd_rn(__fsub_rn(jm, kRoundMagic1), 0.5f) : __fsub_rn(jm, kRoundMagic);
     float r = __fmaf_rn(jh, -kPiHi, x);
     r = __fmaf_rn(jh, -kPiMid, r);
     r = __fmaf_rn(jh, -kPiLo, r);
@@ -204,7 +207,7 @@ __device__ __forceinline__ float sincos_fast(float x, int kind) {
     p = __fmaf_rn(p, s, kQ1);
     p = __fmaf_rn(p, s, kQ0);
     const float v = __fmaf_rn(p, __fmul_rn(s, r), r);
-    return ((__float_as_int(jm) + kind) & 1) ? -v : v;
+    return (__float_as_int(jm) & 1) ? -v : v;
 }
 
 // tan's reduction: r = x - j pi/2, q = j mod 4
