@@ -358,7 +358,7 @@ int run_predict_compiled(const Workspace &W, int p0, int b, const float *X, int6
     const int64_t chunk = std::min<int64_t>(round_up(n_rows, 256), 4096);
     const int n_chunks = (int)((n_rows + chunk - 1) / chunk);
     GP_CUDA(launch_order(W.meta + p0, b, W.order, W.class_count, st, W.counters));
-    const bool vec = aligned16(X) && (n_rows % 4 == 0);
+    const bool vec = aligned16(X) && aligned16(out_pred) && (n_rows % 4 == 0);
     const int fmode = (n_feat <= 2) ? 2 : 0;
     for (int cls = 0; cls < kNumClasses; ++cls) {
         EvalArgs ea{};

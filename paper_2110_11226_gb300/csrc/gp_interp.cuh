@@ -13,8 +13,10 @@
 // rows (sub-tile w, w + warps, ...).  Within a warp the instruction stream
 // is uniform, so the dispatch switch never diverges; across the block the
 // warps walk the same few switch cases, which keeps the SM's instruction
-// working set small.  Lane l owns rows base + l*RPT .. +RPT-1 (vectorised,
-// coalesced loads from the column-major X).  The top of the stack is the
+// working set small.  In a whole sub-tile of 16-byte aligned columns lane l
+// owns rows base + l*RPT .. +RPT-1 (16-byte loads); in a ragged one, or when
+// the column length leaves columns unaligned, rows base + l + 32 j (coalesced
+// 4-byte loads).  The top of the stack is the
 // register array t[RPT]; deeper values sit in the warp's slice of a
 // shared-memory stack, one float4 per (slot, group of 4 rows, lane), so a
 // push or pop is one or two conflict-free 16-byte accesses per lane.  Each
@@ -32,6 +34,13 @@
 // order, writing one partial per (program, chunk).  A separate pass adds the
 // partials of a program in chunk order in FP64.  Every step has a fixed
 // order, so results do not depend on which block ran which item.
+//
+// What surrounds the words -- loads, loss, loop -- costs 139 instructions per
+// program and sub-tile at 8 rows per lane, of some 900 (220 before the rows
+// were kept as pairs throughout, the ragged case put behind one test and the
+// next item taken by one thread: Pagie-1 16M x 4096 301 -> 281 ms; with 28
+// unaligned columns, where a lane's consecutive rows took eight 4-byte loads
+// of 32 sectors each, 22.2 -> 17.9 ms).
 #pragma once
 
 #include "gp_internal.cuh"
@@ -89,6 +98,16 @@ __device__ __forceinline__ float row_loss(int metric, float p, float y) {
     return __fmul_rn(d, d);
 }
 
+// two rows in one 64-bit register pair
+__device__ __forceinline__ uint64_t pack2(float a, float b) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void unpack2(uint64_t r, float &a, float &b) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(r));
+}
+
 // RPT consecutive rows starting at r0 of one column; rows >= re read 0.
 template <int RPT>
 __device__ __forceinline__ void load_rows(float (&v)[RPT], const float *__restrict__ col,
@@ -128,13 +147,40 @@ __device__ __forceinline__ void load_chunk_rows(float (&v)[RPT], const float *__
     }
 }
 
+// The evaluator's rows of a lane as pairs.  packed: RPT consecutive rows
+// from p, 16-byte loads; else rows p[0], p[32], p[64], ..., the last of them
+// at most p[last] (a ragged sub-tile reads its last row again; those rows
+// do not count).
+template <int RPT>
+__device__ __forceinline__ void load_pairs(uint64_t (&v)[RPT / 2], const float *__restrict__ p,
+                                           bool packed, int last) {
+    if (packed) {
+#pragma unroll
+        for (int q = 0; q < RPT / 4; ++q) {
+            const ulonglong2 f = __ldg(reinterpret_cast<const ulonglong2 *>(p) + q);
+            v[2 * q] = f.x;
+            v[2 * q + 1] = f.y;
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < RPT / 2; ++i)
+            v[i] = pack2(__ldg(p + min(64 * i, last)), __ldg(p + min(64 * i + 32, last)));
+    }
+}
+
 // the weighted losses of a lane's rows added in row order (the first nv
 // rows count); the metric and the weights are tested once, not per row
 template <int RPT>
-__device__ __forceinline__ float loss_sum(int metric, const float (&t)[RPT],
-                                          const float (&yv)[RPT], const float (&wv)[RPT],
-                                          bool has_w, bool full, int nv) {
-    float l[RPT];
+__device__ __forceinline__ float loss_sum(int metric, const uint64_t (&tp)[RPT / 2],
+                                          const uint64_t (&yp)[RPT / 2],
+                                          const uint64_t (&wp)[RPT / 2], bool has_w, bool full,
+                                          int nv) {
+    float l[RPT], t[RPT], yv[RPT];
+#pragma unroll
+    for (int i = 0; i < RPT / 2; ++i) {
+        unpack2(tp[i], t[2 * i], t[2 * i + 1]);
+        unpack2(yp[i], yv[2 * i], yv[2 * i + 1]);
+    }
     if (metric == GP_MAE) {
 #pragma unroll
         for (int j = 0; j < RPT; ++j) l[j] = row_loss(GP_MAE, t[j], yv[j]);
@@ -146,6 +192,9 @@ __device__ __forceinline__ float loss_sum(int metric, const float (&t)[RPT],
         for (int j = 0; j < RPT; ++j) l[j] = row_loss(GP_MSE, t[j], yv[j]);
     }
     if (has_w) {
+        float wv[RPT];
+#pragma unroll
+        for (int i = 0; i < RPT / 2; ++i) unpack2(wp[i], wv[2 * i], wv[2 * i + 1]);
 #pragma unroll
         for (int j = 0; j < RPT; ++j) l[j] = __fmul_rn(wv[j], l[j]);
     }
@@ -203,15 +252,6 @@ static __device__ __noinline__ float4 ext_rows4(float4 v, uint32_t f) {
 // is off in the instances with the extended functions: there the division
 // set in the loop cost the extended-set population 23% (their out-of-line
 // calls and the division's own slow-path call do not mix well).
-__device__ __forceinline__ uint64_t pack2(float a, float b) {
-    uint64_t r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ void unpack2(uint64_t r, float &a, float &b) {
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(r));
-}
-
 template <int RPT, int NSLOT, bool DIVS, bool XREG>
 __device__ __forceinline__ void run_fast(uint32_t &pa, uint64_t (&t)[RPT / 2],
                                          const uint64_t (&x0)[RPT / 2],
@@ -231,13 +271,12 @@ __device__ __forceinline__ void run_fast(uint32_t &pa, uint64_t (&t)[RPT / 2],
 }
 
 // Runs one compiled program over RPT rows per lane; returns the top of the
-// stack in t.  stk = this warp's stack slice, already offset by the lane.
-// The instruction buffer (kCodeStride + 2 entries in shared memory, one
-// more than either loop can reach) holds OP_END from the program's end
-// through its last entry, so the loop ends within kCodeStride + 1 steps
-// whatever the buffer holds; op values that name no operation act as
-// OP_END and stack slots are clamped to the stack, so no instruction word
-// can make it run away or leave its memory.
+// stack in tp, rows as pairs.  stk = this warp's stack slice, already offset
+// by the lane; xc, packed and last: the chunk's column 0 at the lane's first
+// row, and how the lane's rows follow it (load_pairs).
+// The instruction buffer holds the words that the pre-pass wrote, the last
+// of them OP_END; op values that name no operation act as OP_END and stack
+// slots are clamped to the stack.
 //
 // Dispatch cost is what this loop is tuned for (per-opcode instruction
 // counts measured with ncu on chains of one operation).  At 4 and 8 rows
@@ -250,44 +289,31 @@ __device__ __forceinline__ void run_fast(uint32_t &pa, uint64_t (&t)[RPT / 2],
 // and the word is loaded when it is needed rather than one ahead, which
 // saves the register copies of a prefetch.
 template <int RPT, int NSLOT, int FMODE, bool EXT>
-__device__ __forceinline__ void interpret(float (&t)[RPT], const uint2 *__restrict__ cbuf,
-                                          const float (&x0)[RPT], const float (&x1)[RPT],
-                                          const float *__restrict__ X, int64_t ld, int64_t r0,
-                                          int64_t re, bool vec, float4 *stk) {
+__device__ __forceinline__ void interpret(uint64_t (&tp)[RPT / 2], const uint2 *__restrict__ cbuf,
+                                          const uint64_t (&x0p)[RPT / 2],
+                                          const uint64_t (&x1p)[RPT / 2],
+                                          const float *__restrict__ xc, int64_t ld, bool packed,
+                                          int last, float4 *stk) {
     // EXT: the extended functions are compiled in (classes 1 and 2).  In
     // class 0, where nearly all programs of the usual function set run,
     // their cases cost 2-3% (measured on Pagie-1 x 4096 programs, which
     // never use them)
     constexpr bool kExt = EXT;
+    // the first word is a push: the rows need no value before it
 #pragma unroll
-    for (int j = 0; j < RPT; ++j) t[j] = 0.0f;
+    for (int i = 0; i < RPT / 2; ++i) asm volatile("" : "=l"(tp[i]));
     // pa: shared-memory address of the next instruction word
     uint32_t pa = (uint32_t)__cvta_generic_to_shared(cbuf);
     const uint32_t sb = (uint32_t)__cvta_generic_to_shared(stk);  // this lane's slot 0
     // 4 or 8 rows per lane: the fast loop runs what it can and hands back
-    // the rest, one word at a time, to the switch below; the rows cross
-    // between the two as pairs {row 2i, row 2i+1} (register moves)
+    // the rest, one word at a time, to the switch below
     constexpr bool kFast = RPT == 4 || RPT == 8;
-    constexpr int kPairs = kFast ? RPT / 2 : 1;
-    uint64_t x0p[kPairs], x1p[kPairs];
-    if constexpr (kFast) {
-#pragma unroll
-        for (int i = 0; i < kPairs; ++i) {
-            x0p[i] = pack2(x0[2 * i], x0[2 * i + 1]);
-            x1p[i] = pack2(x1[2 * i], x1[2 * i + 1]);
-        }
-    }
 #pragma unroll 1
     for (;;) {
         uint2 ins;
         if constexpr (kFast) {
             float hc;
-            uint64_t tp[kPairs];
-#pragma unroll
-            for (int i = 0; i < kPairs; ++i) tp[i] = pack2(t[2 * i], t[2 * i + 1]);
             run_fast<RPT, NSLOT, !EXT, FMODE == 2>(pa, tp, x0p, x1p, sb, ins.x, hc);
-#pragma unroll
-            for (int i = 0; i < kPairs; ++i) unpack2(tp[i], t[2 * i], t[2 * i + 1]);
             ins.y = __float_as_uint(hc);
         } else {
             asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];"
@@ -298,6 +324,9 @@ __device__ __forceinline__ void interpret(float (&t)[RPT], const uint2 *__restri
         const uint32_t w = __shfl_sync(0xffffffffu, ins.x, 0);
         // the end of the program, once per sub-tile: out before the switch
         if ((w & 31u) == OP_END) break;
+        float t[RPT];
+#pragma unroll
+        for (int i = 0; i < RPT / 2; ++i) unpack2(tp[i], t[2 * i], t[2 * i + 1]);
         const float c = __uint_as_float(ins.y);
 // operand helpers: stack slot, X column, constant
 // (the stack is laid out [slot][q][lane] in float4: slot sl, group q of
@@ -325,11 +354,14 @@ __device__ __forceinline__ void interpret(float (&t)[RPT], const uint2 *__restri
 #define GP_X_LOAD(u)                                                            \
     {                                                                           \
         const int feat = (int)(w >> 16);                                        \
+        uint64_t up[RPT / 2];                                                   \
         if (FMODE == 2) {                                                       \
-            _Pragma("unroll") for (int j = 0; j < RPT; ++j) u[j] = feat ? x1[j] : x0[j]; \
+            _Pragma("unroll") for (int i = 0; i < RPT / 2; ++i) up[i] = feat ? x1p[i] : x0p[i]; \
         } else {                                                                \
-            load_rows<RPT>(u, X + (int64_t)feat * ld, r0, re, vec);             \
+            load_pairs<RPT>(up, xc + (int64_t)feat * ld, packed, last);         \
         }                                                                       \
+        _Pragma("unroll") for (int i = 0; i < RPT / 2; ++i)                     \
+            unpack2(up[i], u[2 * i], u[2 * i + 1]);                             \
     }
 #define GP_T(expr) _Pragma("unroll") for (int j = 0; j < RPT; ++j) t[j] = expr;
 #define GP_U_C(u) _Pragma("unroll") for (int j = 0; j < RPT; ++j) u[j] = c;
@@ -390,13 +422,16 @@ __device__ __forceinline__ void interpret(float (&t)[RPT], const uint2 *__restri
             default:  // every value of w & 31 has a case above
                 __builtin_unreachable();
         }
-        continue;
+        goto next;
         // division has one body per operand order, shared by its operand cases
     div_tu:
         GP_T(f_div(t[j], u[j]))
-        continue;
+        goto next;
     div_ut:
         GP_T(f_div(u[j], t[j]))
+    next:
+#pragma unroll
+        for (int i = 0; i < RPT / 2; ++i) tp[i] = pack2(t[2 * i], t[2 * i + 1]);
 #undef GP_T
 #undef GP_U_C
 #undef GP_X_LOAD
@@ -437,112 +472,120 @@ __global__ void __launch_bounds__(eval_warps<RPT>() * 32,
     float4 *stack_all = smem_eval + ((kCodeStride + 2) * sizeof(uint2) + 15) / 16;
     __shared__ float wsum[kEvalWarps];
     __shared__ double wmom[MOM ? kEvalWarps : 1][3];
-    __shared__ unsigned long long s_item;
+    __shared__ int4 s_item[2];  // chunk (-1: the queue is empty), program, words, status
+    __shared__ unsigned long long s_total;
+    __shared__ int s_begin, s_n;
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     float4 *stk = stack_all + (size_t)warp * NSLOT * (RPT / 4) * 32 + lane;
-    const int qc = a.qcls ? a.qcls - 1 : a.cls;  // the span of the program order
-    int cls_begin = 0;
-    for (int b = 0; b < qc; ++b) cls_begin += a.class_count[b];
-    int n_cls = a.class_count[qc];
-    if (a.sub == 1) {  // the long programs of class 0 (first in its order)
-        n_cls = a.class_count[kOrderClasses];
-    } else if (a.sub == 2) {  // the rest of class 0
-        cls_begin = a.class_count[kOrderClasses];
-        n_cls -= cls_begin;
-    }
-    const unsigned long long total = (unsigned long long)n_cls * (unsigned long long)a.n_chunks;
-    const bool vec = a.vec_ok != 0;
-    const bool two_feat = FMODE == 2 && a.ld > 0;
     const float ybar = MOM ? (float)a.ystat[3] : 0.0f;
 
-    for (unsigned long long it = 0; it <= total; ++it) {
-        if (threadIdx.x == 0) s_item = atomicAdd(a.counter, 1ULL);
-        __syncthreads();
-        const unsigned long long item = s_item;
-        if (item >= total || it == total) {  // the cap cannot trigger: one item per pass
-            if (it == total && threadIdx.x == 0) atomicOr(a.dev_status, GP_DEV_QUEUE_CAP);
-            break;
+    // Thread 0 takes the next item while the block works on this one: it
+    // alone waits for the counter and splits the number into (chunk, rank).
+    // What it needs for that, and the item itself, sit in shared memory: in
+    // registers they would stay live across the interpreter
+    auto take = [&](unsigned long long item, int slot) {
+        int4 it = make_int4(-1, 0, 0, 0);
+        if (item < s_total) {
+            const uint32_t n = (uint32_t)s_n;
+            it.x = (int)((s_total >> 32) ? item / n : (uint32_t)item / n);
+            it.y = a.order[s_begin + (int)(item - (unsigned long long)it.x * n)];
+            const ProgMeta m = a.meta[it.y];
+            it.z = m.n_ins;
+            it.w = m.status;
         }
-        const int chunk = (int)(item / (unsigned long long)n_cls);
-        const int rank = (int)(item - (unsigned long long)chunk * n_cls);
-        const int p = a.order[cls_begin + rank];
-        const ProgMeta m = a.meta[p];
-        const int64_t rb = (int64_t)chunk * a.chunk_rows;
-        const int64_t re = min(a.n_rows, rb + a.chunk_rows);
+        s_item[slot] = it;
+    };
+    if (threadIdx.x == 0) {
+        const int qc = a.qcls ? a.qcls - 1 : a.cls;  // the span of the program order
+        int begin = 0, n = a.class_count[qc];
+        for (int b = 0; b < qc; ++b) begin += a.class_count[b];
+        if (a.sub == 1) {  // the long programs of class 0 (first in its order)
+            n = a.class_count[kOrderClasses];
+        } else if (a.sub == 2) {  // the rest of class 0
+            begin = a.class_count[kOrderClasses];
+            n -= begin;
+        }
+        s_begin = begin;
+        s_n = n;
+        s_total = (unsigned long long)n * (unsigned long long)a.n_chunks;
+        take(blockIdx.x, 0);  // the counter hands out the items from gridDim.x on
+    }
+    __syncthreads();
 
-        if (m.status != GP_PROG_OK) {
-            if (PRED) {
-                for (int64_t r = rb + threadIdx.x; r < re; r += kEvalBlock)
-                    a.pred[(size_t)p * a.n_rows + r] = __int_as_float(0x7fc00000);
-            } else if (MOM) {
-                if (threadIdx.x < 3)
-                    a.mom[((size_t)p * a.n_chunks + chunk) * 3 + threadIdx.x] =
-                        __longlong_as_double(0x7ff8000000000000LL);
-            } else if (threadIdx.x == 0) {
-                a.part[(size_t)p * a.n_chunks + chunk] = __int_as_float(0x7fc00000);
-            }
-            __syncthreads();  // s_item is rewritten at the top
-            continue;
+    // one item per pass: every number comes up once, so a block makes at most
+    // s_total passes
+    for (int cur = 0;; cur ^= 1) {
+        const int4 it = s_item[cur];
+        const int chunk = it.x, p = it.y;
+        if (chunk < 0) break;
+        const int64_t rb = (int64_t)chunk * a.chunk_rows;
+        const int n_in = (int)(min(a.n_rows, rb + a.chunk_rows) - rb);
+        const bool ok = it.w == GP_PROG_OK;
+        // the program's words (OP_END the last of them)
+        if (ok) {
+            const uint2 *src = a.code + (size_t)p * (a.code_stride ? a.code_stride : kCodeStride);
+            for (int i = threadIdx.x; i < it.z && i <= kCodeStride; i += kEvalBlock) cbuf[i] = src[i];
         }
-        // the program, then OP_END through the buffer's last entry (the last
-        // one stored apart: as a third pass of the loop it cost the kernel
-        // 15 registers)
-        const uint2 *src = a.code + (size_t)p * (a.code_stride ? a.code_stride : kCodeStride);
-        for (int i = threadIdx.x; i <= kCodeStride; i += kEvalBlock)
-            cbuf[i] = (i < m.n_ins) ? src[i] : make_uint2(make_ins(OP_END, 0, 0), 0u);
-        if (threadIdx.x == 0) cbuf[kCodeStride + 1] = make_uint2(make_ins(OP_END, 0, 0), 0u);
-        __syncthreads();
+        __syncthreads();  // the words are there
+        unsigned long long next = 0;
+        if (threadIdx.x == 0) next = gridDim.x + atomicAdd(a.counter, 1ULL);
 
         float ks = 0.0f, kc = 0.0f;
         float ms[3] = {0.0f, 0.0f, 0.0f}, mc[3] = {0.0f, 0.0f, 0.0f};
         const float shift = MOM ? a.shift[p] : 0.0f;
-        // rows of the chunk in 32-bit offsets from its first row (a chunk
-        // holds at most 2^30 rows); pointers to the chunk's columns once
-        const int n_in = (int)(re - rb);
-        // the column pointers are formed per use from the kernel arguments
-        // (held in constant memory): four live 64-bit pointers would cost
-        // the loop 8 registers and a resident block
-        const int64_t x1off = two_feat ? a.ld : 0;
-        for (int base = warp * 32 * RPT; base < n_in; base += kEvalWarps * 32 * RPT) {
-            const int o = base + lane * RPT;  // this lane's first row in the chunk
-            // every row of the warp is in the chunk except in its last
-            // sub-tile; decided once for the warp (a vote), so the loads and
-            // the loss take no divergent branch (each per-lane test had cost
-            // a reconvergence barrier pair per sub-tile)
-            const bool full = __all_sync(0xffffffffu, o + RPT <= n_in);
-            const int nv = full ? RPT : n_in - o;  // rows of the lane to count
-            float x0[RPT], x1[RPT];
+        for (int base = warp * 32 * RPT; base < n_in && ok; base += kEvalWarps * 32 * RPT) {
+            // whole: every row of the sub-tile is in the chunk; packed: and
+            // the lane's rows are consecutive.  One test for the warp
+            const bool whole = base + 32 * RPT <= n_in;
+            const bool packed = whole && a.vec_ok;
+            const int o = base + (packed ? lane * RPT : lane);  // the lane's first row
+            const int last = n_in - 1 - o;   // its furthest row (negative: none; see load_pairs)
+            const int nv = whole ? RPT : (last + 32) >> 5;  // rows of the lane that count
+            const int64_t r = rb + o;
+            uint64_t x0[RPT / 2], x1[RPT / 2];
             if (FMODE == 2) {
-                load_chunk_rows<RPT>(x0, a.X + (rb + o), full && vec, nv);
-                if (two_feat) load_chunk_rows<RPT>(x1, a.X + (x1off + rb + o), full && vec, nv);
-                else {
-#pragma unroll
-                    for (int j = 0; j < RPT; ++j) x1[j] = x0[j];
-                }
+                load_pairs<RPT>(x0, a.X + r, packed, last);
+                load_pairs<RPT>(x1, a.X + (a.ld + r), packed, last);
             } else {
 #pragma unroll
-                for (int j = 0; j < RPT; ++j) x0[j] = x1[j] = 0.0f;
+                for (int i = 0; i < RPT / 2; ++i) x0[i] = x1[i] = 0;
             }
-            float t[RPT];
-            interpret<RPT, NSLOT, FMODE, EXT>(t, cbuf, x0, x1, a.X, a.ld, rb + o, re, vec, stk);
+            uint64_t t[RPT / 2];
+            interpret<RPT, NSLOT, FMODE, EXT>(t, cbuf, x0, x1, a.X + r, a.ld, packed, last, stk);
             if (PRED) {
-                float *dst = a.pred + (size_t)p * a.n_rows + rb + o;
+                float *dst = a.pred + (size_t)p * a.n_rows + r;
+                if (packed) {
 #pragma unroll
-                for (int j = 0; j < RPT; ++j)
-                    if (j < nv) dst[j] = t[j];
-            } else if (MOM) {
+                    for (int q = 0; q < RPT / 4; ++q)
+                        reinterpret_cast<ulonglong2 *>(dst)[q] = make_ulonglong2(t[2 * q], t[2 * q + 1]);
+                } else {
+#pragma unroll
+                    for (int i = 0; i < RPT / 2; ++i) {
+                        float lo, hi;
+                        unpack2(t[i], lo, hi);
+                        if (2 * i < nv) dst[64 * i] = lo;
+                        if (2 * i + 1 < nv) dst[64 * i + 32] = hi;
+                    }
+                }
+                continue;
+            }
+            uint64_t yv[RPT / 2], wv[RPT / 2];
+            load_pairs<RPT>(yv, a.y + r, packed, last);
+            if (a.w) load_pairs<RPT>(wv, a.w + r, packed, last);
+            if (MOM) {
                 // d = p - shift keeps the sums of squares free of the
                 // cancellation a large mean would cause
-                float yv[RPT], wv[RPT];
-                load_chunk_rows<RPT>(yv, a.y + (rb + o), full && vec, nv);
-                if (a.w) load_chunk_rows<RPT>(wv, a.w + (rb + o), full && vec, nv);
                 float e1 = 0.0f, e2 = 0.0f, e3 = 0.0f;
 #pragma unroll
                 for (int j = 0; j < RPT; ++j) {
-                    const float d = __fsub_rn(t[j], shift);
-                    const float yc_ = __fsub_rn(yv[j], ybar);
-                    const float wd = a.w ? __fmul_rn(wv[j], d) : d;
+                    float tv[2], yy[2], ww[2] = {1.0f, 1.0f};
+                    unpack2(t[j / 2], tv[0], tv[1]);
+                    unpack2(yv[j / 2], yy[0], yy[1]);
+                    if (a.w) unpack2(wv[j / 2], ww[0], ww[1]);
+                    const float d = __fsub_rn(tv[j & 1], shift);
+                    const float yc_ = __fsub_rn(yy[j & 1], ybar);
+                    const float wd = a.w ? __fmul_rn(ww[j & 1], d) : d;
                     const bool in = j < nv;
                     e1 = in ? __fadd_rn(e1, wd) : e1;
                     e2 = in ? __fadd_rn(e2, __fmul_rn(wd, d)) : e2;
@@ -552,12 +595,10 @@ __global__ void __launch_bounds__(eval_warps<RPT>() * 32,
                 kahan_add(ms[1], mc[1], e2);
                 kahan_add(ms[2], mc[2], e3);
             } else {
-                float yv[RPT], wv[RPT];
-                load_chunk_rows<RPT>(yv, a.y + (rb + o), full && vec, nv);
-                if (a.w) load_chunk_rows<RPT>(wv, a.w + (rb + o), full && vec, nv);
-                kahan_add(ks, kc, loss_sum<RPT>(a.metric, t, yv, wv, a.w != nullptr, full, nv));
+                kahan_add(ks, kc, loss_sum<RPT>(a.metric, t, yv, wv, a.w != nullptr, whole, nv));
             }
         }
+        if (threadIdx.x == 0) take(next, cur ^ 1);
         if (MOM) {
             // the lane's compensated sums in FP64, then a fixed butterfly
 #pragma unroll
@@ -573,15 +614,20 @@ __global__ void __launch_bounds__(eval_warps<RPT>() * 32,
             for (int o = 16; o > 0; o >>= 1) v = __fadd_rn(v, __shfl_xor_sync(0xffffffffu, v, o));
             if (lane == 0) wsum[warp] = v;
         }
-        __syncthreads();  // wsum complete; everyone is done with cbuf and s_item
-        if (MOM && threadIdx.x < 3) {
+        __syncthreads();  // wsum and the next item complete; everyone is done with cbuf
+        if (PRED) {
+            if (!ok)
+                for (int i = threadIdx.x; i < n_in; i += kEvalBlock)
+                    a.pred[(size_t)p * a.n_rows + rb + i] = __int_as_float(0x7fc00000);
+        } else if (MOM && threadIdx.x < 3) {
             double v = 0.0;
             for (int w = 0; w < kEvalWarps; ++w) v += wmom[w][threadIdx.x];
-            a.mom[((size_t)p * a.n_chunks + chunk) * 3 + threadIdx.x] = v;
-        } else if (!PRED && !MOM && threadIdx.x == 0) {
+            a.mom[((size_t)p * a.n_chunks + chunk) * 3 + threadIdx.x] =
+                ok ? v : __longlong_as_double(0x7ff8000000000000LL);
+        } else if (!MOM && threadIdx.x == 0) {
             float v = 0.0f;
             for (int w = 0; w < kEvalWarps; ++w) v = __fadd_rn(v, wsum[w]);
-            a.part[(size_t)p * a.n_chunks + chunk] = v;
+            a.part[(size_t)p * a.n_chunks + chunk] = ok ? v : __int_as_float(0x7fc00000);
         }
     }
 }
