@@ -25,8 +25,9 @@ and tan goes to the C++ switch.
 
 Variants: RPT in {4, 8} x DIVS (the division set, square root, reciprocal,
 sin, cos, log and exp run here; without DIVS they are handed back) x
-XREG (columns 0 and 1 held in registers; without it every column read is
-handed back).  A word the loop does not run -- END, the extended
+XREG (columns 0 and 1 held in registers; without it a column read takes
+the rows that were prefetched for it and prefetches the next one's; without
+DIVS and in the gradient variant it is handed back).  A word the loop does not run -- END, the extended
 functions, the trigonometric and exponential arguments outside their fast
 paths, and whatever DIVS or XREG leave out -- is handed back to the
 caller's switch with its constant, the address just past it, and the rows
@@ -75,14 +76,29 @@ def kp(name, neg=False):
 class Gen:
     def __init__(self, rpt, divs, xreg, grad=False):
         self.rpt, self.divs, self.xreg, self.grad = rpt, divs, xreg, grad
+        # columns in memory: the next column read is prefetched into XB
+        self.xmem = not xreg and divs and not grad
         self.np = rpt // 2               # pairs per lane
         p = self.np
-        self.T = [f"%{1 + i}" for i in range(p)]
-        self.HW, self.HC, self.SB, self.NSM1 = f"%{p + 1}", f"%{p + 2}", f"%{p + 3}", f"%{p + 4}"
-        self.X = [[f"%{p + 5 + i}" for i in range(p)], [f"%{2 * p + 5 + i}" for i in range(p)]]
-        self.THR = f"%{3 * p + 5}"
+        names = ["pa"] + [f"T{i}" for i in range(p)]
+        if self.xmem:
+            names += [f"XB{i}" for i in range(p)]
+        names += ["HW", "HC", "SB", "NSM1"]
+        if self.xmem:
+            names += ["XC", "UNIT", "MODE"]
+        else:
+            names += [f"X{c}_{i}" for c in (0, 1) for i in range(p)]
         # gradient variant: the lane's tangent slot 0 and the tangent slots
-        self.DB, self.KT = f"%{3 * p + 6}", f"%{3 * p + 7}"
+        names += ["THR", "DB", "KT"]
+        at = {n: f"%{k}" for k, n in enumerate(names)}
+        self.T = [at[f"T{i}"] for i in range(p)]
+        self.HW, self.HC, self.SB, self.NSM1 = at["HW"], at["HC"], at["SB"], at["NSM1"]
+        self.THR, self.DB, self.KT = at["THR"], at["DB"], at["KT"]
+        if self.xmem:
+            xb = [at[f"XB{i}"] for i in range(p)]
+            self.X, self.XC, self.UNIT, self.MODE = [xb, xb], at["XC"], at["UNIT"], at["MODE"]
+        else:
+            self.X = [[at[f"X{c}_{i}"] for i in range(p)] for c in (0, 1)]
         self.slot_bytes = (rpt // 4) * 512
         self.lines = []
         # the special-value paths (4 rows per lane only: at 8 the loop's
@@ -750,6 +766,60 @@ class Gen:
         e("mov.u32 %%ret, 0;")
         e("bra.uni N%=;")
 
+    # Columns in memory (xmem).  A word that reads a column finds the rows in
+    # XB, uses them and at once issues the loads of the column that the
+    # program reads next (the word's constant; the last such word reads its
+    # own again), so that their latency passes behind the words between.
+    # MODE 0: the lane's rows are consecutive, 16-byte loads; 1: 128 bytes
+    # apart, 4-byte loads, in one block that all these words share; 2 (a
+    # ragged sub-tile): every column read is handed back.  A chain of
+    # additions of columns takes 68 issue cycles a word (98 when handed back to
+    # the C++ switch, which waits for the loads): the L2 delivers 1 KB to an SM
+    # in no less.  One body per word and one shared block, because two copies
+    # of each (the last word without loads, the strided loads in place) cost
+    # more in instruction fetches than they saved (4M x 50: 22.1 against
+    # 24.1 ms)
+    def next_column(self):
+        e = self.e
+        e(f"mad.wide.u32 %%xa, %%cb, {self.UNIT}, {self.XC};")
+        e("@%%pm bra NS%=;")
+        xb = self.X[0]
+        for q in range(self.rpt // 4):
+            off = f"+{16 * q}" if q else ""
+            e(f"ld.global.nc.v2.b64 {{{xb[2 * q]}, {xb[2 * q + 1]}}}, [%%xa{off}];")
+
+    def strided_columns(self):
+        e, xb = self.e, self.X[0]
+        self.label("NS")
+        for i in range(self.np):
+            e(f"ld.global.nc.f32 %%v0, [%%xa+{256 * i}];")
+            e(f"ld.global.nc.f32 %%v1, [%%xa+{256 * i + 128}];")
+            e(f"mov.b64 {xb[i]}, {{%%v0, %%v1}};")
+        e("brx.idx.uni %%dv, TD%=;")
+
+    def xmem_body(self, stem):
+        """the body of a column-reading word: its operation on XB, then the
+        next loads, then (dv) the next word or a division with its operand in
+        U (which, handed back, reads the column again)"""
+        to = dict(DX=1, RDX=2).get(stem, 0)
+        self.e("@%%pb bra EX%=;")
+        if stem == "PXS":
+            self.spill()
+        if stem in ("PX", "PXS"):
+            for i in range(self.np):
+                self.e(f"mov.b64 {self.T[i]}, {self.X[0][i]};")
+        elif stem in ("AX", "SX", "MX"):
+            self.pairwise(dict(AX="add", SX="sub", MX="mul")[stem],
+                          lambda i: (self.T[i], self.X[0][i]))
+        elif stem == "RX":
+            self.pairwise("sub", lambda i: (self.X[0][i], self.T[i]))
+        elif stem in ("DX", "RDX"):
+            for i in range(self.np):
+                self.e(f"mov.b64 %%U{i}, {self.X[0][i]};")
+        self.e(f"mov.u32 %%dv, {to};")
+        self.next_column()
+        self.e("bra.uni " + ("N", "DTU", "RDU")[to] + "%=;")
+
     # cheap bodies (no range test, a handful of instructions) end with a
     # plain branch to the next word; in the gradient variant the others
     # return through ret, and the marked words of the cheap ones run a copy
@@ -767,6 +837,9 @@ class Gen:
         own branch (the divisions go on to the shared division body)"""
         e, p, X = self.e, self.np, self.X
         stem, col = self.stem(name)
+        if self.xmem and stem in ("PX", "PXS", "AX", "SX", "MX", "RX", "DX", "RDX"):
+            self.xmem_body(stem)
+            return True
         if stem == "PX" or stem == "PXS":
             if stem == "PXS":
                 self.spill()
@@ -859,14 +932,15 @@ class Gen:
             for k, v in dict(DIV_S="DS", DIV_C="DC", RDIV_C="RDC", SQRT="SQ", INV="IV",
                              SIN="TRG", COS="TRG", LOG="LG", EXP="XP").items():
                 ent[OPS[k]] = v
-        if self.xreg:
+        if self.xreg or self.xmem:
             xops = dict(PUSH_X="PX", PUSH_X_SP="PXS", ADD_X="AX", SUB_X="SX", RSUB_X="RX",
                         MUL_X="MX")
             if self.divs:
                 xops.update(DIV_X="DX", RDIV_X="RDX")
             for k, v in xops.items():
-                ent[OPS[k]] = v + "0"
-                ent[OPS[k] | COL1] = v + "1"
+                ent[OPS[k]] = v if self.xmem else v + "0"
+                if not self.xmem:
+                    ent[OPS[k] | COL1] = v + "1"
         if self.grad:
             ent[OPS["END"] | COL1] = "MK"
         owner = {}
@@ -890,6 +964,13 @@ class Gen:
         e(f".reg .b64 %%C, %%U<{p}>, %%K<2>, %%KM, %%JM, %%JJ, %%R, %%S, %%P, %%Q, %%F;")
         if self.divs and self.special:
             e(".reg .b64 %%Y;")
+        if self.xmem:
+            e(".reg .pred %%pm, %%pb;")
+            e(".reg .b64 %%xa;")
+            e(".reg .b32 %%dv;")
+            e("TD%=: .branchtargets N%=, DTU%=, RDU%=;")
+            e(f"setp.ne.u32 %%pm, {self.MODE}, 0;")
+            e(f"setp.eq.u32 %%pb, {self.MODE}, 2;")
         e("T%=: .branchtargets " + ", ".join(f"{x}%=" for x in ent) + ";")
         if self.grad:
             part = self.partial_labels(ent)
@@ -937,6 +1018,18 @@ class Gen:
             self.label("DTU")
             self.div_body()
             self.nxt()
+            if self.xmem:
+                # t = u / t, the dividend pairs in U: swap, then divide
+                self.label("RDU")
+
+                def swap():
+                    for i in range(p):
+                        e(f"mov.b64 %%S, {self.T[i]};")
+                        e(f"mov.b64 {self.T[i]}, %%U{i};")
+                        e(f"mov.b64 %%U{i}, %%S;")
+                self.div_check(num=lambda i: f"%%U{i}", den=lambda i: self.T[i], pre=swap)
+                swap()
+                e("bra.uni DTUX%=;")
         if self.grad:
             # stubs into the shared bodies: ret = the word's index + 1 (TR)
             done = set()
@@ -950,6 +1043,8 @@ class Gen:
                 e(f"bra.uni {lab[1:]}%=;")
             self.partial_bodies(sorted(set(tr[1:]) - {"EX"}))
             self.tangent_tail()
+        if self.xmem:
+            self.strided_columns()
         for block in self.deferred:
             block()
         self.label("EX")
@@ -974,13 +1069,19 @@ def function(rpt, divs, xreg, grad=False):
     name = f"fast_r{rpt}_{'divs' if divs else 'nodivs'}_{'x' if xreg else 'nox'}" + \
         ("_grad" if grad else "")
     body = "\n".join(f'        "{ln}\\n\\t"' for ln in lines)
-    outs = ", ".join(['"+r"(pa)'] + [f'"+l"(t[{i}])' for i in range(p)] + ['"=r"(hw)', '"=f"(hc)'])
-    ins = ", ".join(['"r"(sb)', '"n"(NSLOT - 1)'] + [f'"l"(x0[{i}])' for i in range(p)]
-                    + [f'"l"(x1[{i}])' for i in range(p)] + ['"f"(kThr)']
-                    + (['"r"(db)', '"n"(KT)'] if grad else []))
+    xmem = g.xmem
+    outs = ", ".join(['"+r"(pa)'] + [f'"+l"(t[{i}])' for i in range(p)]
+                     + ([f'"+l"(xb[{i}])' for i in range(p)] if xmem else [])
+                     + ['"=r"(hw)', '"=f"(hc)'])
+    ins = ", ".join(['"r"(sb)', '"n"(NSLOT - 1)']
+                    + (['"l"(xc)', '"r"(unit)', '"r"(mode)'] if xmem else
+                       [f'"l"(x0[{i}])' for i in range(p)] + [f'"l"(x1[{i}])' for i in range(p)])
+                    + ['"f"(kThr)'] + (['"r"(db)', '"n"(KT)'] if grad else []))
+    args = (f"uint64_t (&xb)[{p}], const float *xc, uint32_t unit,\n        uint32_t mode"
+            if xmem else f"const uint64_t (&x0)[{p}], const uint64_t (&x1)[{p}]")
     return (f"template <int NSLOT{', int KT' if grad else ''}>\n"
             f"__device__ __forceinline__ void {name}(uint32_t &pa, uint64_t (&t)[{p}],\n"
-            f"        const uint64_t (&x0)[{p}], const uint64_t (&x1)[{p}], uint32_t sb,\n"
+            f"        {args}, uint32_t sb,\n"
             f"        {'uint32_t db, ' if grad else ''}uint32_t &hw, float &hc) {{\n"
             f"    asm volatile(\n{body}\n"
             f"        : {outs}\n"
@@ -996,8 +1097,12 @@ HEADER = '''// gp_fast.cuh -- the evaluator's indexed-branch fast loop in inline
 // the first word it does not run, returns that word and its constant in
 // hw and hc, leaves pa just past it and the rows untouched by it.  sb is
 // the lane's slot-0 address in the shared-memory stack ([slot][q][lane]
-// float4); slots are clamped to NSLOT - 1; x0 and x1 hold columns 0 and 1
-// of the lane's rows (read only by the _x variants).  Every one of the 64
+// float4); slots are clamped to NSLOT - 1.  The _x variants take columns 0
+// and 1 of the lane's rows in x0 and x1; the _nox ones read columns from
+// memory: xb holds the rows of the column that the program reads next, xc
+// is column 0 at the lane's first row, a word's constant times unit the bytes
+// from there to the next column, mode how the lane's rows lie (without the
+// division set, and in the gradient's, column reads are handed back).  Every one of the 64
 // values of the six-bit dispatch index has a table entry.  The statement
 // declares no memory clobber: the shared memory it reads and writes (the
 // code buffer, written before a barrier, and the stack, touched elsewhere

@@ -320,6 +320,11 @@ __global__ void __launch_bounds__(kCompileWarps * 32) compile_kernel(CompileArgs
     // emit, from the end of the list
     int n = 0, sp_car = 0, depth = 0;
     bool ext = false;  // an extended-set instruction was emitted
+    // more than two columns: each column read names the next one; the chunk's
+    // last is completed when a later chunk emits one (at: its place, -1 none)
+    const bool linked = a.n_feat > 2;
+    int link_at = -1;
+    uint32_t first_feat = 0u;
     for (int c = chunks - 1; c >= 0; --c) {
         const int j = c * 32 + lane;
         const bool in = j < len;
@@ -339,14 +344,15 @@ __global__ void __launch_bounds__(kCompileWarps * 32) compile_kernel(CompileArgs
         // operand, j_other: the other operand's node; -1 where the partial
         // derivative is 1 and leaves the tangents as they are)
         int j_top = -1, j_other = -1;
-        bool fresh = false;
+        bool fresh = false, column = false;
         if (emit && ar == 0) {
             const bool x = op == GP_VAR;
             const uint32_t feat = x ? nd.x >> 16 : 0u;
             const bool spill = sp > 0;  // the old top goes to slot sp-1
             const uint32_t w = (spill ? (x ? OP_PUSH_X_SP : OP_PUSH_C_SP) : (x ? OP_PUSH_X : OP_PUSH_C)) |
-                               (feat == 1u ? kOpCol1 : 0u);
+                               (feat == 1u && !linked ? kOpCol1 : 0u);
             word = make_uint2(make_ins(w, spill ? sp - 1 : 0, feat), k ? __float_as_uint(S.val[j]) : nd.y);
+            column = x;
             if (!x) {  // the constant's own tangent starts at 1
                 j_other = j;
                 fresh = true;
@@ -381,7 +387,9 @@ __global__ void __launch_bounds__(kCompileWarps * 32) compile_kernel(CompileArgs
                 // top's tangents as they are)
                 const uint32_t fwd = b == 0 ? OP_ADD_X : b == 1 ? OP_SUB_X : b == 2 ? OP_MUL_X : OP_DIV_X;
                 const uint32_t rev = b == 0 ? OP_ADD_X : b == 1 ? OP_RSUB_X : b == 2 ? OP_MUL_X : OP_RDIV_X;
-                const uint32_t w = (((mode == 1) ? fwd : rev) + (x ? 0u : 1u)) | (feat == 1u ? kOpCol1 : 0u);
+                const uint32_t w = (((mode == 1) ? fwd : rev) + (x ? 0u : 1u)) |
+                                   (feat == 1u && !linked ? kOpCol1 : 0u);
+                column = x;
                 word = make_uint2(make_ins(w, 0, feat), x ? t.y : __float_as_uint(S.val[tj]));
                 j_top = (b == 0 || (b == 1 && mode == 1)) ? -1 : (mode == 1) ? lc : rc;
                 j_other = tj;
@@ -403,18 +411,34 @@ __global__ void __launch_bounds__(kCompileWarps * 32) compile_kernel(CompileArgs
             }
         }
         const unsigned words = __ballot_sync(full, emit), marks = __ballot_sync(full, mark.x != 0u);
+        int at = n + __popc(words & gt) + __popc(marks & gt) + (mark.x != 0u);
+        if (linked) {
+            const unsigned cols = __ballot_sync(full, column);
+            const uint32_t feat = word.x >> 16;
+            const int succ = 31 - __clz(cols & lt);  // the lane emitted next; -1: a later chunk's
+            const uint32_t next = __shfl_sync(full, feat, succ & 31);
+            if (column && succ >= 0) word.y = next;
+            if (cols) {
+                const int head = 31 - __clz(cols), tail = __ffs(cols) - 1;
+                const uint32_t f = __shfl_sync(full, feat, head);
+                if (link_at < 0) first_feat = f;
+                else if (lane == 0) out[link_at].y = f;
+                link_at = __shfl_sync(full, at, tail);
+            }
+        }
         if (emit) {
-            int at = n + __popc(words & gt) + __popc(marks & gt);
-            if (mark.x) out[at++] = mark;
+            if (mark.x) out[at - 1] = mark;
             out[at] = word;
         }
+        __syncwarp();  // (out[link_at] is completed by another lane)
         n += __popc(words) + __popc(marks);
         sp_car += __popc(up) - __popc(down);
     }
     depth = __reduce_max_sync(full, depth);
     ext = __any_sync(full, ext);
     if (lane == 0) {
-        out[n] = make_uint2(make_ins(OP_END, 0, 0), 0u);
+        if (link_at >= 0) out[link_at].y = out[link_at].x >> 16;  // no next: its own
+        out[n] = make_uint2(make_ins(OP_END, 0, 0), first_feat);
         a.meta[p] = ProgMeta{n + 1, GP_PROG_OK, (int16_t)depth, (int16_t)(ext ? 1 : 0), n_consts};
     }
 }

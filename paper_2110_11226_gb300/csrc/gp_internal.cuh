@@ -54,7 +54,14 @@ enum : uint32_t {
     // binary (max, min; the right operand always in a stack slot)
     OP_EXT1 = 30, OP_EXT2 = 31
 };
-constexpr uint32_t kOpCol1 = 32;  // bit 5: a column read of column 1
+// bit 5 of a column read: column 1, with at most two columns.  With more,
+// a column read's word y is the column of the next such word (its rows are
+// prefetched; the last one names its own), and END's word y that of the first
+constexpr uint32_t kOpCol1 = 32;
+// the operations that read a column, one bit each
+constexpr uint32_t kColumnOps = 1u << OP_PUSH_X | 1u << OP_PUSH_X_SP | 1u << OP_ADD_X |
+                                1u << OP_SUB_X | 1u << OP_RSUB_X | 1u << OP_MUL_X | 1u << OP_DIV_X |
+                                1u << OP_RDIV_X;
 
 // Gradient form of a program (forward-mode derivatives with respect to its
 // constants).  The constants are numbered 0, 1, ... in prefix order, so the
@@ -248,6 +255,10 @@ struct EvalArgs {
     float *pred;       // predict mode
     unsigned int *dev_status;
     int vec_ok;
+    // fmode 0: bytes that an offset of the prefetched column reads counts (16,
+    // or 4 for unaligned columns); 0: the table is too large for 32-bit
+    // offsets, and columns are read one by one
+    int x_unit;
     // moments mode (correlation fitness): per-item sums of w d, w d^2 and
     // w d yc with d = p - shift[p], yc = y - ybar
     double *mom;

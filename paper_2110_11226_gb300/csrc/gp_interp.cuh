@@ -254,17 +254,17 @@ static __device__ __noinline__ float4 ext_rows4(float4 v, uint32_t f) {
 // calls and the division's own slow-path call do not mix well).
 template <int RPT, int NSLOT, bool DIVS, bool XREG>
 __device__ __forceinline__ void run_fast(uint32_t &pa, uint64_t (&t)[RPT / 2],
-                                         const uint64_t (&x0)[RPT / 2],
-                                         const uint64_t (&x1)[RPT / 2], uint32_t sb,
+                                         uint64_t (&x0)[RPT / 2], const uint64_t (&x1)[RPT / 2],
+                                         const float *xc, uint32_t unit, uint32_t mode, uint32_t sb,
                                          uint32_t &hw, float &hc) {
     if constexpr (RPT == 4) {
         if constexpr (DIVS && XREG) fast_r4_divs_x<NSLOT>(pa, t, x0, x1, sb, hw, hc);
-        else if constexpr (DIVS) fast_r4_divs_nox<NSLOT>(pa, t, x0, x1, sb, hw, hc);
+        else if constexpr (DIVS) fast_r4_divs_nox<NSLOT>(pa, t, x0, xc, unit, mode, sb, hw, hc);
         else if constexpr (XREG) fast_r4_nodivs_x<NSLOT>(pa, t, x0, x1, sb, hw, hc);
         else fast_r4_nodivs_nox<NSLOT>(pa, t, x0, x1, sb, hw, hc);
     } else {
         if constexpr (DIVS && XREG) fast_r8_divs_x<NSLOT>(pa, t, x0, x1, sb, hw, hc);
-        else if constexpr (DIVS) fast_r8_divs_nox<NSLOT>(pa, t, x0, x1, sb, hw, hc);
+        else if constexpr (DIVS) fast_r8_divs_nox<NSLOT>(pa, t, x0, xc, unit, mode, sb, hw, hc);
         else if constexpr (XREG) fast_r8_nodivs_x<NSLOT>(pa, t, x0, x1, sb, hw, hc);
         else fast_r8_nodivs_nox<NSLOT>(pa, t, x0, x1, sb, hw, hc);
     }
@@ -272,8 +272,10 @@ __device__ __forceinline__ void run_fast(uint32_t &pa, uint64_t (&t)[RPT / 2],
 
 // Runs one compiled program over RPT rows per lane; returns the top of the
 // stack in tp, rows as pairs.  stk = this warp's stack slice, already offset
-// by the lane; xc, packed and last: the chunk's column 0 at the lane's first
-// row, and how the lane's rows follow it (load_pairs).
+// by the lane; xc, packed and last: column 0 at the lane's first row, and how
+// the lane's rows follow it (load_pairs).  x0p and x1p: columns 0 and 1
+// (FMODE 2), else the first column that the program reads in x0p (unit and
+// mode: how the loop reads the next ones, see gp_fast.cuh).
 // The instruction buffer holds the words that the pre-pass wrote, the last
 // of them OP_END; op values that name no operation act as OP_END and stack
 // slots are clamped to the stack.
@@ -290,10 +292,10 @@ __device__ __forceinline__ void run_fast(uint32_t &pa, uint64_t (&t)[RPT / 2],
 // saves the register copies of a prefetch.
 template <int RPT, int NSLOT, int FMODE, bool EXT>
 __device__ __forceinline__ void interpret(uint64_t (&tp)[RPT / 2], const uint2 *__restrict__ cbuf,
-                                          const uint64_t (&x0p)[RPT / 2],
+                                          uint64_t (&x0p)[RPT / 2],
                                           const uint64_t (&x1p)[RPT / 2],
-                                          const float *__restrict__ xc, int64_t ld, bool packed,
-                                          int last, float4 *stk) {
+                                          const float *__restrict__ xc, int64_t ld, uint32_t unit,
+                                          uint32_t mode, bool packed, int last, float4 *stk) {
     // EXT: the extended functions are compiled in (classes 1 and 2).  In
     // class 0, where nearly all programs of the usual function set run,
     // their cases cost 2-3% (measured on Pagie-1 x 4096 programs, which
@@ -313,7 +315,7 @@ __device__ __forceinline__ void interpret(uint64_t (&tp)[RPT / 2], const uint2 *
         uint2 ins;
         if constexpr (kFast) {
             float hc;
-            run_fast<RPT, NSLOT, !EXT, FMODE == 2>(pa, tp, x0p, x1p, sb, ins.x, hc);
+            run_fast<RPT, NSLOT, !EXT, FMODE == 2>(pa, tp, x0p, x1p, xc, unit, mode, sb, ins.x, hc);
             ins.y = __float_as_uint(hc);
         } else {
             asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];"
@@ -525,7 +527,13 @@ __global__ void __launch_bounds__(eval_warps<RPT>() * 32,
         // the program's words (OP_END the last of them)
         if (ok) {
             const uint2 *src = a.code + (size_t)p * (a.code_stride ? a.code_stride : kCodeStride);
-            for (int i = threadIdx.x; i < it.z && i <= kCodeStride; i += kEvalBlock) cbuf[i] = src[i];
+            for (int i = threadIdx.x; i < it.z && i <= kCodeStride; i += kEvalBlock) {
+                uint2 v = src[i];
+                // a column read's constant: the next column read, as an offset
+                if (FMODE == 0 && !EXT && (kColumnOps >> (v.x & 31u) & 1u))
+                    v.y = (uint32_t)((uint64_t)v.y * (uint64_t)(a.x_unit == 16 ? a.ld >> 2 : a.ld));
+                cbuf[i] = v;
+            }
         }
         __syncthreads();  // the words are there
         unsigned long long next = 0;
@@ -534,6 +542,18 @@ __global__ void __launch_bounds__(eval_warps<RPT>() * 32,
         float ks = 0.0f, kc = 0.0f;
         float ms[3] = {0.0f, 0.0f, 0.0f}, mc[3] = {0.0f, 0.0f, 0.0f};
         const float shift = MOM ? a.shift[p] : 0.0f;
+        // FMODE 0: x0 holds the first column that the program reads (END's
+        // constant); its loads for the next sub-tile are issued before the
+        // loss of this one
+        uint64_t x0[RPT / 2], x1[RPT / 2];
+        auto first_column = [&](int base) {
+            const bool pk = base + 32 * RPT <= n_in && a.vec_ok;
+            const int o = base + (pk ? lane * RPT : lane);
+            const int64_t feat = cbuf[s_item[cur].z - 1].y;
+            load_pairs<RPT>(x0, a.X + (feat * a.ld + rb + o), pk, n_in - 1 - o);
+        };
+        constexpr bool kAhead = FMODE == 0 && !EXT;  // the loop reads columns ahead
+        if (kAhead && ok && warp * 32 * RPT < n_in) first_column(warp * 32 * RPT);
         for (int base = warp * 32 * RPT; base < n_in && ok; base += kEvalWarps * 32 * RPT) {
             // whole: every row of the sub-tile is in the chunk; packed: and
             // the lane's rows are consecutive.  One test for the warp
@@ -543,16 +563,16 @@ __global__ void __launch_bounds__(eval_warps<RPT>() * 32,
             const int last = n_in - 1 - o;   // its furthest row (negative: none; see load_pairs)
             const int nv = whole ? RPT : (last + 32) >> 5;  // rows of the lane that count
             const int64_t r = rb + o;
-            uint64_t x0[RPT / 2], x1[RPT / 2];
             if (FMODE == 2) {
                 load_pairs<RPT>(x0, a.X + r, packed, last);
                 load_pairs<RPT>(x1, a.X + (a.ld + r), packed, last);
-            } else {
-#pragma unroll
-                for (int i = 0; i < RPT / 2; ++i) x0[i] = x1[i] = 0;
             }
             uint64_t t[RPT / 2];
-            interpret<RPT, NSLOT, FMODE, EXT>(t, cbuf, x0, x1, a.X + r, a.ld, packed, last, stk);
+            const uint32_t mode = a.x_unit == 0 || !whole ? 2u : packed ? 0u : 1u;
+            interpret<RPT, NSLOT, FMODE, EXT>(t, cbuf, x0, x1, a.X + r, a.ld, (uint32_t)a.x_unit, mode,
+                                              packed, last, stk);
+            if (kAhead && base + kEvalWarps * 32 * RPT < n_in)
+                first_column(base + kEvalWarps * 32 * RPT);
             if (PRED) {
                 float *dst = a.pred + (size_t)p * a.n_rows + r;
                 if (packed) {
