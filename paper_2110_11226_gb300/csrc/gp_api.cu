@@ -432,27 +432,32 @@ int run_predict(const gp_node *progs, const int32_t *offsets, int n_progs, const
 }
 
 // Spearman: the target's ranks once, then batches of programs predicted
-// into [B][N] (B chosen so the batch and its sort buffers take <= 2 GB),
-// ranked and reduced
-constexpr size_t kRankBudget = 2ull << 30;
+// into [B][N], ranked and reduced.  A batch takes up to 4.5 GB (at 1M rows
+// 160 programs, whose splitters are then sorted on every SM at once), or 2 GB
+// when the device has no room for that
+constexpr size_t kRankBudgets[] = {4608ull << 20, 2ull << 30};
 
 int run_spearman(const gp_node *progs, const int32_t *offsets, int n_progs, const float *X,
                  int64_t n_rows, int n_feat, const float *y, const float *w, float *out,
                  double *out64, int32_t *out_status, DevCtx *c, cudaStream_t st) {
     if (n_rows >= ((int64_t)1 << 31) - 2) return GP_ERR_ARG;
-    const int64_t per_prog = n_rows * 4 * 6;  // prediction, 4 sort arrays, slack
-    int B = (int)std::max<int64_t>(1, std::min<int64_t>(n_progs, (int64_t)kRankBudget / per_prog));
-    const size_t b_pred = (size_t)round_up((int64_t)B * n_rows * 4, 256);
+    // prediction, then 4 sort arrays and slack, or the buckets
+    const int64_t per_prog = n_rows * 4 + (int64_t)rank_scratch_bytes(1, n_rows, w != nullptr);
     const size_t b_r2y = (size_t)round_up(n_rows * 4, 256);
     const size_t b_tp = (size_t)round_up((int64_t)target_part_bytes(n_rows), 256);
-    const size_t b_scr = rank_scratch_bytes(B, n_rows);
-    int rc;
+    int rc = GP_ERR_NOMEM, B = 0;
+    size_t b_pred = 0;
     char *base = nullptr;
-    {
+    for (size_t budget : kRankBudgets) {
+        B = (int)std::max<int64_t>(1, std::min<int64_t>(n_progs, (int64_t)budget / per_prog));
+        b_pred = (size_t)round_up((int64_t)B * n_rows * 4, 256);
+        const size_t b_scr = rank_scratch_bytes(B, n_rows, w != nullptr);
         std::lock_guard<std::mutex> g(g_mu);
-        if ((rc = grow(&c->rank, &c->rank_bytes, b_pred + b_r2y + b_tp + b_scr))) return rc;
+        rc = grow(&c->rank, &c->rank_bytes, b_pred + b_r2y + b_tp + b_scr);
         base = static_cast<char *>(c->rank);
+        if (rc == GP_OK) break;
     }
+    if (rc) return rc;
     float *pred = reinterpret_cast<float *>(base);
     uint32_t *r2y = reinterpret_cast<uint32_t *>(base + b_pred);
     double *tpart = reinterpret_cast<double *>(base + b_pred + b_r2y);

@@ -400,7 +400,7 @@ cudaError_t probe_pipes(double *out, cudaStream_t st);
 // values; the target's doubled ranks by row and its per-tile weighted rank
 // sums (target_part_bytes(n) bytes); one batch of predictions [n_seg][n]
 // to fitness
-size_t rank_scratch_bytes(int n_seg, int64_t n);
+size_t rank_scratch_bytes(int n_seg, int64_t n, bool weighted);
 size_t target_part_bytes(int64_t n);
 cudaError_t target_ranks(const float *y, const float *w, int64_t n, void *scratch, uint32_t *r2y,
                          double *tpart, cudaStream_t st);

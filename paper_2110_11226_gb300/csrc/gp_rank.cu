@@ -7,9 +7,14 @@
 // order-preserving 32-bit keys with the row index as payload; the first
 // pass reads the predictions themselves), ties get the mean of their
 // positions, and the weighted moments of the rank pairs are summed in FP64
-// with a fixed partition.  The target's ranks are computed the same way
+// with a fixed partition.  Without weights, and up to 4M rows, the values are
+// ranked bucket by bucket instead (below), and the sort is what remains for
+// segments that the buckets' sample misjudged.  The target's ranks are sorted
 // once per call.  Ranks are kept doubled (first + last position, 1-based),
 // which is an integer; the correlation does not see the factor 2.
+#include <algorithm>
+#include <type_traits>
+
 #include "gp_internal.cuh"
 
 namespace gpk {
@@ -46,15 +51,33 @@ __device__ __forceinline__ uint32_t load_key(const void *src, int64_t m) {
     return static_cast<const uint32_t *>(src)[m];
 }
 
+// The segments that a kernel's blocks work on: all of them, one per
+// blockIdx.y, or, with a list on the device, the *count listed ones, taken
+// in turn by the gridDim.y rows of blocks.
+struct Segs {
+    const int32_t *list;
+    const int32_t *count;
+    int all;
+};
+template <class F>
+__device__ __forceinline__ void each_segment(const Segs &sg, F body) {
+    const int n = sg.list ? *sg.count : sg.all;
+    for (int i = blockIdx.y; i < n; i += gridDim.y) {
+        body(sg.list ? sg.list[i] : i);
+        __syncthreads();  // the next one reuses the shared memory
+    }
+}
+
 // digit counts of one tile: hist[seg][digit][tile].  Each thread loads its
 // 16 keys first (independent loads), then counts them into its warp's own
 // histogram; a warp whose 32 keys share one digit adds once.
 template <bool FROM_FLOAT>
 __global__ void __launch_bounds__(kSortThreads) hist_kernel(const void *__restrict__ src, int64_t n,
                                                             int n_tiles, int shift, int32_t *hist,
-                                                            uint32_t *nan_flag) {
+                                                            uint32_t *nan_flag, Segs sg) {
     __shared__ int32_t wh[kSortWarps][kBins];
-    const int seg = blockIdx.y, tile = blockIdx.x, t = threadIdx.x;
+    each_segment(sg, [&](int seg) {
+    const int tile = blockIdx.x, t = threadIdx.x;
     const int lane = t & 31, warp = t >> 5;
 #pragma unroll
     for (int w = 0; w < kSortWarps; ++w) wh[w][t] = 0;
@@ -94,16 +117,18 @@ __global__ void __launch_bounds__(kSortThreads) hist_kernel(const void *__restri
 #pragma unroll
     for (int w = 0; w < kSortWarps; ++w) c += wh[w][t];
     hist[((int64_t)seg * kBins + t) * n_tiles + tile] = c;
+    });
 }
 
 // per (segment, digit), one warp: exclusive scan of the tile counts in
 // place, and the digit's total in tot[seg][digit]
-__global__ void __launch_bounds__(256) tile_scan_kernel(int32_t *hist, int32_t *tot, int n_rows_hd,
-                                                        int n_tiles) {
+__global__ void __launch_bounds__(256) tile_scan_kernel(int32_t *hist, int32_t *tot, int n_tiles,
+                                                        Segs sg) {
     const int lane = threadIdx.x & 31;
-    const int row = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
-    if (row >= n_rows_hd) return;
-    int32_t *h = hist + (int64_t)row * n_tiles;
+    const int digit = (int)(blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5));  // < kBins
+    each_segment(sg, [&](int seg) {
+    const int64_t row = (int64_t)seg * kBins + digit;
+    int32_t *h = hist + row * n_tiles;
     int32_t carry = 0;
     for (int base = 0; base < n_tiles; base += 32) {
         const int i = base + lane;
@@ -118,6 +143,7 @@ __global__ void __launch_bounds__(256) tile_scan_kernel(int32_t *hist, int32_t *
         carry += __shfl_sync(0xffffffffu, x, 31);
     }
     if (lane == 0) tot[row] = carry;
+    });
 }
 
 // exclusive scan of one value per thread over the block (blockDim.x
@@ -177,14 +203,15 @@ template <bool FROM_FLOAT>
 __global__ void __launch_bounds__(kScatThreads, 2) scatter_kernel(
     const void *__restrict__ src, const uint32_t *__restrict__ vals, int64_t n, int n_tiles,
     int shift, const int32_t *__restrict__ offs, const int32_t *__restrict__ tot,
-    uint32_t *keys_out, uint32_t *vals_out) {
+    uint32_t *keys_out, uint32_t *vals_out, Segs sg) {
     __shared__ uint32_t sk[kSortTile];
     __shared__ uint32_t sv[kSortTile];
     __shared__ int32_t wcnt[kScatWarps][kBins];
     __shared__ int32_t dstart[kBins];
     __shared__ int32_t gbase[kBins];
     __shared__ int32_t wsum[kScatWarps];
-    const int seg = blockIdx.y, tile = blockIdx.x, t = threadIdx.x;
+    each_segment(sg, [&](int seg) {
+    const int tile = blockIdx.x, t = threadIdx.x;
     const int lane = t & 31, warp = t >> 5;
     const int64_t t0 = (int64_t)tile * kSortTile;
     const int tl = (int)min((int64_t)kSortTile, n - t0);
@@ -264,6 +291,7 @@ __global__ void __launch_bounds__(kScatThreads, 2) scatter_kernel(
         keys_out[g] = k;
         vals_out[g] = sv[pos];
     }
+    });
 }
 
 // first index in [lo, hi) of k with k[i] >= v (k ascending)
@@ -290,17 +318,18 @@ __device__ int64_t upper_bound_u32(const uint32_t *k, int64_t lo, int64_t hi, ui
 // key).  One thread per tile; the binary search runs only when the group
 // crosses the edge, which keeps the rank pass free of dependent global loads.
 __global__ void __launch_bounds__(256) edges_kernel(const uint32_t *__restrict__ keys, int64_t n,
-                                                    int n_tiles, int n_seg, int2 *edge) {
-    const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= (int64_t)n_tiles * n_seg) return;
-    const int seg = (int)(g / n_tiles), tile = (int)(g - (int64_t)seg * n_tiles);
+                                                    int n_tiles, int2 *edge, Segs sg) {
+    const int tile = blockIdx.x * blockDim.x + threadIdx.x;
+    each_segment(sg, [&](int seg) {
+    if (tile >= n_tiles) return;
     const uint32_t *k = keys + (int64_t)seg * n;
     const int64_t t0 = (int64_t)tile * kTile;
     const int64_t t1 = min(n, t0 + kTile);  // one past the tile's last key
     const uint32_t first = k[t0], last = k[t1 - 1];
     const int64_t lo = (t0 > 0 && k[t0 - 1] == first) ? lower_bound_u32(k, 0, t0, first) : t0;
     const int64_t hi = (t1 < n && k[t1] == last) ? upper_bound_u32(k, t1, n, last) - 1 : t1 - 1;
-    edge[g] = make_int2((int)lo, (int)hi);
+    edge[(int64_t)seg * n_tiles + tile] = make_int2((int)lo, (int)hi);
+    });
 }
 
 // Doubled average rank of every sorted position (first + last + 2, 1-based
@@ -319,13 +348,14 @@ __global__ void __launch_bounds__(256) edges_kernel(const uint32_t *__restrict__
 __global__ void __launch_bounds__(kTileThreads) rank_kernel(
     const uint32_t *__restrict__ keys, const uint32_t *__restrict__ vals, int64_t n, int n_tiles,
     int mode, const int2 *__restrict__ edge, uint32_t *r2, const uint32_t *__restrict__ r2y,
-    const float *__restrict__ w, double *part, int vals_are_ranks) {
+    const float *__restrict__ w, double *part, int vals_are_ranks, Segs sg) {
     constexpr int kSegs = kTile / 32;  // 32-position segments of the tile
     __shared__ uint32_t sk[kTile];
     __shared__ int16_t sfirst[kTile], slast[kTile];
     __shared__ int seg_first[kSegs], seg_last[kSegs];
     __shared__ double red[3][kTileThreads / 32];
-    const int seg = blockIdx.y, tile = blockIdx.x, t = threadIdx.x;
+    each_segment(sg, [&](int seg) {
+    const int tile = blockIdx.x, t = threadIdx.x;
     const int lane = t & 31;
     const uint32_t *k = keys + (int64_t)seg * n;
     const uint32_t *vl = vals + (int64_t)seg * n;
@@ -469,6 +499,7 @@ __global__ void __launch_bounds__(kTileThreads) rank_kernel(
         for (int q = 0; q < kTileThreads / 32; ++q) v += red[t][q];
         part[((int64_t)seg * n_tiles + tile) * 3 + t] = v;
     }
+    });
 }
 
 // sum of tile triples in a fixed order: lane-strided, then lanes in order
@@ -485,21 +516,38 @@ __device__ __forceinline__ void sum_tiles(const double *p, int n_tiles, double (
         for (int j = 0; j < 3; ++j) S[j] += __shfl_sync(0xffffffffu, s[j], l);
 }
 
-// one warp per segment: |r| of the ranks from the program's tile sums and
-// the target's (sum w, sum w b, sum w b^2)
+// the sums of a's ranks that the bucket path collects: exact integers, the
+// two products as limbs v = hi 2^32 + lo
+struct RankSums {
+    unsigned long long a, a2lo, a2hi, ablo, abhi;
+};
+
+__device__ __forceinline__ double limbs(unsigned long long hi, unsigned long long lo) {
+    return (double)(long long)hi * 4294967296.0 + (double)(long long)lo;
+}
+
+// one warp per segment: |r| of the ranks from the program's sums -- exact
+// (sums; kept: segments of the bucket path) or per tile -- and the target's
+// totals (sum w, sum w b, sum w b^2)
 __global__ void __launch_bounds__(256) spearman_final_kernel(
-    const double *part, const double *tpart, int n_seg, int n_tiles, const uint32_t *nan_flag,
-    float *out, double *out64) {
+    const double *part, const RankSums *sums, const int32_t *listed, const double *total, int n_seg,
+    int n_tiles, const uint32_t *nan_flag, float *out, double *out64) {
     const int lane = threadIdx.x & 31;
     const int seg = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
     if (seg >= n_seg) return;
-    double P[3], T[3];
-    sum_tiles(part + (int64_t)seg * n_tiles * 3, n_tiles, P);
-    sum_tiles(tpart, n_tiles, T);
+    double P[3];
+    if (sums && !listed[seg]) {
+        const RankSums s = sums[seg];
+        P[0] = (double)(long long)s.a;
+        P[1] = limbs(s.a2hi, s.a2lo);
+        P[2] = limbs(s.abhi, s.ablo);
+    } else {
+        sum_tiles(part + (int64_t)seg * n_tiles * 3, n_tiles, P);
+    }
     if (lane != 0) return;
-    const double sw = T[0];
-    const double ma = P[0] / sw, mb = T[1] / sw;
-    const double va = P[1] / sw - ma * ma, vb = T[2] / sw - mb * mb;
+    const double sw = total[0];
+    const double ma = P[0] / sw, mb = total[1] / sw;
+    const double va = P[1] / sw - ma * ma, vb = total[2] / sw - mb * mb;
     const double cov = P[2] / sw - ma * mb;
     double f;
     if (nan_flag[seg] || !isfinite(va) || !isfinite(vb) || !isfinite(cov)) f = __longlong_as_double(0x7ff8000000000000LL);
@@ -509,17 +557,24 @@ __global__ void __launch_bounds__(256) spearman_final_kernel(
     if (out64) out64[seg] = f;
 }
 
+// the target's totals after its tile sums
+__global__ void __launch_bounds__(32) target_total_kernel(const double *tpart, int n_tiles,
+                                                          double *total) {
+    double T[3];
+    sum_tiles(tpart, n_tiles, T);
+    if (threadIdx.x < 3) total[threadIdx.x] = T[threadIdx.x];
+}
+
 // Sorts each of n_seg segments of n float values into keys (order-preserving
 // integers) with the row index as payload, or payload[row] when a per-row
 // table is given; the result is in keys/vals.
 // hist holds n_seg * 256 * n_tiles counts, tot n_seg * 256.
 cudaError_t radix_sort_values(const float *v, uint32_t *keys, uint32_t *vals, uint32_t *keys2,
-                              uint32_t *vals2, int n_seg, int64_t n, int32_t *hist, int32_t *tot,
-                              uint32_t *nan_flag, const uint32_t *payload, cudaStream_t st) {
+                              uint32_t *vals2, int64_t n, int32_t *hist, int32_t *tot,
+                              uint32_t *nan_flag, const uint32_t *payload, const Segs &sg,
+                              int rows_of_blocks, cudaStream_t st) {
     const int n_tiles = (int)((n + kSortTile - 1) / kSortTile);
-    const dim3 grid(n_tiles, n_seg);
-    const int scan_rows = n_seg * kBins;
-    const int scan_blocks = (scan_rows + 7) / 8;
+    const dim3 grid(n_tiles, rows_of_blocks), scan_grid(kBins / 8, rows_of_blocks);
     for (int pass = 0; pass < kPasses; ++pass) {
         const int shift = pass * kRadixBits;
         // pass 0: values -> keys2; then keys2 -> keys -> keys2 -> keys
@@ -528,20 +583,485 @@ cudaError_t radix_sort_values(const float *v, uint32_t *keys, uint32_t *vals, ui
         uint32_t *ko = (pass & 1) ? keys : keys2;
         uint32_t *vo = (pass & 1) ? vals : vals2;
         if (pass == 0) {
-            hist_kernel<true><<<grid, kSortThreads, 0, st>>>(v, n, n_tiles, shift, hist, nan_flag);
+            hist_kernel<true><<<grid, kSortThreads, 0, st>>>(v, n, n_tiles, shift, hist, nan_flag, sg);
         } else {
-            hist_kernel<false><<<grid, kSortThreads, 0, st>>>(ki, n, n_tiles, shift, hist, nullptr);
+            hist_kernel<false><<<grid, kSortThreads, 0, st>>>(ki, n, n_tiles, shift, hist, nullptr, sg);
         }
-        tile_scan_kernel<<<scan_blocks, 256, 0, st>>>(hist, tot, scan_rows, n_tiles);
+        tile_scan_kernel<<<scan_grid, 256, 0, st>>>(hist, tot, n_tiles, sg);
         if (pass == 0) {
             scatter_kernel<true><<<grid, kScatThreads, 0, st>>>(v, payload, n, n_tiles, shift, hist,
-                                                                tot, ko, vo);
+                                                                tot, ko, vo, sg);
         } else {
             scatter_kernel<false><<<grid, kScatThreads, 0, st>>>(ki, vi, n, n_tiles, shift, hist,
-                                                                 tot, ko, vo);
+                                                                 tot, ko, vo, sg);
         }
     }
     return cudaGetLastError();  // 4 passes: the result is in keys/vals
+}
+
+// ---- ranks by buckets --------------------------------------------------
+// Without weights the coefficient needs each value's rank only next to the
+// target's rank of its row, so no segment has to be sorted as a whole:
+//   splitter_kernel   a sorted sample of the segment's keys gives splitters
+//                     for buckets of about kBucketAim keys
+//   partition_kernel  every key goes, with the target's rank of its row, to
+//                     its bucket (of at most kBucketCap places).  Keys equal
+//                     to a splitter -- every value frequent enough to fill a
+//                     bucket is one -- need no place: they share one rank, so
+//                     their number and the sum of their targets' ranks do
+//   base_kernel       first position of every bucket; the splitters' shares
+//   local_kernel      a bucket in shared memory: 4096 equal bins over its key
+//                     range, about one key each, then a key's rank is the
+//                     bin's start plus the smaller keys in the bin
+// The sums are integers and exact, so no order shows in them.  A segment
+// with an overfull bucket (the sample misjudged it) is listed, and the radix
+// sort below runs for the listed segments alone.
+// Bound by the global traffic of the partition (4 B read, 8 B written as runs
+// of about 6 keys, 8 B read) and shared-memory atomics; the radix sort moves
+// 84 B a key and spends about 800 instructions on it, these 158 and 208 in
+// the last two steps.  512 programs x 1M rows: 20.4 -> 10.9 ms; a batch of 156
+// programs takes 0.50 ms of predictions, 0.12 of splitters, 1.34 of
+// partition (tiles of 4096 keys or other block sizes: 1.42 to 1.65) and 1.42
+// of local ranks.
+constexpr int kBucketCap = 6144;
+constexpr int kBucketAim = kBucketCap / 3;
+constexpr int kMaxBuckets = 2048;
+constexpr int kOversample = 16;  // sampled keys per bucket
+constexpr int kPartThreads = 512, kPartItems = 16, kPartTile = kPartThreads * kPartItems;
+constexpr int kLocThreads = 512, kLocItems = kBucketCap / kLocThreads, kLocBins = 4096;
+constexpr int kLocKeys = 8192;   // kBucketCap to a power of two, for the bitonic sort
+constexpr int kCrowded = 128;  // keys in one bin that make the bucket sort
+
+static inline int pow2_at_least(int v) {
+    int p = 1;
+    while (p < v) p *= 2;
+    return p;
+}
+// a few thousand rows are one bucket, taken straight from the predictions
+static inline int bucket_count(int64_t n) {
+    return n <= kBucketCap ? 1 : (int)std::min<int64_t>((n + kBucketAim - 1) / kBucketAim, kMaxBuckets + 1);
+}
+// weighted sums are FP64 and need a fixed order; beyond kMaxBuckets the
+// partition's runs get too short
+static inline bool bucket_path(const float *w, int64_t n) {
+    return w == nullptr && bucket_count(n) <= kMaxBuckets;
+}
+
+// per segment of a batch
+struct Buckets {
+    int nb, p2;               // buckets; splitters padded to a power of two
+    uint32_t *split;          // [seg][p2], ascending, then 0xffffffff
+    int32_t *cnt, *eqc;       // [seg][nb] keys in the bucket, equal to its splitter
+    unsigned long long *eqb;  // [seg][nb] sum of the targets' centred ranks of the latter
+    int32_t *base;            // [seg][nb] first position
+    RankSums *sums;           // [seg]
+    int32_t *listed;          // [seg] 1: left to the radix sort
+    int32_t *list, *count;    // those segments
+    uint2 *kv;                // [seg][nb][kBucketCap]
+};
+
+// ascending bitonic sort of p2 keys in shared memory by the whole block
+__device__ void bitonic_sort(uint32_t *k, int p2) {
+    for (int size = 2; size <= p2; size *= 2)
+        for (int d = size / 2; d > 0; d /= 2) {
+            __syncthreads();
+            for (int i = threadIdx.x; i < p2 / 2; i += blockDim.x) {
+                const int lo = 2 * i - (i & (d - 1)), hi = lo + d;
+                const uint32_t a = k[lo], b = k[hi];
+                const bool up = (lo & size) == 0;
+                k[lo] = up ? min(a, b) : max(a, b);
+                k[hi] = up ? max(a, b) : min(a, b);
+            }
+        }
+    __syncthreads();
+}
+
+__global__ void __launch_bounds__(1024) splitter_kernel(const float *__restrict__ pred, int64_t n,
+                                                        int samples, Buckets B, uint32_t *nan_flag) {
+    extern __shared__ uint32_t sample[];
+    const int seg = blockIdx.x, t = threadIdx.x;
+    const float *v = pred + (int64_t)seg * n;
+    for (int i = t; i < samples; i += blockDim.x)
+        sample[i] = float_key(v[((int64_t)(2 * i + 1) * n) / (2 * (int64_t)samples)]);
+    for (int j = t; j < B.nb; j += blockDim.x) {
+        const int64_t q = (int64_t)seg * B.nb + j;
+        B.cnt[q] = 0;
+        B.eqc[q] = 0;
+        B.eqb[q] = 0ull;
+    }
+    if (t == 0) {
+        B.sums[seg] = RankSums{0ull, 0ull, 0ull, 0ull, 0ull};
+        B.listed[seg] = 0;
+        nan_flag[seg] = 0u;
+        if (seg == 0) *B.count = 0;
+    }
+    bitonic_sort(sample, samples);
+    for (int j = t; j < B.p2; j += blockDim.x)
+        B.split[(int64_t)seg * B.p2 + j] =
+            j < B.nb - 1 ? sample[((int64_t)(j + 1) * samples) / B.nb] : 0xffffffffu;
+}
+
+__global__ void __launch_bounds__(kPartThreads, 2) partition_kernel(
+    const float *__restrict__ pred, int64_t n, const uint32_t *__restrict__ r2y, Buckets B,
+    uint32_t *nan_flag) {
+    extern __shared__ uint32_t smem_part[];
+    uint2 *stage = reinterpret_cast<uint2 *>(smem_part);                      // [kPartTile]
+    int2 *place = reinterpret_cast<int2 *>(stage + kPartTile);                // [nb] see below
+    uint32_t *split = reinterpret_cast<uint32_t *>(place + B.nb);             // [p2]
+    uint32_t *tree = split + B.p2;                                            // [p2] see below
+    int32_t *cnt = reinterpret_cast<int32_t *>(tree + B.p2);                  // [nb] the tile's counts
+    uint16_t *sj = reinterpret_cast<uint16_t *>(cnt + B.nb);                  // [kPartTile] bucket
+    __shared__ int32_t wsum[kPartThreads / 32];
+    const int seg = blockIdx.y, t = threadIdx.x, lane = t & 31;
+    const int64_t t0 = (int64_t)blockIdx.x * kPartTile;
+    const int tl = (int)min((int64_t)kPartTile, n - t0);
+    const float *v = pred + (int64_t)seg * n + t0;
+    uint32_t key[kPartItems];
+    int j[kPartItems];
+    bool nan = false;
+#pragma unroll
+    for (int r = 0; r < kPartItems; ++r) {
+        const int i = r * kPartThreads + t;
+        const float f = i < tl ? v[i] : 0.0f;
+        nan |= f != f;
+        key[r] = float_key(f);
+        j[r] = 1;
+    }
+    // the splitters as a search tree by levels (node i over nodes 2i and
+    // 2i + 1): a level's nodes lie side by side, so the lanes' reads of the
+    // upper levels meet no bank twice (a binary search over the sorted array
+    // reads addresses 32 apart there, all in one bank)
+    for (int i = t; i < B.p2; i += kPartThreads) {
+        const uint32_t *sp = B.split + (int64_t)seg * B.p2;
+        split[i] = sp[i];
+        if (i == 0) continue;  // node 1 is the root
+        const int level = 31 - __clz(i);
+        tree[i] = sp[(2 * (i - (1 << level)) + 1) * (B.p2 >> (level + 1)) - 1];
+    }
+    for (int i = t; i < B.nb; i += kPartThreads) cnt[i] = 0;
+    if (__any_sync(0xffffffffu, nan) && lane == 0) atomicOr(nan_flag + seg, 1u);
+    __syncthreads();
+    // the number of splitters below the key
+    for (int size = B.p2; size > 1; size /= 2) {
+#pragma unroll
+        for (int r = 0; r < kPartItems; ++r) j[r] = 2 * j[r] + (tree[j[r]] < key[r] ? 1 : 0);
+    }
+    int off[kPartItems];  // place in the tile's share of the bucket; -1: none needed
+#pragma unroll
+    for (int r = 0; r < kPartItems; ++r) {
+        const int i = r * kPartThreads + t;
+        const bool in = i < tl;
+        j[r] = min(j[r] - B.p2, B.nb - 1);
+        const bool eq = in && j[r] < B.nb - 1 && split[j[r]] == key[r];
+        off[r] = in && !eq ? atomicAdd(&cnt[j[r]], 1) : -1;
+        unsigned em = __ballot_sync(0xffffffffu, eq);
+        while (em) {  // the lanes equal to one splitter add once
+            const int src = __ffs(em) - 1;
+            const int j0 = __shfl_sync(0xffffffffu, j[r], src);
+            const bool mine = eq && j[r] == j0;
+            const unsigned mm = __ballot_sync(0xffffffffu, mine);
+            const int b = mine ? (int)((int64_t)r2y[t0 + i] - (n + 1)) : 0;
+            const int sb = __reduce_add_sync(0xffffffffu, b);  // 32 |b| < 2^31
+            if (lane == src) {
+                const int64_t q = (int64_t)seg * B.nb + j0;
+                atomicAdd(&B.eqc[q], __popc(mm));
+                atomicAdd(&B.eqb[q], (unsigned long long)(long long)sb);
+            }
+            em &= ~mm;
+        }
+    }
+    __syncthreads();
+    // place[b]: the first of bucket b's keys in the tile, and from there to
+    // their places in the bucket (at most 4 buckets per thread)
+    int run = 0, c[kMaxBuckets / kPartThreads];
+    const int per = (B.nb + kPartThreads - 1) / kPartThreads;
+#pragma unroll
+    for (int q = 0; q < kMaxBuckets / kPartThreads; ++q) {
+        const int b = t * per + q;
+        c[q] = q < per && b < B.nb ? cnt[b] : 0;
+        run += c[q];
+    }
+    int start = block_exclusive_scan(run, wsum);
+#pragma unroll
+    for (int q = 0; q < kMaxBuckets / kPartThreads; ++q) {
+        const int b = t * per + q;
+        if (q < per && b < B.nb) {
+            const int at = c[q] ? atomicAdd(&B.cnt[(int64_t)seg * B.nb + b], c[q]) : 0;
+            place[b] = make_int2(start, at - start);
+        }
+        start += c[q];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < kPartItems; ++r) {
+        if (off[r] < 0) continue;
+        const int pos = place[j[r]].x + off[r];
+        stage[pos] = make_uint2(key[r], r2y[t0 + r * kPartThreads + t]);
+        sj[pos] = (uint16_t)j[r];
+    }
+    if (t == kPartThreads - 1) wsum[0] = start;  // the keys staged in all
+    __syncthreads();
+    const int m = wsum[0];
+    uint2 *kv = B.kv + (int64_t)seg * B.nb * kBucketCap;
+    for (int pos = t; pos < m; pos += kPartThreads) {
+        const int b = sj[pos], at = place[b].y + pos;
+        if (at < kBucketCap) kv[(int64_t)b * kBucketCap + at] = stage[pos];
+    }
+}
+
+// adds to a segment's sums: its a, and products as limbs (exact)
+__device__ __forceinline__ void add_sums(RankSums *s, long long a, unsigned long long a2lo,
+                                         long long a2hi, unsigned long long ablo, long long abhi) {
+    atomicAdd(&s->a, (unsigned long long)a);
+    atomicAdd(&s->a2lo, a2lo);
+    atomicAdd(&s->a2hi, (unsigned long long)a2hi);
+    atomicAdd(&s->ablo, ablo);
+    atomicAdd(&s->abhi, (unsigned long long)abhi);
+}
+
+constexpr long long kLow32 = 0xffffffffll;
+
+__global__ void __launch_bounds__(256) base_kernel(int64_t n, Buckets B) {
+    __shared__ int32_t wsum[8];
+    const int seg = blockIdx.x, t = threadIdx.x;
+    const int per = (B.nb + 255) / 256;  // <= 8
+    int run = 0;
+    bool over = false;
+    for (int q = 0; q < per; ++q) {
+        const int b = t * per + q;
+        if (b >= B.nb) break;
+        const int64_t at = (int64_t)seg * B.nb + b;
+        over |= B.cnt[at] > kBucketCap;
+        run += B.cnt[at] + B.eqc[at];
+    }
+    int pos = block_exclusive_scan(run, wsum);
+    over = __syncthreads_or(over);
+    if (over && t == 0) {
+        B.listed[seg] = 1;
+        B.list[atomicAdd(B.count, 1)] = seg;
+    }
+    for (int q = 0; q < per; ++q) {
+        const int b = t * per + q;
+        if (b >= B.nb) break;
+        const int64_t at = (int64_t)seg * B.nb + b;
+        B.base[at] = pos;
+        pos += B.cnt[at];
+        const int c = B.eqc[at];
+        if (c) {  // positions pos .. pos + c - 1 (0-based) share the doubled rank
+            const long long a = 2ll * pos + c + 1 - (n + 1), a2 = a * a;
+            const long long sb = (long long)B.eqb[at];
+            // a sb in 128 bits, as limbs
+            const unsigned long long ab = (unsigned long long)(a * sb);
+            const long long abhi = (long long)((unsigned long long)__mul64hi(a, sb) << 32 | ab >> 32);
+            add_sums(&B.sums[seg], c * a, (unsigned long long)(c * (a2 & kLow32)), c * (a2 >> 32),
+                     ab & (unsigned long long)kLow32, abhi);
+        }
+        pos += c;
+    }
+}
+
+// DIRECT: the segment is one bucket, read from the predictions themselves
+template <bool DIRECT>
+__global__ void __launch_bounds__(kLocThreads, 3) local_kernel(
+    const float *__restrict__ pred, const uint32_t *__restrict__ r2y, int64_t n, Buckets B,
+    uint32_t *nan_flag) {
+    __shared__ __align__(16) uint32_t bins[kLocBins + 4];
+    extern __shared__ uint32_t keys[];  // [kLocKeys]
+    __shared__ int32_t wsum[kLocThreads / 32];
+    __shared__ uint32_t s_lo, s_hi;
+    __shared__ long long red[3][kLocThreads / 32];
+    const int seg = DIRECT ? blockIdx.x : blockIdx.y, t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int64_t q = DIRECT ? 0 : (int64_t)seg * B.nb + blockIdx.x;
+    const int m = DIRECT ? (int)n : B.cnt[q];
+    if (m == 0 || m > kBucketCap) return;  // overfull: the segment is listed
+    const int64_t base = DIRECT ? 0 : B.base[q];
+    // the key range: between the bucket's splitters, or, at the segment's
+    // ends, the keys' own
+    const bool ends = DIRECT || blockIdx.x == 0 || blockIdx.x == B.nb - 1;
+    uint32_t lo = 0xffffffffu, hi = 0u;
+    if (!ends) {
+        lo = B.split[(int64_t)seg * B.p2 + blockIdx.x - 1] + 1u;
+        hi = B.split[(int64_t)seg * B.p2 + blockIdx.x] - 1u;
+    }
+    uint32_t key[kLocItems];
+    bool nan = false;
+#pragma unroll
+    for (int r = 0; r < kLocItems; ++r) {
+        if (r * kLocThreads >= m) break;
+        const int i = r * kLocThreads + t;
+        key[r] = 0u;
+        if (i < m) {
+            if (DIRECT) {
+                const float f = pred[(int64_t)seg * n + i];
+                nan |= f != f;
+                key[r] = float_key(f);
+            } else {
+                key[r] = B.kv[q * kBucketCap + i].x;
+            }
+            if (ends) {
+                lo = min(lo, key[r]);
+                hi = max(hi, key[r]);
+            }
+        }
+    }
+    uint4 *bins4 = reinterpret_cast<uint4 *>(bins);
+    static_assert(kLocBins == 8 * kLocThreads, "two uint4 of bins per thread");
+    bins4[t] = bins4[kLocThreads + t] = make_uint4(0u, 0u, 0u, 0u);
+    if (t == 0) {
+        s_lo = 0xffffffffu;
+        s_hi = 0u;
+    }
+    if (DIRECT) nan = __syncthreads_or(nan);
+    else __syncthreads();
+    if (ends) {
+        lo = __reduce_min_sync(0xffffffffu, lo);
+        hi = __reduce_max_sync(0xffffffffu, hi);
+        if (lane == 0) {
+            atomicMin(&s_lo, lo);
+            atomicMax(&s_hi, hi);
+        }
+        __syncthreads();
+        lo = s_lo;
+        hi = s_hi;
+    }
+    // bin = (key - lo) kLocBins / (range + 1), rounded down; key - lo itself
+    // when that is below kLocBins (the quotient in FP32, 2^-22 too small, so
+    // the largest key stays below the last bin's end)
+    const uint32_t range = hi - lo;
+    const uint32_t mult =
+        range < kLocBins ? 0u
+                         : (uint32_t)__fdiv_rd((float)kLocBins * 4294967296.0f * (1.0f - 0x1p-22f),
+                                               __uint2float_ru(range));
+    auto bin_of = [&](uint32_t k) { return mult ? __umulhi(k - lo, mult) : k - lo; };
+    uint32_t off[kLocItems];
+#pragma unroll
+    for (int r = 0; r < kLocItems; ++r) {
+        if (r * kLocThreads >= m) break;
+        if (r * kLocThreads + t < m) off[r] = atomicAdd(&bins[bin_of(key[r])], 1u);
+    }
+    __syncthreads();
+    uint32_t most;
+    {
+        const uint4 u = bins4[2 * t], v = bins4[2 * t + 1];
+        const uint32_t c[8] = {u.x, u.y, u.z, u.w, v.x, v.y, v.z, v.w};
+        uint32_t run = 0u, x[8];
+        most = 0u;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            x[i] = run;
+            run += c[i];
+            most = max(most, c[i]);
+        }
+        const uint32_t at = (uint32_t)block_exclusive_scan((int32_t)run, wsum);
+        bins4[2 * t] = make_uint4(at + x[0], at + x[1], at + x[2], at + x[3]);
+        bins4[2 * t + 1] = make_uint4(at + x[4], at + x[5], at + x[6], at + x[7]);
+        if (t == kLocThreads - 1) bins[kLocBins] = at + run;
+    }
+    // a bin with many keys of one value is fine only where one value fills it
+    const bool crowded = __syncthreads_or(most > kCrowded && mult != 0u);
+#pragma unroll
+    for (int r = 0; r < kLocItems; ++r) {
+        if (r * kLocThreads >= m) break;
+        if (r * kLocThreads + t < m) keys[bins[bin_of(key[r])] + off[r]] = key[r];
+    }
+    if (crowded) {
+        const int p2 = 1 << (32 - __clz(max(m - 1, 1)));
+        for (int i = m + t; i < p2; i += kLocThreads) keys[i] = 0xffffffffu;
+        bitonic_sort(keys, p2);
+    }
+    __syncthreads();
+    long long s[3] = {0, 0, 0};
+#pragma unroll
+    for (int r = 0; r < kLocItems; ++r) {
+        if (r * kLocThreads >= m) break;
+        if (r * kLocThreads + t >= m) continue;
+        const uint32_t k = key[r];
+        int less, same;
+        if (crowded) {
+            int x = 0, y = m;
+            while (x < y) {
+                const int mid = (x + y) / 2;
+                if (keys[mid] < k) x = mid + 1;
+                else y = mid;
+            }
+            less = x;
+            y = m;
+            while (x < y) {
+                const int mid = (x + y) / 2;
+                if (keys[mid] <= k) x = mid + 1;
+                else y = mid;
+            }
+            same = x - less;
+        } else if (mult == 0u) {  // one value per bin
+            less = (int)bins[k - lo];
+            same = (int)bins[k - lo + 1] - less;
+        } else {
+            const uint32_t bin = bin_of(k);
+            const int b0 = (int)bins[bin], b1 = (int)bins[bin + 1];
+            less = b0;
+            same = 0;
+            for (int x = b0; x < b1; ++x) {
+                less += keys[x] < k;
+                same += keys[x] == k;
+            }
+        }
+        const long long a = 2ll * (base + less) + same + 1 - (n + 1);
+        // the target's rank, from the cache: held in a register since the key's
+        // load it would cost a resident block
+        const int i = r * kLocThreads + t;
+        const long long b = (long long)(DIRECT ? r2y[i] : B.kv[q * kBucketCap + i].y) - (n + 1);
+        s[0] += a;
+        s[1] += a * a;
+        s[2] += a * b;
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s[k] += __shfl_xor_sync(0xffffffffu, s[k], o);
+        if (lane == 0) red[k][warp] = s[k];
+    }
+    __syncthreads();
+    if (t != 0) return;
+    for (int w = 1; w < kLocThreads / 32; ++w)
+        for (int k = 0; k < 3; ++k) red[k][0] += red[k][w];
+    const unsigned long long a2lo = red[1][0] & kLow32, ablo = red[2][0] & kLow32;
+    if (DIRECT) {
+        B.sums[seg] = RankSums{(unsigned long long)red[0][0], a2lo, (unsigned long long)(red[1][0] >> 32),
+                               ablo, (unsigned long long)(red[2][0] >> 32)};
+        B.listed[seg] = 0;
+        nan_flag[seg] = nan ? 1u : 0u;
+    } else {
+        add_sums(&B.sums[seg], red[0][0], a2lo, red[1][0] >> 32, ablo, red[2][0] >> 32);
+    }
+}
+
+size_t partition_smem(const Buckets &B) {
+    return (size_t)kPartTile * (sizeof(uint2) + sizeof(uint16_t)) + (size_t)B.p2 * 8 + (size_t)B.nb * 12;
+}
+
+cudaError_t bucket_ranks(const float *pred, int n_seg, int64_t n, const uint32_t *r2y,
+                         const Buckets &B, uint32_t *nan_flag, cudaStream_t st) {
+    const size_t smem_l = kLocKeys * sizeof(uint32_t);
+    cudaError_t e = cudaFuncSetAttribute(B.nb == 1 ? local_kernel<true> : local_kernel<false>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_l);
+    if (e != cudaSuccess) return e;
+    if (B.nb == 1) {
+        local_kernel<true><<<n_seg, kLocThreads, smem_l, st>>>(pred, r2y, n, B, nan_flag);
+        return cudaGetLastError();
+    }
+    const int samples = pow2_at_least(B.nb * kOversample);
+    const size_t smem_s = (size_t)samples * 4, smem_p = partition_smem(B);
+    e = cudaFuncSetAttribute(splitter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)smem_s);
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(partition_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_p);
+    if (e != cudaSuccess) return e;
+    splitter_kernel<<<n_seg, std::min(1024, samples / 2), smem_s, st>>>(pred, n, samples, B, nan_flag);
+    const dim3 tiles((unsigned)((n + kPartTile - 1) / kPartTile), n_seg);
+    partition_kernel<<<tiles, kPartThreads, smem_p, st>>>(pred, n, r2y, B, nan_flag);
+    base_kernel<<<n_seg, 256, 0, st>>>(n, B);
+    local_kernel<false><<<dim3(B.nb, n_seg), kLocThreads, smem_l, st>>>(pred, r2y, n, B, nan_flag);
+    return cudaGetLastError();
 }
 
 }  // namespace
@@ -558,45 +1078,90 @@ struct RankScratch {
     size_t bytes;
 };
 
-RankScratch carve_rank(void *scratch, int n_seg, int64_t n) {
+RankScratch carve_rank(void *scratch, int n_seg, int64_t n, bool buckets, Buckets *B) {
     const int64_t sort_tiles = (n + kSortTile - 1) / kSortTile;
     const int64_t rank_tiles = (n + kTile - 1) / kTile;
     auto al = [](int64_t x) { return (size_t)((x + 255) / 256 * 256); };
     char *b = static_cast<char *>(scratch);
     RankScratch r{};
     size_t o = 0;
-    const size_t arr = al((int64_t)n_seg * n * 4);
-    r.keys = reinterpret_cast<uint32_t *>(b + o); o += arr;
-    r.vals = reinterpret_cast<uint32_t *>(b + o); o += arr;
-    r.keys2 = reinterpret_cast<uint32_t *>(b + o); o += arr;
-    r.vals2 = reinterpret_cast<uint32_t *>(b + o); o += arr;
-    r.hist = reinterpret_cast<int32_t *>(b + o); o += al((int64_t)n_seg * kBins * sort_tiles * 4);
-    r.tot = reinterpret_cast<int32_t *>(b + o); o += al((int64_t)n_seg * kBins * 4);
-    r.part = reinterpret_cast<double *>(b + o); o += al((int64_t)n_seg * rank_tiles * 3 * 8);
-    r.edge = reinterpret_cast<int2 *>(b + o); o += al((int64_t)n_seg * rank_tiles * 8);
-    r.nan_flag = reinterpret_cast<uint32_t *>(b + o); o += al((int64_t)n_seg * 4);
-    r.bytes = o;
+    auto take = [&](auto **p, int64_t bytes) {
+        *p = reinterpret_cast<std::remove_reference_t<decltype(*p)>>(b + o);
+        o += al(bytes);
+    };
+    take(&r.nan_flag, (int64_t)n_seg * 4);
+    size_t end = 0;
+    if (buckets) {
+        *B = Buckets{};
+        B->nb = bucket_count(n);
+        B->p2 = pow2_at_least(B->nb);
+        take(&B->sums, (int64_t)n_seg * sizeof(RankSums));
+        take(&B->listed, (int64_t)n_seg * 4);
+        if (B->nb > 1) {
+            take(&B->split, (int64_t)n_seg * B->p2 * 4);
+            take(&B->cnt, (int64_t)n_seg * B->nb * 4);
+            take(&B->eqc, (int64_t)n_seg * B->nb * 4);
+            take(&B->eqb, (int64_t)n_seg * B->nb * 8);
+            take(&B->base, (int64_t)n_seg * B->nb * 4);
+            take(&B->list, (int64_t)n_seg * 4);
+            take(&B->count, 4);
+            // the buckets lie where the radix sort's arrays do: it runs after
+            // they are done with
+            B->kv = reinterpret_cast<uint2 *>(b + o);
+            end = o + al((int64_t)n_seg * B->nb * kBucketCap * 8);
+        } else {
+            r.bytes = o;  // one bucket never overflows
+            return r;
+        }
+    }
+    take(&r.keys, (int64_t)n_seg * n * 4);
+    take(&r.vals, (int64_t)n_seg * n * 4);
+    take(&r.keys2, (int64_t)n_seg * n * 4);
+    take(&r.vals2, (int64_t)n_seg * n * 4);
+    take(&r.hist, (int64_t)n_seg * kBins * sort_tiles * 4);
+    take(&r.tot, (int64_t)n_seg * kBins * 4);
+    take(&r.part, (int64_t)n_seg * rank_tiles * 3 * 8);
+    take(&r.edge, (int64_t)n_seg * rank_tiles * 8);
+    r.bytes = std::max(o, end);
     return r;
 }
 
-size_t rank_scratch_bytes(int n_seg, int64_t n) {
-    return carve_rank(nullptr, n_seg, n).bytes;
+// the radix path's sort, tie groups and rank sums for the segments sg
+cudaError_t radix_ranks(const float *v, int64_t n, const RankScratch &r, const uint32_t *payload,
+                        int mode, uint32_t *r2, const uint32_t *r2y, const float *w, double *part,
+                        uint32_t *nan_flag, const Segs &sg, int rows_of_blocks, cudaStream_t st) {
+    const int64_t n_tiles = (n + kTile - 1) / kTile;
+    cudaError_t e = radix_sort_values(v, r.keys, r.vals, r.keys2, r.vals2, n, r.hist, r.tot, nan_flag,
+                                      payload, sg, rows_of_blocks, st);
+    if (e != cudaSuccess) return e;
+    edges_kernel<<<dim3((unsigned)((n_tiles + 255) / 256), rows_of_blocks), 256, 0, st>>>(
+        r.keys, n, (int)n_tiles, r.edge, sg);
+    rank_kernel<<<dim3((unsigned)n_tiles, rows_of_blocks), kTileThreads, 0, st>>>(
+        r.keys, r.vals, n, (int)n_tiles, mode, r.edge, r2, r2y, w, part, payload ? 1 : 0, sg);
+    return cudaGetLastError();
 }
 
-size_t target_part_bytes(int64_t n) { return (size_t)((n + kTile - 1) / kTile) * 3 * 8; }
+size_t rank_scratch_bytes(int n_seg, int64_t n, bool weighted) {
+    Buckets B;
+    const float one = 1.0f;
+    // the target's own sort uses the same memory
+    return std::max(carve_rank(nullptr, n_seg, n, bucket_path(weighted ? &one : nullptr, n), &B).bytes,
+                    carve_rank(nullptr, 1, n, false, &B).bytes);
+}
+
+// tile sums, then their totals
+size_t target_part_bytes(int64_t n) { return ((size_t)((n + kTile - 1) / kTile) + 1) * 3 * 8; }
 
 cudaError_t target_ranks(const float *y, const float *w, int64_t n, void *scratch, uint32_t *r2y,
                          double *tpart, cudaStream_t st) {
     const int64_t n_tiles = (n + kTile - 1) / kTile;
-    const RankScratch r = carve_rank(scratch, 1, n);
+    Buckets B;
+    const RankScratch r = carve_rank(scratch, 1, n, false, &B);
     cudaError_t e = cudaMemsetAsync(r.nan_flag, 0, 4, st);
     if (e != cudaSuccess) return e;
-    e = radix_sort_values(y, r.keys, r.vals, r.keys2, r.vals2, 1, n, r.hist, r.tot, r.nan_flag,
-                          nullptr, st);
+    e = radix_ranks(y, n, r, nullptr, 0, r2y, nullptr, w, tpart, r.nan_flag, Segs{nullptr, nullptr, 1}, 1, st);
     if (e != cudaSuccess) return e;
-    edges_kernel<<<(unsigned)((n_tiles + 255) / 256), 256, 0, st>>>(r.keys, n, (int)n_tiles, 1, r.edge);
-    rank_kernel<<<dim3((unsigned)n_tiles, 1), kTileThreads, 0, st>>>(
-        r.keys, r.vals, n, (int)n_tiles, 0, r.edge, r2y, nullptr, w, tpart, 0);
+    target_total_kernel<<<1, 32, 0, st>>>(tpart, (int)n_tiles, tpart + 3 * n_tiles);
     return cudaGetLastError();
 }
 
@@ -604,21 +1169,27 @@ cudaError_t spearman_batch(const float *pred, int n_seg, int64_t n, const uint32
                            const double *tpart, const float *w, void *scratch, float *out,
                            double *out64, cudaStream_t st) {
     const int64_t n_tiles = (n + kTile - 1) / kTile;
-    const RankScratch r = carve_rank(scratch, n_seg, n);
-    cudaError_t e = cudaMemsetAsync(r.nan_flag, 0, (size_t)n_seg * 4, st);
-    if (e != cudaSuccess) return e;
+    const bool buckets = bucket_path(w, n);
+    Buckets B{};
+    const RankScratch r = carve_rank(scratch, n_seg, n, buckets, &B);
+    cudaError_t e = cudaSuccess;
+    if (buckets) {
+        if ((e = bucket_ranks(pred, n_seg, n, r2y, B, r.nan_flag, st)) != cudaSuccess) return e;
+    } else {
+        if ((e = cudaMemsetAsync(r.nan_flag, 0, (size_t)n_seg * 4, st)) != cudaSuccess) return e;
+    }
     // unweighted rows need only the target's rank of each row: the sort
     // carries it as the payload, so the rank pass reads it in sorted order
     // instead of gathering it by row
-    const bool carry_ranks = w == nullptr;
-    e = radix_sort_values(pred, r.keys, r.vals, r.keys2, r.vals2, n_seg, n, r.hist, r.tot,
-                          r.nan_flag, carry_ranks ? r2y : nullptr, st);
-    if (e != cudaSuccess) return e;
-    edges_kernel<<<(unsigned)((n_tiles * n_seg + 255) / 256), 256, 0, st>>>(r.keys, n, (int)n_tiles,
-                                                                           n_seg, r.edge);
-    rank_kernel<<<dim3((unsigned)n_tiles, n_seg), kTileThreads, 0, st>>>(
-        r.keys, r.vals, n, (int)n_tiles, 1, r.edge, nullptr, r2y, w, r.part, carry_ranks ? 1 : 0);
-    spearman_final_kernel<<<(n_seg + 7) / 8, 256, 0, st>>>(r.part, tpart, n_seg, (int)n_tiles,
+    const uint32_t *payload = w == nullptr ? r2y : nullptr;
+    if (!buckets || B.nb > 1) {
+        const Segs sg = buckets ? Segs{B.list, B.count, 0} : Segs{nullptr, nullptr, n_seg};
+        e = radix_ranks(pred, n, r, payload, 1, nullptr, r2y, w, r.part, r.nan_flag, sg,
+                        buckets ? std::min(n_seg, 4) : n_seg, st);
+        if (e != cudaSuccess) return e;
+    }
+    spearman_final_kernel<<<(n_seg + 7) / 8, 256, 0, st>>>(r.part, buckets ? B.sums : nullptr, B.listed,
+                                                           tpart + 3 * n_tiles, n_seg, (int)n_tiles,
                                                            r.nan_flag, out, out64);
     return cudaGetLastError();
 }
