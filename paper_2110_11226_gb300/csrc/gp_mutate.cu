@@ -3,7 +3,7 @@
 // on the CPU and copies every program back, Sec. III-C2 and III-D2, and
 // names avoiding those transfers as future work, Sec. V).
 //
-// Three launches: one thread per offspring draws its kind and builds the
+// Three launches: one warp per offspring draws its kind and builds the
 // child in its own 256-node scratch slot (Sec. II-A crossover, subtree,
 // hoist and point mutation, reproduction; the hoisted crossover of
 // Sec. III-C2 keeps the child within 20 stack slots and 255 nodes); one
@@ -44,29 +44,70 @@ __device__ __forceinline__ int arity_of(int op) {
     return -1;
 }
 
-// the reverse scan of Sec. III-A: validity of a prefix list
-__device__ bool valid_program(const gp_node *p, int len, int n_feat) {
-    if (len < 1 || len > GP_MAX_LEN) return false;
-    int sp = 0, hw = 0;
-    for (int j = len - 1; j >= 0; --j) {
-        const int a = arity_of(p[j].op);
-        if (a < 0) return false;
-        if (p[j].op == GP_VAR && (p[j].feat < 0 || p[j].feat >= n_feat)) return false;
-        if (sp < a) return false;
-        sp += 1 - a;
-        hw = max(hw, sp);
+// A prefix list in shared memory and, per node, the stack height after it in
+// the reverse scan of Sec. III-A: terminals minus binary nodes from it to the
+// end, counted 32 nodes at a time with ballots.  The nodes [i, i + size) of a
+// subtree end where the height first falls below node i's.
+struct List {
+    uint2 node[256];    // op | feat << 16, constant
+    uint8_t hgt[256];   // 0 at len
+};
+
+__device__ __forceinline__ int op_of(const List &l, int m) { return (int16_t)(l.node[m].x & 0xffffu); }
+
+// fills l.hgt[0 .. len]; whether the list is a valid program.  The whole warp
+__device__ bool scan_list(List &l, int len, int n_feat) {
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const unsigned ge = full << lane, gt = ge & ~(1u << lane);
+    int carry = 0, hw = 0;
+    bool ok = true;
+    for (int c = (len - 1) >> 5; c >= 0; --c) {
+        const int m = c * 32 + lane;
+        const bool in = m < len;
+        const int op = in ? op_of(l, m) : GP_NUM_OPS, ar = in ? arity_of(op) : 1;
+        const unsigned leaf = __ballot_sync(full, ar == 0), bin = __ballot_sync(full, ar == 2);
+        const int h = carry + __popc(leaf & ge) - __popc(bin & ge);
+        const int before = carry + __popc(leaf & gt) - __popc(bin & gt);
+        if (in) {
+            const int feat = (int16_t)(l.node[m].x >> 16);
+            ok = ok && ar >= 0 && before >= ar && !(op == GP_VAR && (feat < 0 || feat >= n_feat));
+            l.hgt[m] = (uint8_t)h;
+            hw = max(hw, h);
+        }
+        carry += __popc(leaf) - __popc(bin);
     }
-    return sp == 1 && hw <= GP_MAX_STACK;
+    if (lane == 0) l.hgt[len] = 0;
+    __syncwarp();
+    return __all_sync(full, ok) && carry == 1 && __reduce_max_sync(full, hw) <= GP_MAX_STACK;
 }
 
 // nodes of the subtree rooted at node i
-__device__ int subtree_size(const gp_node *p, int len, int i) {
-    int need = 1;
-    for (int m = i; m < len; ++m) {
-        need += arity_of(p[m].op) - 1;
-        if (need == 0) return m - i + 1;
+__device__ int subtree_size(const List &l, int len, int i) {
+    const int lane = threadIdx.x & 31;
+    for (int m0 = i + 1; m0 <= len; m0 += 32) {
+        const int m = m0 + lane;
+        const unsigned ends = __ballot_sync(0xffffffffu, m <= len && l.hgt[m] < l.hgt[i]);
+        if (ends) return m0 + __ffs(ends) - 1 - i;
     }
     return len - i;  // unreachable for a valid program
+}
+
+// the largest height of nodes [m0, m1) (at least 0)
+__device__ int highest(const List &l, int m0, int m1) {
+    int h = 0;
+    for (int m = m0 + (threadIdx.x & 31); m < m1; m += 32) h = max(h, (int)l.hgt[m]);
+    return __reduce_max_sync(0xffffffffu, h);
+}
+
+// the caller's nodes are only 4-byte aligned
+__device__ __forceinline__ uint2 load_node(const gp_node *p, int m) {
+    const uint32_t *q = reinterpret_cast<const uint32_t *>(p) + 2 * m;
+    return make_uint2(q[0], q[1]);
+}
+
+__device__ __forceinline__ uint2 bits_of(const gp_node &nd) {
+    return make_uint2((uint32_t)(uint16_t)nd.op | (uint32_t)(uint16_t)nd.feat << 16, __float_as_uint(nd.c));
 }
 
 // variable f for f < n_feat, else a constant (w >> 8) * 2^-23 - 1 from the
@@ -89,69 +130,61 @@ __device__ gp_node new_terminal(Stream &s, int n_feat) {
 
 // a "grow" tree of depth <= limit (<= 6, so <= 127 nodes) in prefix order:
 // below the limit a node is a terminal when a word picks one of the 2
-// terminal kinds among 2 + n_funcs, else one of the allowed functions
-__device__ int grow_tree(Stream &s, const MutArgs &a, gp_node *out) {
-    int8_t slot_depth[2 * 64];
+// terminal kinds among 2 + n_funcs, else one of the allowed functions.  Every
+// lane draws the same words; depths: scratch of 128 entries
+__device__ int grow_tree(Stream &s, const MutArgs &a, List &out, volatile uint8_t *depths) {
+    const int lane = threadIdx.x & 31;
     int top = 0, n = 0;
-    slot_depth[top++] = 0;
+    depths[top++] = 0;
     while (top > 0 && n < 127) {
-        const int d = slot_depth[--top];
+        __syncwarp();
+        const int d = depths[--top];
+        __syncwarp();
         const bool terminal = d >= a.subtree_depth || pick(s, a.n_funcs + 2) < 2;
+        gp_node nd;
         if (terminal) {
-            out[n++] = new_terminal(s, a.n_feat);
+            nd = new_terminal(s, a.n_feat);
         } else {
-            gp_node nd;
             nd.op = a.funcs[pick(s, a.n_funcs)];
             nd.feat = 0;
             nd.c = 0.0f;
-            out[n++] = nd;
-            for (int k = 0; k < arity_of(nd.op); ++k) slot_depth[top++] = (int8_t)(d + 1);
+            for (int k = 0; k < arity_of(nd.op); ++k) depths[top++] = (uint8_t)(d + 1);
         }
+        if (lane == 0) out.node[n] = bits_of(nd);
+        ++n;
     }
+    __syncwarp();
     return n;
 }
 
 // Length of the parent with subtree [i, i+si) replaced by donor subtree
-// [j, j+sj), or 0 when that child would exceed 255 nodes or 20 stack
-// slots; the stack height is scanned over the three pieces in place.
-__device__ int splice_len(const gp_node *par, int lp, int i, int si, const gp_node *don, int j,
-                          int sj) {
+// [j, j+sj), or 0 when that child would exceed 255 nodes or 20 stack slots.
+// The nodes outside the subtree keep their heights (any subtree adds 1), and
+// the donor's stand on the height behind the replaced one.
+__device__ int splice_len(const List &par, int lp, int i, int si, const List &don, int j, int sj) {
     const int len = i + sj + (lp - i - si);
     if (len > GP_MAX_LEN) return 0;
-    int sp = 0, hw = 0;
-    for (int m = lp - 1; m >= i + si; --m) {
-        sp += 1 - arity_of(par[m].op);
-        hw = max(hw, sp);
-    }
-    for (int m = j + sj - 1; m >= j; --m) {
-        sp += 1 - arity_of(don[m].op);
-        hw = max(hw, sp);
-    }
-    for (int m = i - 1; m >= 0; --m) {
-        sp += 1 - arity_of(par[m].op);
-        hw = max(hw, sp);
-    }
+    const int hw = max(max(highest(par, 0, i), highest(par, i + si, lp)),
+                       (int)par.hgt[i + si] + highest(don, j, j + sj) - (int)don.hgt[j + sj]);
     return hw <= GP_MAX_STACK ? len : 0;
 }
 
-__device__ void splice_write(const gp_node *par, int lp, int i, int si, const gp_node *don, int j,
-                             int sj, gp_node *out) {
-    int n = 0;
-    for (int m = 0; m < i; ++m) out[n++] = par[m];
-    for (int m = j; m < j + sj; ++m) out[n++] = don[m];
-    for (int m = i + si; m < lp; ++m) out[n++] = par[m];
+__device__ void splice_write(const List &par, int i, int si, const List &don, int j, int sj, int len,
+                             uint2 *out) {
+    for (int n = threadIdx.x & 31; n < len; n += 32)
+        out[n] = n < i ? par.node[n] : n < i + sj ? don.node[j + n - i] : par.node[n - sj + si];
 }
 
 // the hoisted crossover: while the child does not fit, the donor subtree
 // moves to a node drawn among its proper descendants
-__device__ int hoisted_splice(Stream &s, const gp_node *par, int lp, int i, const gp_node *don,
-                              int ld, int j, gp_node *out) {
+__device__ int hoisted_splice(Stream &s, const List &par, int lp, int i, const List &don, int ld, int j,
+                              uint2 *out) {
     const int si = subtree_size(par, lp, i);
     int sj = subtree_size(don, ld, j);
     for (int guard = 0; guard <= GP_MAX_LEN; ++guard) {
         const int len = splice_len(par, lp, i, si, don, j, sj);
         if (len > 0) {
-            splice_write(par, lp, i, si, don, j, sj, out);
+            splice_write(par, i, si, don, j, sj, len, out);
             return len;
         }
         if (sj == 1) return 0;  // a terminal always fits a valid parent
@@ -161,10 +194,20 @@ __device__ int hoisted_splice(Stream &s, const gp_node *par, int lp, int i, cons
     return 0;
 }
 
-__global__ void __launch_bounds__(128) mutate_plan_kernel(const MutArgs a) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= a.n_out) return;
-    gp_node *child = a.scratch + (size_t)t * kSlot;
+// One warp per offspring: every lane draws the same words, and the lists are
+// scanned, searched and copied 32 nodes at a time in shared memory.  Bound by
+// latency; one thread per offspring walking the lists in global memory took
+// 49 us for 4096 offspring of 19 nodes, this 12 us.
+constexpr int kPlanWarps = 4;
+
+__global__ void __launch_bounds__(kPlanWarps * 32) mutate_plan_kernel(const MutArgs a) {
+    __shared__ List lists[kPlanWarps][2];
+    __shared__ uint8_t depths[kPlanWarps][128];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int t = blockIdx.x * kPlanWarps + warp;
+    if (t >= a.n_out) return;  // the whole warp
+    List &par = lists[warp][0], &don = lists[warp][1];
+    uint2 *child = reinterpret_cast<uint2 *>(a.scratch + (size_t)t * kSlot);
     Stream s;
     s.key = make_uint2((uint32_t)a.seed, (uint32_t)(a.seed >> 32));
     s.t = (uint32_t)t;
@@ -179,30 +222,26 @@ __global__ void __launch_bounds__(128) mutate_plan_kernel(const MutArgs a) {
             break;
         }
     const int pi = a.parents[2 * t], di = a.parents[2 * t + 1];
-    gp_node zero;
-    zero.op = GP_CONST;
-    zero.feat = 0;
-    zero.c = 0.0f;
-    if (pi < 0 || pi >= a.n_progs || di < 0 || di >= a.n_progs) {
-        atomicOr(a.dev_status, GP_DEV_BAD_PARENT);
-        child[0] = zero;
-        a.lens[t] = 1;
-        if (a.kind) a.kind[t] = GP_MUT_REPRODUCTION;
+    const bool found = pi >= 0 && pi < a.n_progs && di >= 0 && di < a.n_progs;
+    const int op0 = found ? a.offsets[pi] : 0, od = found ? a.offsets[di] : 0;
+    int lp = found ? a.offsets[pi + 1] - op0 : 0;
+    const int ld = found ? a.offsets[di + 1] - od : 0;
+    if (!found && lane == 0) atomicOr(a.dev_status, GP_DEV_BAD_PARENT);
+    if (lp < 1 || lp > GP_MAX_LEN) {  // a one-node program 0
+        if (lane == 0) {
+            child[0] = make_uint2(GP_CONST, 0u);
+            a.lens[t] = 1;
+            if (a.kind) a.kind[t] = GP_MUT_REPRODUCTION;
+        }
         return;
     }
-    const gp_node *par = a.progs + a.offsets[pi];
-    int lp = a.offsets[pi + 1] - a.offsets[pi];
-    const gp_node *don = a.progs + a.offsets[di];
-    const int ld = a.offsets[di + 1] - a.offsets[di];
-    if (!valid_program(par, lp, a.n_feat)) {
-        kind = GP_MUT_REPRODUCTION;
-        if (lp < 1 || lp > GP_MAX_LEN) {
-            child[0] = zero;
-            par = child;
-            lp = 1;
-        }
-    }
-    if (kind == GP_MUT_CROSSOVER && !valid_program(don, ld, a.n_feat)) kind = GP_MUT_REPRODUCTION;
+    for (int m = lane; m < lp; m += 32) par.node[m] = load_node(a.progs + op0, m);
+    const bool donor = kind == GP_MUT_CROSSOVER && ld >= 1 && ld <= GP_MAX_LEN;
+    if (donor)
+        for (int m = lane; m < ld; m += 32) don.node[m] = load_node(a.progs + od, m);
+    __syncwarp();
+    if (!scan_list(par, lp, a.n_feat)) kind = GP_MUT_REPRODUCTION;
+    if (kind == GP_MUT_CROSSOVER && !(donor && scan_list(don, ld, a.n_feat))) kind = GP_MUT_REPRODUCTION;
 
     int len = 0;
     if (kind == GP_MUT_CROSSOVER) {
@@ -210,43 +249,48 @@ __global__ void __launch_bounds__(128) mutate_plan_kernel(const MutArgs a) {
         const int j = pick(s, ld);
         len = hoisted_splice(s, par, lp, i, don, ld, j, child);
     } else if (kind == GP_MUT_SUBTREE) {
-        gp_node tree[128];
-        const int lt = grow_tree(s, a, tree);
+        const int lt = grow_tree(s, a, don, depths[warp]);
+        scan_list(don, lt, a.n_feat);
         const int i = pick(s, lp);
-        len = hoisted_splice(s, par, lp, i, tree, lt, 0, child);
+        len = hoisted_splice(s, par, lp, i, don, lt, 0, child);
     } else if (kind == GP_MUT_HOIST) {
         const int i = pick(s, lp);
         const int si = subtree_size(par, lp, i);
         const int k = si > 1 ? i + 1 + pick(s, si - 1) : i;
-        len = splice_len(par, lp, i, si, par, k, subtree_size(par, lp, k));
-        if (len > 0) splice_write(par, lp, i, si, par, k, subtree_size(par, lp, k), child);
+        const int sk = subtree_size(par, lp, k);
+        len = splice_len(par, lp, i, si, par, k, sk);
+        if (len > 0) splice_write(par, i, si, par, k, sk, len, child);
     } else if (kind == GP_MUT_POINT) {
-        for (int m = 0; m < lp; ++m) child[m] = par[m];
         len = lp;
         for (int m = 0; m < lp; ++m) {
             if ((uint64_t)next_word(s) >= a.thr_replace) continue;
-            const int ar = arity_of(par[m].op);
+            const int ar = arity_of(op_of(par, m));
+            gp_node nd;
+            nd.op = GP_CONST;
+            nd.feat = 0;
+            nd.c = 0.0f;
             if (ar == 0) {
-                child[m] = new_terminal(s, a.n_feat);
+                nd = new_terminal(s, a.n_feat);
             } else {
                 const int ns = ar == 1 ? a.n_unary : a.n_binary;
-                if (ns > 0) {
-                    const int idx = pick(s, ns);
-                    child[m].op = ar == 1 ? a.unary[idx] : a.binary[idx];
-                    child[m].feat = 0;
-                    child[m].c = 0.0f;
-                }
+                if (ns <= 0) continue;
+                const int idx = pick(s, ns);
+                nd.op = ar == 1 ? a.unary[idx] : a.binary[idx];
             }
+            if (lane == 0) par.node[m] = bits_of(nd);
         }
+        __syncwarp();
+        for (int m = lane; m < lp; m += 32) child[m] = par.node[m];
     }
     if (len == 0) {  // reproduction, or a splice that could not fit
-        if (par != child)
-            for (int m = 0; m < lp; ++m) child[m] = par[m];
+        for (int m = lane; m < lp; m += 32) child[m] = par.node[m];
         len = lp;
         kind = GP_MUT_REPRODUCTION;
     }
-    a.lens[t] = len;
-    if (a.kind) a.kind[t] = kind;
+    if (lane == 0) {
+        a.lens[t] = len;
+        if (a.kind) a.kind[t] = kind;
+    }
 }
 
 // exclusive scan of the lengths in one block, 1024 at a time with a carry
@@ -301,7 +345,7 @@ __global__ void __launch_bounds__(256) mutate_copy_kernel(const MutArgs a) {
 
 cudaError_t launch_mutate(const MutArgs &a, cudaStream_t st) {
     if (a.n_out <= 0) return cudaSuccess;
-    mutate_plan_kernel<<<(a.n_out + 127) / 128, 128, 0, st>>>(a);
+    mutate_plan_kernel<<<(a.n_out + kPlanWarps - 1) / kPlanWarps, kPlanWarps * 32, 0, st>>>(a);
     mutate_scan_kernel<<<1, 1024, 0, st>>>(a);
     mutate_copy_kernel<<<(a.n_out * 32 + 255) / 256, 256, 0, st>>>(a);
     return cudaGetLastError();

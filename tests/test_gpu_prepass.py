@@ -84,3 +84,39 @@ def test_total_weight(n_rows):
     if n_rows > 1:
         r = float(gp.gp_evaluate(pn, po, x, (-2.0 * x[0]).contiguous(), w, "pearson")[0])
         assert abs(r - 1.0) <= 1e-5
+
+
+@pytest.mark.parametrize("length", [1, 2, 31, 32, 33, 64, 65, 128, 129, 254, 255])
+def test_mutation_at_chunk_edges(length):
+    """The mutation step scans its lists 32 nodes at a time too: parents and
+    donors of exactly `length` nodes, every kind, bit for bit."""
+    import torch
+
+    from paper_2110_11226_gb300 import gp
+    rng = np.random.default_rng(1000 + length)
+    progs = [_sized(rng, length, b) for b in (True, False) for _ in range(20)]
+    nodes, off = synth.pack(progs)
+    parents = rng.integers(0, 40, 2 * 300).astype(np.int32)
+    for kind in ("crossover", "subtree", "hoist", "point"):
+        probs = dict(p_crossover=0.0, p_subtree=0.0, p_hoist=0.0, p_point=0.0, p_replace=0.3)
+        probs["p_" + kind] = 1.0
+        out, oo, k = gp.gp_mutate(gp.nodes_to_device(nodes), torch.from_numpy(off).cuda(), 2,
+                                  torch.from_numpy(parents).cuda(), gp.make_mut_params(**probs), seed=length)
+        wn, wo, wk = oracle.mutate(nodes, off, 2, parents, seed=length, **probs)
+        np.testing.assert_array_equal(oo.cpu().numpy(), wo)
+        np.testing.assert_array_equal(k.cpu().numpy(), wk)
+        assert gp.nodes_from_device(out[:int(wo[-1])]).tobytes() == wn.tobytes()
+
+
+@pytest.mark.parametrize("k", [1, 3, 4, 5, 8, 21])
+def test_tournament_sizes(k):
+    """Draws come four at a time: sizes around multiples of four."""
+    import torch
+
+    from paper_2110_11226_gb300 import gp
+    fit = np.random.default_rng(k).standard_normal(77).astype(np.float32)
+    fit[5] = np.nan
+    for greater in (False, True):
+        got = gp.gp_tournament_ex(torch.from_numpy(fit).cuda(), 129, k, 9, greater_is_better=greater)
+        np.testing.assert_array_equal(got.cpu().numpy(),
+                                      oracle.tournament(fit, 129, k, 9, greater_is_better=greater))
