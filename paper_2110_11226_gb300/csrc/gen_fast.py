@@ -23,6 +23,12 @@ so the division forms share one body (the divisor staged in U;
 the reversed forms swap the rows into U first), sin and cos share one,
 and tan goes to the C++ switch.
 
+The evaluator's words are laid out for it by the block that copies them to
+shared memory: one index that the branch takes as it is (an `and` less) and a
+stack pointer instead of slot numbers (two instructions less per push and
+pop).  The gradient variant reads the pre-pass's words, whose other bits hold
+slots and marker shapes.
+
 Variants: RPT in {4, 8} x DIVS (the division set, square root, reciprocal,
 sin, cos, log and exp run here; without DIVS they are handed back) x
 XREG (columns 0 and 1 held in registers; without it a column read takes
@@ -83,7 +89,11 @@ class Gen:
         names = ["pa"] + [f"T{i}" for i in range(p)]
         if self.xmem:
             names += [f"XB{i}" for i in range(p)]
-        names += ["HW", "HC", "SB", "NSM1"]
+        # the evaluator's words are the dispatch index and a constant, and the
+        # stack has a pointer; the gradient's carry slots and markers
+        self.plain = not grad
+        names += ["SP", "HW", "HC"] if self.plain else ["HW", "HC", "SB", "NSM1"]
+        self.I = "%%w" if self.plain else "%%i"   # the dispatch index
         if self.xmem:
             names += ["XC", "UNIT", "MODE"]
         else:
@@ -92,7 +102,11 @@ class Gen:
         names += ["THR", "DB", "KT"]
         at = {n: f"%{k}" for k, n in enumerate(names)}
         self.T = [at[f"T{i}"] for i in range(p)]
-        self.HW, self.HC, self.SB, self.NSM1 = at["HW"], at["HC"], at["SB"], at["NSM1"]
+        self.HW, self.HC = at["HW"], at["HC"]
+        if self.plain:
+            self.SP = at["SP"]
+        else:
+            self.SB, self.NSM1 = at["SB"], at["NSM1"]
         self.THR, self.DB, self.KT = at["THR"], at["DB"], at["KT"]
         if self.xmem:
             xb = [at[f"XB{i}"] for i in range(p)]
@@ -131,12 +145,24 @@ class Gen:
         self.e(f"mad.lo.u32 %%a, %%a, {self.slot_bytes}, {self.SB};")
 
     def slot_load(self):
+        if self.plain:
+            self.e(f"sub.u32 {self.SP}, {self.SP}, {self.slot_bytes};")
+            for q in range(self.rpt // 4):
+                off = f"+{512 * q}" if q else ""
+                self.e(f"ld.shared.v2.b64 {{%%U{2 * q}, %%U{2 * q + 1}}}, [{self.SP}{off}];")
+            return
         self.slot_addr()
         for q in range(self.rpt // 4):
             off = f"+{512 * q}" if q else ""
             self.e(f"ld.shared.v2.b64 {{%%U{2 * q}, %%U{2 * q + 1}}}, [%%a{off}];")
 
     def spill(self):
+        if self.plain:
+            for q in range(self.rpt // 4):
+                off = f"+{512 * q}" if q else ""
+                self.e(f"st.shared.v2.b64 [{self.SP}{off}], {{{self.T[2 * q]}, {self.T[2 * q + 1]}}};")
+            self.e(f"add.u32 {self.SP}, {self.SP}, {self.slot_bytes};")
+            return
         self.slot_addr()
         for q in range(self.rpt // 4):
             off = f"+{512 * q}" if q else ""
@@ -237,7 +263,7 @@ class Gen:
         if kind is None:
             self.range_check("trig_fast", special=lambda: self.rows_test(
                 lambda i: self.T[i], lambda v: self.beyond("trig_fast", v)))
-            self.e(f"sub.u32 %%kd, %%i, {OPS['SIN']};")
+            self.e(f"sub.u32 %%kd, {self.I}, {OPS['SIN']};")
             self.e("setp.ne.u32 %%p, %%kd, 0;")
             self.e("selp.b64 %%KM, 0xBF000000BF000000, 0x8000000080000000, %%p;")  # -kind/2
             self.e("selp.b64 %%F, 0x3F0000003F000000, 0x0000000000000000, %%p;")   # +kind/2
@@ -991,8 +1017,9 @@ class Gen:
         e("ld.shared.v2.b32 {%%w, %%cb}, [%0];")
         e("mov.b32 %%cf, %%cb;")
         e("add.u32 %0, %0, 8;")
-        e("and.b32 %%i, %%w, 63;")
-        e("brx.idx.uni %%i, T%=;")
+        if not self.plain:
+            e("and.b32 %%i, %%w, 63;")
+        e(f"brx.idx.uni {self.I}, T%=;")
         X = self.X
         for name in used:
             self.label(name)
@@ -1072,16 +1099,16 @@ def function(rpt, divs, xreg, grad=False):
     xmem = g.xmem
     outs = ", ".join(['"+r"(pa)'] + [f'"+l"(t[{i}])' for i in range(p)]
                      + ([f'"+l"(xb[{i}])' for i in range(p)] if xmem else [])
-                     + ['"=r"(hw)', '"=f"(hc)'])
-    ins = ", ".join(['"r"(sb)', '"n"(NSLOT - 1)']
+                     + ([] if grad else ['"+r"(sp)']) + ['"=r"(hw)', '"=f"(hc)'])
+    ins = ", ".join((['"r"(sb)', '"n"(NSLOT - 1)'] if grad else [])
                     + (['"l"(xc)', '"r"(unit)', '"r"(mode)'] if xmem else
                        [f'"l"(x0[{i}])' for i in range(p)] + [f'"l"(x1[{i}])' for i in range(p)])
                     + ['"f"(kThr)'] + (['"r"(db)', '"n"(KT)'] if grad else []))
     args = (f"uint64_t (&xb)[{p}], const float *xc, uint32_t unit,\n        uint32_t mode"
             if xmem else f"const uint64_t (&x0)[{p}], const uint64_t (&x1)[{p}]")
-    return (f"template <int NSLOT{', int KT' if grad else ''}>\n"
+    return (("template <int NSLOT, int KT>\n" if grad else "") +
             f"__device__ __forceinline__ void {name}(uint32_t &pa, uint64_t (&t)[{p}],\n"
-            f"        {args}, uint32_t sb,\n"
+            f"        {args}, {'uint32_t sb' if grad else 'uint32_t &sp'},\n"
             f"        {'uint32_t db, ' if grad else ''}uint32_t &hw, float &hc) {{\n"
             f"    asm volatile(\n{body}\n"
             f"        : {outs}\n"
@@ -1091,13 +1118,13 @@ def function(rpt, divs, xreg, grad=False):
 HEADER = '''// gp_fast.cuh -- the evaluator's indexed-branch fast loop in inline PTX.
 // GENERATED by gen_fast.py (same directory); edit that script, not this file.
 //
-// fast_r<RPT>_<divs|nodivs>_<x|nox><NSLOT>(pa, t, x0, x1, sb, hw, hc) runs
-// compiled instruction words from the shared-memory address pa over RPT
-// rows per lane, held as RPT/2 pairs {row 2i, row 2i+1} in t.  It stops at
-// the first word it does not run, returns that word and its constant in
-// hw and hc, leaves pa just past it and the rows untouched by it.  sb is
-// the lane's slot-0 address in the shared-memory stack ([slot][q][lane]
-// float4); slots are clamped to NSLOT - 1.  The _x variants take columns 0
+// fast_r<RPT>_<divs|nodivs>_<x|nox>(pa, t, ..., sp, hw, hc) runs compiled
+// words -- the dispatch index and a constant -- from the shared-memory address
+// pa over RPT rows per lane, held as RPT/2 pairs {row 2i, row 2i+1} in t.  It
+// stops at the first word it does not run, returns that word and its constant
+// in hw and hc, leaves pa just past it and the rows untouched by it.  sp is the
+// lane's next free slot of the shared-memory stack ([slot][q][lane] float4); a
+// division handed back by the divs variants has taken its operand off.  The _x variants take columns 0
 // and 1 of the lane's rows in x0 and x1; the _nox ones read columns from
 // memory: xb holds the rows of the column that the program reads next, xc
 // is column 0 at the lane's first row, a word's constant times unit the bytes

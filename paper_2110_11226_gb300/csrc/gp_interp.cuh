@@ -35,12 +35,13 @@
 // partials of a program in chunk order in FP64.  Every step has a fixed
 // order, so results do not depend on which block ran which item.
 //
-// What surrounds the words -- loads, loss, loop -- costs 139 instructions per
-// program and sub-tile at 8 rows per lane, of some 900 (220 before the rows
-// were kept as pairs throughout, the ragged case put behind one test and the
-// next item taken by one thread: Pagie-1 16M x 4096 301 -> 281 ms; with 28
-// unaligned columns, where a lane's consecutive rows took eight 4-byte loads
-// of 32 sectors each, 22.2 -> 17.9 ms).
+// What surrounds the words -- loads, loss, loop -- costs 110 instructions per
+// program and sub-tile at 8 rows per lane, of some 850 (220 before the rows
+// were kept as pairs throughout, the ragged case put behind one vote, the next
+// item taken by one thread and squares added with FMA: Pagie-1 16M x 4096
+// 301 -> 260 ms with the shorter dispatch; with 28 unaligned columns, where a
+// lane's consecutive rows took eight 4-byte loads of 32 sectors each, 22.2 ->
+// 16.3 ms).
 #pragma once
 
 #include "gp_internal.cuh"
@@ -151,7 +152,7 @@ __device__ __forceinline__ void load_chunk_rows(float (&v)[RPT], const float *__
 // from p, 16-byte loads; else rows p[0], p[32], p[64], ..., the last of them
 // at most p[last] (a ragged sub-tile reads its last row again; those rows
 // do not count).
-template <int RPT>
+template <int RPT, int FMODE>
 __device__ __forceinline__ void load_pairs(uint64_t (&v)[RPT / 2], const float *__restrict__ p,
                                            bool packed, int last) {
     if (packed) {
@@ -162,19 +163,52 @@ __device__ __forceinline__ void load_pairs(uint64_t (&v)[RPT / 2], const float *
             v[2 * q + 1] = f.y;
         }
     } else {
+        // keeps the minima in this branch: hoisted above it they cost feature
+        // mode 0 registers and 8 instructions a sub-tile (4M x 50: 21.2 ->
+        // 19.7 ms); mode 2 is better off without (16M x 4096: 259 against 263)
+        if (FMODE == 0) asm volatile("" : "+r"(last));
 #pragma unroll
         for (int i = 0; i < RPT / 2; ++i)
             v[i] = pack2(__ldg(p + min(64 * i, last)), __ldg(p + min(64 * i + 32, last)));
     }
 }
 
-// the weighted losses of a lane's rows added in row order (the first nv
-// rows count); the metric and the weights are tested once, not per row
+__device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
+// the weighted losses of a lane's rows added up (the first nv rows count);
+// the metric and the weights are tested once, not per row.  The squares of
+// whole sub-tiles are added as they are formed, without a rounding of their
+// own, even and odd rows apart (9 instructions for 8 rows instead of 24)
 template <int RPT>
 __device__ __forceinline__ float loss_sum(int metric, const uint64_t (&tp)[RPT / 2],
                                           const uint64_t (&yp)[RPT / 2],
                                           const uint64_t (&wp)[RPT / 2], bool has_w, bool full,
                                           int nv) {
+    if (full && (metric == GP_MSE || metric == GP_RMSE)) {
+        uint64_t e2 = 0ull;
+#pragma unroll
+        for (int i = 0; i < RPT / 2; ++i) {
+            const uint64_t d = sub2(tp[i], yp[i]);
+            e2 = fma2(has_w ? mul2(wp[i], d) : d, d, e2);
+        }
+        float lo, hi;
+        unpack2(e2, lo, hi);
+        return __fadd_rn(lo, hi);
+    }
     float l[RPT], t[RPT], yv[RPT];
 #pragma unroll
     for (int i = 0; i < RPT / 2; ++i) {
@@ -252,21 +286,21 @@ static __device__ __noinline__ float4 ext_rows4(float4 v, uint32_t f) {
 // is off in the instances with the extended functions: there the division
 // set in the loop cost the extended-set population 23% (their out-of-line
 // calls and the division's own slow-path call do not mix well).
-template <int RPT, int NSLOT, bool DIVS, bool XREG>
+template <int RPT, bool DIVS, bool XREG>
 __device__ __forceinline__ void run_fast(uint32_t &pa, uint64_t (&t)[RPT / 2],
                                          uint64_t (&x0)[RPT / 2], const uint64_t (&x1)[RPT / 2],
-                                         const float *xc, uint32_t unit, uint32_t mode, uint32_t sb,
+                                         const float *xc, uint32_t unit, uint32_t mode, uint32_t &sp,
                                          uint32_t &hw, float &hc) {
     if constexpr (RPT == 4) {
-        if constexpr (DIVS && XREG) fast_r4_divs_x<NSLOT>(pa, t, x0, x1, sb, hw, hc);
-        else if constexpr (DIVS) fast_r4_divs_nox<NSLOT>(pa, t, x0, xc, unit, mode, sb, hw, hc);
-        else if constexpr (XREG) fast_r4_nodivs_x<NSLOT>(pa, t, x0, x1, sb, hw, hc);
-        else fast_r4_nodivs_nox<NSLOT>(pa, t, x0, x1, sb, hw, hc);
+        if constexpr (DIVS && XREG) fast_r4_divs_x(pa, t, x0, x1, sp, hw, hc);
+        else if constexpr (DIVS) fast_r4_divs_nox(pa, t, x0, xc, unit, mode, sp, hw, hc);
+        else if constexpr (XREG) fast_r4_nodivs_x(pa, t, x0, x1, sp, hw, hc);
+        else fast_r4_nodivs_nox(pa, t, x0, x1, sp, hw, hc);
     } else {
-        if constexpr (DIVS && XREG) fast_r8_divs_x<NSLOT>(pa, t, x0, x1, sb, hw, hc);
-        else if constexpr (DIVS) fast_r8_divs_nox<NSLOT>(pa, t, x0, xc, unit, mode, sb, hw, hc);
-        else if constexpr (XREG) fast_r8_nodivs_x<NSLOT>(pa, t, x0, x1, sb, hw, hc);
-        else fast_r8_nodivs_nox<NSLOT>(pa, t, x0, x1, sb, hw, hc);
+        if constexpr (DIVS && XREG) fast_r8_divs_x(pa, t, x0, x1, sp, hw, hc);
+        else if constexpr (DIVS) fast_r8_divs_nox(pa, t, x0, xc, unit, mode, sp, hw, hc);
+        else if constexpr (XREG) fast_r8_nodivs_x(pa, t, x0, x1, sp, hw, hc);
+        else fast_r8_nodivs_nox(pa, t, x0, x1, sp, hw, hc);
     }
 }
 
@@ -276,9 +310,10 @@ __device__ __forceinline__ void run_fast(uint32_t &pa, uint64_t (&t)[RPT / 2],
 // the lane's rows follow it (load_pairs).  x0p and x1p: columns 0 and 1
 // (FMODE 2), else the first column that the program reads in x0p (unit and
 // mode: how the loop reads the next ones, see gp_fast.cuh).
-// The instruction buffer holds the words that the pre-pass wrote, the last
-// of them OP_END; op values that name no operation act as OP_END and stack
-// slots are clamped to the stack.
+// The instruction buffer holds the pre-pass's words, the last of them OP_END,
+// as a dispatch index and a constant each, and their upper halves (the column
+// or the extended function, read by the switch alone) in aux.  Its pushes and
+// pops balance within the class's stack, so a pointer serves for the slots.
 //
 // Dispatch cost is what this loop is tuned for (per-opcode instruction
 // counts measured with ncu on chains of one operation).  At 4 and 8 rows
@@ -295,7 +330,8 @@ __device__ __forceinline__ void interpret(uint64_t (&tp)[RPT / 2], const uint2 *
                                           uint64_t (&x0p)[RPT / 2],
                                           const uint64_t (&x1p)[RPT / 2],
                                           const float *__restrict__ xc, int64_t ld, uint32_t unit,
-                                          uint32_t mode, bool packed, int last, float4 *stk) {
+                                          uint32_t mode, bool packed, int last, float4 *stk,
+                                          const uint16_t *aux) {
     // EXT: the extended functions are compiled in (classes 1 and 2).  In
     // class 0, where nearly all programs of the usual function set run,
     // their cases cost 2-3% (measured on Pagie-1 x 4096 programs, which
@@ -306,7 +342,8 @@ __device__ __forceinline__ void interpret(uint64_t (&tp)[RPT / 2], const uint2 *
     for (int i = 0; i < RPT / 2; ++i) asm volatile("" : "=l"(tp[i]));
     // pa: shared-memory address of the next instruction word
     uint32_t pa = (uint32_t)__cvta_generic_to_shared(cbuf);
-    const uint32_t sb = (uint32_t)__cvta_generic_to_shared(stk);  // this lane's slot 0
+    uint32_t sp = (uint32_t)__cvta_generic_to_shared(stk);  // this lane's next free slot
+    constexpr uint32_t kSlotBytes = RPT / 4 * 32u * 16u;
     // 4 or 8 rows per lane: the fast loop runs what it can and hands back
     // the rest, one word at a time, to the switch below
     constexpr bool kFast = RPT == 4 || RPT == 8;
@@ -315,7 +352,7 @@ __device__ __forceinline__ void interpret(uint64_t (&tp)[RPT / 2], const uint2 *
         uint2 ins;
         if constexpr (kFast) {
             float hc;
-            run_fast<RPT, NSLOT, !EXT, FMODE == 2>(pa, tp, x0p, x1p, xc, unit, mode, sb, ins.x, hc);
+            run_fast<RPT, !EXT, FMODE == 2>(pa, tp, x0p, x1p, xc, unit, mode, sp, ins.x, hc);
             ins.y = __float_as_uint(hc);
         } else {
             asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];"
@@ -330,37 +367,38 @@ __device__ __forceinline__ void interpret(uint64_t (&tp)[RPT / 2], const uint2 *
 #pragma unroll
         for (int i = 0; i < RPT / 2; ++i) unpack2(tp[i], t[2 * i], t[2 * i + 1]);
         const float c = __uint_as_float(ins.y);
+// the word's upper half
+#define GP_HI ((uint32_t)aux[(pa - (uint32_t)__cvta_generic_to_shared(cbuf)) / 8u - 1u])
 // operand helpers: stack slot, X column, constant
-// (the stack is laid out [slot][q][lane] in float4: slot sl, group q of
-// this lane sits (sl * RPT/4 + q) * 32 float4 past its slot 0)
+// (the stack is laid out [slot][q][lane] in float4)
 #define GP_SLOT_LOAD(u)                                                         \
     {                                                                           \
-        const uint32_t sl = min((w >> 8) & 255u, (uint32_t)NSLOT - 1u);         \
         _Pragma("unroll") for (int q = 0; q < RPT / 4; ++q) {                   \
             asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"             \
                          : "=f"(u[4 * q]), "=f"(u[4 * q + 1]),                  \
                            "=f"(u[4 * q + 2]), "=f"(u[4 * q + 3])               \
-                         : "r"(sb + (sl * (RPT / 4) + q) * 32u * 16u));          \
+                         : "r"(sp + q * 512u));                                 \
         }                                                                       \
     }
+#define GP_POP(u) { sp -= kSlotBytes; GP_SLOT_LOAD(u) }
 #define GP_SPILL()                                                              \
     {                                                                           \
-        const uint32_t sl = min((w >> 8) & 255u, (uint32_t)NSLOT - 1u);         \
         _Pragma("unroll") for (int q = 0; q < RPT / 4; ++q)                     \
             asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};"             \
-                         ::"r"(sb + (sl * (RPT / 4) + q) * 32u * 16u),           \
+                         ::"r"(sp + q * 512u),                                  \
                            "f"(t[4 * q]), "f"(t[4 * q + 1]), "f"(t[4 * q + 2]),  \
                            "f"(t[4 * q + 3])                                    \
                          : "memory");                                           \
+        sp += kSlotBytes;                                                       \
     }
 #define GP_X_LOAD(u)                                                            \
     {                                                                           \
-        const int feat = (int)(w >> 16);                                        \
+        const int feat = FMODE == 2 ? (int)(w >> 5) : (int)GP_HI;               \
         uint64_t up[RPT / 2];                                                   \
         if (FMODE == 2) {                                                       \
             _Pragma("unroll") for (int i = 0; i < RPT / 2; ++i) up[i] = feat ? x1p[i] : x0p[i]; \
         } else {                                                                \
-            load_pairs<RPT>(up, xc + (int64_t)feat * ld, packed, last);         \
+            load_pairs<RPT, FMODE>(up, xc + (int64_t)feat * ld, packed, last);         \
         }                                                                       \
         _Pragma("unroll") for (int i = 0; i < RPT / 2; ++i)                     \
             unpack2(up[i], u[2 * i], u[2 * i + 1]);                             \
@@ -373,10 +411,12 @@ __device__ __forceinline__ void interpret(uint64_t (&tp)[RPT / 2], const uint2 *
             case OP_PUSH_C: GP_T(c) break;
             case OP_PUSH_X_SP: GP_SPILL() GP_X_LOAD(u) GP_T(u[j]) break;
             case OP_PUSH_C_SP: GP_SPILL() GP_T(c) break;
-            case OP_ADD_S: GP_SLOT_LOAD(u) GP_T(f_add(t[j], u[j])) break;
-            case OP_SUB_S: GP_SLOT_LOAD(u) GP_T(f_sub(t[j], u[j])) break;
-            case OP_MUL_S: GP_SLOT_LOAD(u) GP_T(f_mul(t[j], u[j])) break;
-            case OP_DIV_S: GP_SLOT_LOAD(u) goto div_tu;
+            case OP_ADD_S: GP_POP(u) GP_T(f_add(t[j], u[j])) break;
+            case OP_SUB_S: GP_POP(u) GP_T(f_sub(t[j], u[j])) break;
+            case OP_MUL_S: GP_POP(u) GP_T(f_mul(t[j], u[j])) break;
+            case OP_DIV_S:  // (the loop has moved sp for a division that it hands back)
+                if (kFast && !EXT) GP_SLOT_LOAD(u) else GP_POP(u)
+                goto div_tu;
             case OP_ADD_X: GP_X_LOAD(u) GP_T(f_add(t[j], u[j])) break;
             case OP_ADD_C: GP_T(f_add(t[j], c)) break;
             case OP_SUB_X: GP_X_LOAD(u) GP_T(f_sub(t[j], u[j])) break;
@@ -400,10 +440,11 @@ __device__ __forceinline__ void interpret(uint64_t (&tp)[RPT / 2], const uint2 *
             case OP_INV: GP_T(f_inv(t[j])) break;
             case OP_EXT1:  // out of line, four rows per call
                 if constexpr (kExt) {
+                    const uint32_t fn = GP_HI;
                     _Pragma("unroll") for (int g = 0; g < RPT / 4; ++g) {
                         const float4 r = ext_rows4(
                             make_float4(t[4 * g], t[4 * g + 1], t[4 * g + 2], t[4 * g + 3]),
-                            (w >> 16) & 7u);
+                            fn);
                         t[4 * g] = r.x; t[4 * g + 1] = r.y; t[4 * g + 2] = r.z; t[4 * g + 3] = r.w;
                     }
                     break;
@@ -412,8 +453,8 @@ __device__ __forceinline__ void interpret(uint64_t (&tp)[RPT / 2], const uint2 *
                 }
             case OP_EXT2:  // max / min, right operand in a stack slot
                 if constexpr (kExt) {
-                    GP_SLOT_LOAD(u)
-                    if (((w >> 16) & 7u) == EXT_MAX) { GP_T(f_max(t[j], u[j])) }
+                    GP_POP(u)
+                    if (GP_HI == EXT_MAX) { GP_T(f_max(t[j], u[j])) }
                     else { GP_T(f_min(t[j], u[j])) }
                     break;
                 } else {
@@ -438,6 +479,8 @@ __device__ __forceinline__ void interpret(uint64_t (&tp)[RPT / 2], const uint2 *
 #undef GP_U_C
 #undef GP_X_LOAD
 #undef GP_SPILL
+#undef GP_HI
+#undef GP_POP
 #undef GP_SLOT_LOAD
     }
 done:;
@@ -477,6 +520,7 @@ __global__ void __launch_bounds__(eval_warps<RPT>() * 32,
     __shared__ int4 s_item[2];  // chunk (-1: the queue is empty), program, words, status
     __shared__ unsigned long long s_total;
     __shared__ int s_begin, s_n;
+    __shared__ uint16_t aux[kCodeStride + 2];
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     float4 *stk = stack_all + (size_t)warp * NSLOT * (RPT / 4) * 32 + lane;
@@ -529,10 +573,11 @@ __global__ void __launch_bounds__(eval_warps<RPT>() * 32,
             const uint2 *src = a.code + (size_t)p * (a.code_stride ? a.code_stride : kCodeStride);
             for (int i = threadIdx.x; i < it.z && i <= kCodeStride; i += kEvalBlock) {
                 uint2 v = src[i];
+                aux[i] = (uint16_t)(v.x >> 16);
                 // a column read's constant: the next column read, as an offset
                 if (FMODE == 0 && !EXT && (kColumnOps >> (v.x & 31u) & 1u))
                     v.y = (uint32_t)((uint64_t)v.y * (uint64_t)(a.x_unit == 16 ? a.ld >> 2 : a.ld));
-                cbuf[i] = v;
+                cbuf[i] = make_uint2(v.x & 63u, v.y);
             }
         }
         __syncthreads();  // the words are there
@@ -547,30 +592,42 @@ __global__ void __launch_bounds__(eval_warps<RPT>() * 32,
         // loss of this one
         uint64_t x0[RPT / 2], x1[RPT / 2];
         auto first_column = [&](int base) {
-            const bool pk = base + 32 * RPT <= n_in && a.vec_ok;
+            const bool pk = __all_sync(0xffffffffu, base + 32 * RPT <= n_in) && a.vec_ok;
             const int o = base + (pk ? lane * RPT : lane);
-            const int64_t feat = cbuf[s_item[cur].z - 1].y;
-            load_pairs<RPT>(x0, a.X + (feat * a.ld + rb + o), pk, n_in - 1 - o);
+            const volatile int4 *it = &s_item[cur];
+            const int64_t feat = cbuf[it->z - 1].y;
+            load_pairs<RPT, FMODE>(x0, a.X + (feat * a.ld + (int64_t)it->x * a.chunk_rows + o), pk,
+                            n_in - 1 - o);
         };
         constexpr bool kAhead = FMODE == 0 && !EXT;  // the loop reads columns ahead
         if (kAhead && ok && warp * 32 * RPT < n_in) first_column(warp * 32 * RPT);
         for (int base = warp * 32 * RPT; base < n_in && ok; base += kEvalWarps * 32 * RPT) {
             // whole: every row of the sub-tile is in the chunk; packed: and
-            // the lane's rows are consecutive.  One test for the warp
-            const bool whole = base + 32 * RPT <= n_in;
+            // the lane's rows are consecutive.  One test for the warp (a vote:
+            // the compiler then knows that the warp agrees, and needs no
+            // reconvergence around the loads and the loss)
+            const bool whole = __all_sync(0xffffffffu, base + 32 * RPT <= n_in);
             const bool packed = whole && a.vec_ok;
             const int o = base + (packed ? lane * RPT : lane);  // the lane's first row
             const int last = n_in - 1 - o;   // its furthest row (negative: none; see load_pairs)
-            const int nv = whole ? RPT : (last + 32) >> 5;  // rows of the lane that count
-            const int64_t r = rb + o;
-            if (FMODE == 2) {
-                load_pairs<RPT>(x0, a.X + r, packed, last);
-                load_pairs<RPT>(x1, a.X + (a.ld + r), packed, last);
-            }
             uint64_t t[RPT / 2];
-            const uint32_t mode = a.x_unit == 0 || !whole ? 2u : packed ? 0u : 1u;
-            interpret<RPT, NSLOT, FMODE, EXT>(t, cbuf, x0, x1, a.X + r, a.ld, (uint32_t)a.x_unit, mode,
-                                              packed, last, stk);
+            {
+                const float *xr = a.X + (rb + o);
+                if (FMODE == 2) {
+                    load_pairs<RPT, FMODE>(x0, xr, packed, last);
+                    load_pairs<RPT, FMODE>(x1, xr + a.ld, packed, last);
+                }
+                const uint32_t mode = a.x_unit == 0 || !whole ? 2u : packed ? 0u : 1u;
+                interpret<RPT, NSLOT, FMODE, EXT>(t, cbuf, x0, x1, xr, a.ld, (uint32_t)a.x_unit, mode,
+                                                  packed, last, stk, aux);
+            }
+            // the lane's first row again; in feature mode 0 from the item, as held
+            // across the interpreter it would cost two registers that spill
+            // (4M x 50: 21.5 -> 20.4 ms; with two columns, where nothing
+            // spills, 16M x 4096 260 -> 268 ms)
+            const int64_t r =
+                (FMODE == 2 ? rb : (int64_t)*const_cast<volatile int *>(&s_item[cur].x) * a.chunk_rows) + o;
+            const int nv = whole ? RPT : (last + 32) >> 5;  // rows of the lane that count
             if (kAhead && base + kEvalWarps * 32 * RPT < n_in)
                 first_column(base + kEvalWarps * 32 * RPT);
             if (PRED) {
@@ -591,8 +648,8 @@ __global__ void __launch_bounds__(eval_warps<RPT>() * 32,
                 continue;
             }
             uint64_t yv[RPT / 2], wv[RPT / 2];
-            load_pairs<RPT>(yv, a.y + r, packed, last);
-            if (a.w) load_pairs<RPT>(wv, a.w + r, packed, last);
+            load_pairs<RPT, FMODE>(yv, a.y + r, packed, last);
+            if (a.w) load_pairs<RPT, FMODE>(wv, a.w + r, packed, last);
             if (MOM) {
                 // d = p - shift keeps the sums of squares free of the
                 // cancellation a large mean would cause
