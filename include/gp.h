@@ -199,11 +199,13 @@ size_t gp_workspace_size(int n_progs, int64_t n_rows, int n_feat,
 
 /* The tunables gp_evaluate_ex would use for this shape: `opts` (may be NULL)
  * with every zero field filled from the autotuner's record for the shape, or
- * else from the built-in defaults (rows_per_thread 4; chunk_rows sized for
+ * else from the built-in defaults (rows_per_thread 8; chunk_rows sized for
  * about 16 work items per resident warp, 1024..16384 rows; blocks_per_sm 0 =
- * as many as fit).  Programs deeper than 8 stack slots, and programs that
- * use a function from GP_SQ on, always run with 4 rows per thread, whatever
- * rows_per_thread says.  Returns GP_ERR_ARG for invalid opts. */
+ * as many as fit).  Programs with a compiled stack of more than 8 values, and
+ * those of exactly 8 without GP_TAN and the functions from GP_SQ on, always
+ * run with 4 rows per thread, whatever rows_per_thread says; the others with
+ * one of those functions run with 8 when it is 8 and with 4 otherwise.
+ * Returns GP_ERR_ARG for invalid opts. */
 int gp_resolve_opts(int n_progs, int64_t n_rows, int n_feat, const gp_eval_opts *opts,
                     gp_eval_opts *out);
 
@@ -228,10 +230,9 @@ int gp_predict(const gp_node *progs, const int32_t *offsets, int n_progs,
 
 /* Predictions as gp_predict, with the evaluator's rows per thread taken
  * from opts (NULL: the defaults; only rows_per_thread is read, 4 or 8, and
- * it applies to the programs of the common class -- stack of at most 7
- * values, no extended function -- the others always run 4 rows per
- * thread).  Every prediction is the same bits whatever rows_per_thread
- * says: the per-row operations do not depend on how rows are grouped.
+ * it applies to the programs that gp_resolve_opts names -- the others
+ * always run 4 rows per thread).  Every prediction is the same bits whatever
+ * rows_per_thread says: the per-row operations do not depend on how rows are grouped.
  * Returns GP_ERR_ARG for bad arguments or opts. */
 int gp_predict_ex(const gp_node *progs, const int32_t *offsets, int n_progs,
                   const float *X, int64_t n_rows, int n_feat, const gp_eval_opts *opts,

@@ -21,7 +21,7 @@ issue; the same bodies as scalar FFMA, a packed one costing two issue slots
 anyway, took a third more code and Pagie-1 16M x 4096 from 301 to 398 ms),
 so the division forms share one body (the divisor staged in U;
 the reversed forms swap the rows into U first), sin and cos share one,
-and tan goes to the C++ switch.
+and the rarer functions go to the C++ switch.
 
 The evaluator's words are laid out for it by the block that copies them to
 shared memory: one index that the branch takes as it is (an `and` less) and a
@@ -29,14 +29,13 @@ stack pointer instead of slot numbers (two instructions less per push and
 pop).  The gradient variant reads the pre-pass's words, whose other bits hold
 slots and marker shapes.
 
-Variants: RPT in {4, 8} x DIVS (the division set, square root, reciprocal,
-sin, cos, log and exp run here; without DIVS they are handed back) x
-XREG (columns 0 and 1 held in registers; without it a column read takes
-the rows that were prefetched for it and prefetches the next one's; without
-DIVS and in the gradient variant it is handed back).  A word the loop does not run -- END, the extended
-functions, the trigonometric and exponential arguments outside their fast
-paths, and whatever DIVS or XREG leave out -- is handed back to the
-caller's switch with its constant, the address just past it, and the rows
+Variants: RPT in {4, 8} x ext (tan, sq, cube, max and min run here too) x XREG
+(columns 0 and 1 held in registers; without it a column read takes the rows
+that were prefetched for it and prefetches the next one's; in the gradient
+variant it is handed back).  A word the loop does not run -- END, the other
+extended functions, the trigonometric and exponential arguments outside
+their fast paths, and whatever the variant leaves out -- is handed back to
+the caller's switch with its constant, the address just past it, and the rows
 untouched.
 
 Run: python paper_2110_11226_gb300/csrc/gen_fast.py  (rewrites gp_fast.cuh)
@@ -53,11 +52,17 @@ OPS = dict(PUSH_X=0, PUSH_C=1, PUSH_X_SP=2, PUSH_C_SP=3, ADD_S=4, SUB_S=5, MUL_S
            DIV_X=16, DIV_C=17, RDIV_X=18, RDIV_C=19, SQRT=20, LOG=21, EXP=22, SIN=23, COS=24,
            TAN=25, ABS=26, NEG=27, INV=28, END=29, EXT1=30, EXT2=31)
 COL1 = 32
+# dispatch indexes of the cheap extended functions in the loop (ext): free
+# ones, given to their words when a block copies the program
+EXT_INDEX = dict(SQR=52, CUB=53, MAX=54, MIN=55)
 
 # float bit patterns (pinned by static_asserts in gp_math.cuh)
 K = dict(inv_pi=0x3EA2F983, magic=0x4B400000, magic1=0x4B400001, pi_hi=0x40490FDB, pi_mid=0xB3BBBD2E,
          pi_lo=0xA7772CED, q0=0xBE2AAAA6, q1=0x3C088769, q2=0xB94FB7D4, q3=0x362EDC67,
          trig_fast=0x47800000,
+         two_over_pi=0x3F22F983, pio2_hi=0x3FC90FDB, pio2_mid=0xB33BBD2E, pio2_lo=0xA6F72CED,
+         ts0=0xBE2AAAAB, ts1=0x3C088884, ts2=0xB95007C0, ts3=0x363668F9,
+         tc0=0x3D2AAAAB, tc1=0xBAB60B5C, tc2=0x37D0086F, tc3=0xB4920F4E,
          lp0=0xBEFFFFFD, lp1=0x3EAAAB7A, lp2=0xBE80024D, lp3=0x3E4C6960, lp4=0xBE29AE98,
          lp5=0x3E18C293, lp6=0xBE12824F, lp7=0x3DB2E3B9, ln2_hi=0x3F317200, ln2_lo=0x35BFBE8E,
          e1=0x3F800000, e2=0x3EFFFFFE, e3=0x3E2AAA06, e4=0x3D2AAC20, e5=0x3C09371C,
@@ -80,10 +85,10 @@ def kp(name, neg=False):
 
 
 class Gen:
-    def __init__(self, rpt, divs, xreg, grad=False):
-        self.rpt, self.divs, self.xreg, self.grad = rpt, divs, xreg, grad
+    def __init__(self, rpt, xreg, ext=False, grad=False):
+        self.rpt, self.xreg, self.ext, self.grad = rpt, xreg, ext, grad
         # columns in memory: the next column read is prefetched into XB
-        self.xmem = not xreg and divs and not grad
+        self.xmem = not xreg and not grad
         self.np = rpt // 2               # pairs per lane
         p = self.np
         names = ["pa"] + [f"T{i}" for i in range(p)]
@@ -305,6 +310,58 @@ class Gen:
             for r in (0, 1):
                 self.e(f"mad.lo.u32 %%m{r}, %%n{r}, 0x80000000, %%m{r};")
             self.e(f"mov.b64 {dst(i) if dst else self.T[i]}, {{%%m0, %%m1}};")
+
+    # tan of every row (the steps of trig_rows): r = x - j pi/2, the sine's and
+    # cosine's polynomials, their quotient, or minus the inverse one for odd
+    # j, by the division's steps.  0 (whose quotient's sign they lose), tiny
+    # and huge arguments are handed back, where the library's division takes
+    # twice as long (a word of 8 rows: 510 -> 264 issue cycles).  In the ext
+    # variants only: in the others, wherever it stood, it made populations
+    # without tan 1.5-5% slower (code size), so programs with tan run there
+    def tan(self):
+        self.range_check("trig_fast", lo="two_m60")
+        for i in range(self.np):
+            t = self.T[i]
+            self.e(f"mov.b64 %%K0, {kp('two_over_pi')};")
+            self.e(f"mov.b64 %%K1, {kp('magic')};")
+            self.e(f"fma.rn.f32x2 %%JM, {t}, %%K0, %%K1;")
+            self.e("sub.rn.f32x2 %%JJ, %%JM, %%K1;")
+            for n, (c, src) in enumerate((("pio2_hi", t), ("pio2_mid", "%%R"), ("pio2_lo", "%%R"))):
+                self.e(f"mov.b64 %%K0, {kp(c, True)};")
+                self.e(f"fma.rn.f32x2 %%R, %%JJ, %%K0, {src};")
+            self.e("mul.rn.f32x2 %%S, %%R, %%R;")
+            self.e(f"mov.b64 %%K0, {kp('ts3')};")
+            self.e(f"mov.b64 %%P, {kp('ts2')};")
+            self.e("fma.rn.f32x2 %%P, %%K0, %%S, %%P;")
+            for c in ("ts1", "ts0"):
+                self.e(f"mov.b64 %%K0, {kp(c)};")
+                self.e("fma.rn.f32x2 %%P, %%P, %%S, %%K0;")
+            self.e("mul.rn.f32x2 %%Q, %%S, %%R;")
+            self.e("fma.rn.f32x2 %%R, %%P, %%Q, %%R;")          # sine
+            self.e(f"mov.b64 %%K0, {kp('tc3')};")
+            self.e(f"mov.b64 %%P, {kp('tc2')};")
+            self.e("fma.rn.f32x2 %%P, %%K0, %%S, %%P;")
+            for c in ("tc1", "tc0", "mhalf", "one"):
+                self.e(f"mov.b64 %%K0, {kp(c)};")
+                self.e("fma.rn.f32x2 %%P, %%P, %%S, %%K0;")     # cosine
+            self.unpack(i, "%%n0", "%%n1", "%%JM")
+            self.e("mov.b64 {%%s0, %%s1}, %%R;")
+            self.e("mov.b64 {%%c0, %%c1}, %%P;")
+            for r in (0, 1):
+                self.e(f"and.b32 %%a, %%n{r}, 1;")
+                self.e("setp.ne.u32 %%p, %%a, 0;")
+                self.e(f"selp.f32 %%v{r}, %%c{r}, %%s{r}, %%p;")   # dividend
+                self.e(f"selp.f32 %%u{r}, %%s{r}, %%c{r}, %%p;")   # divisor
+            self.e("mov.b64 %%S, {%%v0, %%v1};")
+            self.e("mov.b64 %%U0, {%%u0, %%u1};")
+            self.rcp_pair("%%U0", "%%JJ")
+            self.e("mul.rn.f32x2 %%R, %%S, %%JJ;")
+            self.e("fma.rn.f32x2 %%Q, %%F, %%R, %%S;")             # a - b q
+            self.e("fma.rn.f32x2 %%R, %%Q, %%JJ, %%R;")
+            self.e("mov.b64 {%%m0, %%m1}, %%R;")
+            for r in (0, 1):
+                self.e(f"mad.lo.u32 %%m{r}, %%n{r}, 0x80000000, %%m{r};")
+            self.e(f"mov.b64 {t}, {{%%m0, %%m1}};")
 
     # log of every row (f_log: the logarithm of max(|t|, thr), 0 below the
     # threshold, inf and NaN passed through)
@@ -931,12 +988,32 @@ class Gen:
             swap()
             e("bra.uni DTUX%=;")
             return True
+        elif stem == "SQR" or stem == "CUB":
+            # t t and (t t) t, each product rounded
+            for i in range(p):
+                dst = "%%S" if stem == "CUB" else self.T[i]
+                e(f"mul.rn.f32x2 {dst}, {self.T[i]}, {self.T[i]};")
+                if stem == "CUB":
+                    e(f"mul.rn.f32x2 {self.T[i]}, %%S, {self.T[i]};")
+        elif stem in ("MAX", "MIN"):
+            # t when it is the larger (smaller) or NaN, else the slot's value
+            self.slot_load()
+            for i in range(p):
+                self.unpack(i, "%%v0", "%%v1")
+                e(f"mov.b64 {{%%u0, %%u1}}, %%U{i};")
+                for v, u in (("%%v0", "%%u0"), ("%%v1", "%%u1")):
+                    e(f"setp.{'gt' if stem == 'MAX' else 'lt'}.f32 %%p, {v}, {u};")
+                    e(f"setp.nan.or.f32 %%p, {v}, {v}, %%p;")
+                    e(f"selp.f32 {v}, {v}, {u}, %%p;")
+                self.pack(i, "%%v0", "%%v1")
         elif stem == "SQ":
             self.sqrt()
         elif stem == "IV":
             self.inv()
         elif stem == "TRG":
             self.trig()
+        elif stem == "TN":
+            self.tan()
         elif stem == "LG":
             self.log()
         elif stem == "XP":
@@ -954,24 +1031,27 @@ class Gen:
                     ADD_C="AC", SUB_C="SC", RSUB_C="RC", MUL_C="MC", ABS="AB", NEG="NG")
         for k, v in base.items():
             ent[OPS[k]] = v
-        if self.divs:
-            for k, v in dict(DIV_S="DS", DIV_C="DC", RDIV_C="RDC", SQRT="SQ", INV="IV",
-                             SIN="TRG", COS="TRG", LOG="LG", EXP="XP").items():
-                ent[OPS[k]] = v
+        for k, v in dict(DIV_S="DS", DIV_C="DC", RDIV_C="RDC", SQRT="SQ", INV="IV", SIN="TRG",
+                         COS="TRG", LOG="LG", EXP="XP").items():
+            ent[OPS[k]] = v
+        if self.ext:
+            ent[OPS["TAN"]] = "TN"
         if self.xreg or self.xmem:
             xops = dict(PUSH_X="PX", PUSH_X_SP="PXS", ADD_X="AX", SUB_X="SX", RSUB_X="RX",
                         MUL_X="MX")
-            if self.divs:
-                xops.update(DIV_X="DX", RDIV_X="RDX")
+            xops.update(DIV_X="DX", RDIV_X="RDX")
             for k, v in xops.items():
                 ent[OPS[k]] = v if self.xmem else v + "0"
                 if not self.xmem:
                     ent[OPS[k] | COL1] = v + "1"
+        if self.ext:
+            for k, v in EXT_INDEX.items():
+                ent[v] = k
         if self.grad:
             ent[OPS["END"] | COL1] = "MK"
         owner = {}
         for op, lab in enumerate(ent):
-            base = op & (COL1 - 1)
+            base = op if lab in EXT_INDEX else op & (COL1 - 1)
             if lab == "EX":
                 continue
             kind = {OPS["SIN"]: "trig", OPS["COS"]: "trig"}.get(base, base)
@@ -988,7 +1068,7 @@ class Gen:
         e(".reg .b32 %%w, %%cb, %%i, %%a, %%kd, %%n<2>, %%m<2>, %%k<2>;")
         e(".reg .f32 %%cf, %%q, %%m, %%mx, %%mn, %%v<2>, %%u<2>, %%s<2>, %%c<2>;")
         e(f".reg .b64 %%C, %%U<{p}>, %%K<2>, %%KM, %%JM, %%JJ, %%R, %%S, %%P, %%Q, %%F;")
-        if self.divs and self.special:
+        if self.special:
             e(".reg .b64 %%Y;")
         if self.xmem:
             e(".reg .pred %%pm, %%pb;")
@@ -1040,23 +1120,22 @@ class Gen:
                     self.body(name)
                     self.partial_code(self.PARTIAL[name])
                     e("brx.idx.uni %%tl, TQ%=;")
-        if self.divs:
-            # t = t / u with the protection, the divisor pairs in U
-            self.label("DTU")
-            self.div_body()
-            self.nxt()
-            if self.xmem:
-                # t = u / t, the dividend pairs in U: swap, then divide
-                self.label("RDU")
+        # t = t / u with the protection, the divisor pairs in U
+        self.label("DTU")
+        self.div_body()
+        self.nxt()
+        if self.xmem:
+            # t = u / t, the dividend pairs in U: swap, then divide
+            self.label("RDU")
 
-                def swap():
-                    for i in range(p):
-                        e(f"mov.b64 %%S, {self.T[i]};")
-                        e(f"mov.b64 {self.T[i]}, %%U{i};")
-                        e(f"mov.b64 %%U{i}, %%S;")
-                self.div_check(num=lambda i: f"%%U{i}", den=lambda i: self.T[i], pre=swap)
-                swap()
-                e("bra.uni DTUX%=;")
+            def swap():
+                for i in range(p):
+                    e(f"mov.b64 %%S, {self.T[i]};")
+                    e(f"mov.b64 {self.T[i]}, %%U{i};")
+                    e(f"mov.b64 %%U{i}, %%S;")
+            self.div_check(num=lambda i: f"%%U{i}", den=lambda i: self.T[i], pre=swap)
+            swap()
+            e("bra.uni DTUX%=;")
         if self.grad:
             # stubs into the shared bodies: ret = the word's index + 1 (TR)
             done = set()
@@ -1089,11 +1168,11 @@ class Gen:
 
 
 
-def function(rpt, divs, xreg, grad=False):
-    g = Gen(rpt, divs, xreg, grad)
+def function(rpt, xreg, ext=False, grad=False):
+    g = Gen(rpt, xreg, ext, grad)
     lines = g.generate()
     p = rpt // 2
-    name = f"fast_r{rpt}_{'divs' if divs else 'nodivs'}_{'x' if xreg else 'nox'}" + \
+    name = f"fast_r{rpt}_{'ext' if ext else 'divs'}_{'x' if xreg else 'nox'}" + \
         ("_grad" if grad else "")
     body = "\n".join(f'        "{ln}\\n\\t"' for ln in lines)
     xmem = g.xmem
@@ -1118,18 +1197,19 @@ def function(rpt, divs, xreg, grad=False):
 HEADER = '''// gp_fast.cuh -- the evaluator's indexed-branch fast loop in inline PTX.
 // GENERATED by gen_fast.py (same directory); edit that script, not this file.
 //
-// fast_r<RPT>_<divs|nodivs>_<x|nox>(pa, t, ..., sp, hw, hc) runs compiled
+// fast_r<RPT>_<divs|ext>_<x|nox>(pa, t, ..., sp, hw, hc) runs compiled
 // words -- the dispatch index and a constant -- from the shared-memory address
 // pa over RPT rows per lane, held as RPT/2 pairs {row 2i, row 2i+1} in t.  It
 // stops at the first word it does not run, returns that word and its constant
 // in hw and hc, leaves pa just past it and the rows untouched by it.  sp is the
 // lane's next free slot of the shared-memory stack ([slot][q][lane] float4); a
-// division handed back by the divs variants has taken its operand off.  The _x variants take columns 0
+// division handed back has taken its operand off.  ext: with tan, sq, cube,
+// max and min.  The _x variants take columns 0
 // and 1 of the lane's rows in x0 and x1; the _nox ones read columns from
 // memory: xb holds the rows of the column that the program reads next, xc
 // is column 0 at the lane's first row, a word's constant times unit the bytes
-// from there to the next column, mode how the lane's rows lie (without the
-// division set, and in the gradient's, column reads are handed back).  Every one of the 64
+// from there to the next column, mode how the lane's rows lie (in the gradient's
+// variant column reads are handed back).  Every one of the 64
 // values of the six-bit dispatch index has a table entry.  The statement
 // declares no memory clobber: the shared memory it reads and writes (the
 // code buffer, written before a barrier, and the stack, touched elsewhere
@@ -1148,13 +1228,13 @@ namespace gpk {
 def main():
     parts = [HEADER]
     for rpt in (4, 8):
-        for divs in (True, False):
+        for ext in (False, True):
             for xreg in (True, False):
-                parts.append(function(rpt, divs, xreg))
+                parts.append(function(rpt, xreg, ext))
                 parts.append("\n")
     # the constant gradient's loop (4 rows per lane, the division set)
     for xreg in (True, False):
-        parts.append(function(4, True, xreg, grad=True))
+        parts.append(function(4, xreg, grad=True))
         parts.append("\n")
     parts.append("}  // namespace gpk\n")
     with open(os.path.join(HERE, "gp_fast.cuh"), "w") as f:

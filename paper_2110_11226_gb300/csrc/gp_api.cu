@@ -303,11 +303,15 @@ int run_evaluate(const gp_node *progs, const int32_t *offsets, int n_progs, cons
             ea.shift = W.shift;
             ea.ystat = W.ystat;
         }
-        // classes 1-3 keep 4 rows per thread (the 19-slot stack would
-        // otherwise leave room for one block per SM; classes 2 and 3 are
-        // rare); the same chunk partition serves all four
+        // classes 1 and 3 keep 4 rows per thread (the 19-slot stack would
+        // otherwise leave room for one block per SM; class 3 is rare); class 2
+        // takes 8 when class 0 does (Pearson over the extended set, 1024 x
+        // 262K x 28: 2.33 -> 2.30 ms; its cheap words take half as long); the
+        // same chunk partition serves all four
         const int rpt_long = (mom && pl.o.long_rows_per_thread == 16) ? 8 : pl.o.long_rows_per_thread;
-        const int rpt_c = (cls == kClassShallow) ? (ea.sub == 1 ? rpt_long : rpt) : 4;
+        const int rpt_c = cls == kClassShallow      ? (ea.sub == 1 ? rpt_long : rpt)
+                          : cls == kClassShallowExt ? (rpt == 8 ? 8 : 4)
+                                                    : 4;
         const int want = ea.sub == 1 ? pl.o.long_blocks_per_sm : pl.o.blocks_per_sm;
         const int block = kEvalBlockThreads;
         int occ = eval_info(rpt_c, fmode, cls, block, nullptr, mom);
@@ -389,7 +393,7 @@ int run_predict_compiled(const Workspace &W, int p0, int b, const float *X, int6
         ea.dev_status = c->status;
         ea.vec_ok = vec ? 1 : 0;
         ea.x_unit = x_unit(n_feat, ea.ld, vec);
-        if (cls == kClassShallow && rpt == 8) {
+        if ((cls == kClassShallow || cls == kClassShallowExt) && rpt == 8) {
             // the class-0 instance at 8 rows per thread (its store epilogue)
             const int occ = eval_info(8, fmode, cls, kEvalBlockThreads, nullptr, false, true);
             GP_CUDA(eval_launch(ea, 8, fmode, c->sms * std::max(occ, 1), kEvalBlockThreads, st));

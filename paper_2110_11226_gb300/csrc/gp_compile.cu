@@ -319,7 +319,7 @@ __global__ void __launch_bounds__(kCompileWarps * 32) compile_kernel(CompileArgs
 
     // emit, from the end of the list
     int n = 0, sp_car = 0, depth = 0;
-    bool ext = false;  // an extended-set instruction was emitted
+    bool ext = false;  // an instruction of the extended classes was emitted
     // more than two columns: each column read names the next one; the chunk's
     // last is completed when a later chunk emits one (at: its place, -1 none)
     const bool linked = a.n_feat > 2;
@@ -359,7 +359,9 @@ __global__ void __launch_bounds__(kCompileWarps * 32) compile_kernel(CompileArgs
             }
         } else if (emit && ar == 1) {
             const bool e = op > GP_INV;  // extended function: its number in the feature field
-            ext |= e;
+            // the loop of class 0 does not run tan (the gradient's classes go by
+            // the extended functions alone)
+            ext |= e || (op == GP_TAN && !a.grad);
             word.x = e ? make_ins(OP_EXT1, 0, (uint32_t)(op - GP_SQ))
                        : make_ins(OP_SQRT + (op - GP_SQRT), 0, 0);
             j_top = j + 1;

@@ -87,6 +87,9 @@ constexpr uint32_t kGradMark = OP_END | kOpCol1;
 constexpr int kGradCodeStride = 512;  // words of the gradient form (<= 2 per node + END)
 enum : uint32_t { EXT_SQ = 0, EXT_CUBE, EXT_CBRT, EXT_TANH, EXT_ATAN, EXT_SINH, EXT_COSH };
 enum : uint32_t { EXT_MAX = 0, EXT_MIN = 1 };
+// the fast loop's dispatch indexes of the extended functions that it runs
+// (free ones; gen_fast.py's EXT_INDEX)
+constexpr uint32_t kIndexSq = 52, kIndexCube = 53, kIndexMax = 54, kIndexMin = 55;
 
 __host__ __device__ constexpr uint32_t make_ins(uint32_t op, uint32_t slot, uint32_t feat) {
     return op | (slot << 8) | (feat << 16);
@@ -114,18 +117,18 @@ struct ProgMeta {
     int32_t n_ins;     // instructions including END
     int32_t status;    // gp_prog_status
     int16_t depth;     // largest stack height of the compiled form
-    int16_t ext;       // 1: uses an extended function (EXT1/EXT2 words)
+    int16_t ext;       // 1: uses tan or an extended function (EXT1/EXT2 words)
     int32_t n_consts;  // CONST nodes
 };
 
-// Program classes, one evaluator instance each.  Programs without the
-// extended functions whose compiled stack fits kShallowDepth form class 0,
+// Program classes, one evaluator instance each.  Programs without tan and
+// the extended functions whose compiled stack fits kShallowDepth form class 0,
 // the common one: a 6-slot shared-memory stack, so that at 8 rows per
 // thread 4 blocks of 8 warps fit per SM (a 7-slot stack fits 3).  Those of
 // depth kSmallDepth form class 3 (7 slots, 4 rows per thread); programs
-// with the extended functions and a stack of at most kSmallDepth, class 2
-// (7 slots; their dispatch entries would slow class 0 down); deeper
-// programs, class 1 (19 slots, every function).
+// with tan or the extended functions and a stack of at most kSmallDepth,
+// class 2 (7 slots, up to 8 rows per thread; their code would slow class 0
+// down); deeper programs, class 1 (19 slots, every function, 4 rows).
 constexpr int kSmallDepth = 8;     // 7 stack slots + t
 constexpr int kShallowDepth = 7;   // 6 stack slots + t
 constexpr int kNumClasses = 4;

@@ -275,32 +275,29 @@ static __device__ __noinline__ float4 ext_rows4(float4 v, uint32_t f) {
 // per lane: a lane's rows sit in RPT/2 64-bit pairs and add, sub, mul and
 // fma run as one packed f32x2 instruction per pair (per-element round to
 // nearest, no flush to zero: the bits of the scalar operations).  It runs
-// pushes and stack moves, add/sub/mul with every operand form, abs, neg,
-// column reads from registers (XREG) and, with DIVS, the protected
-// divisions, square root, reciprocal, sin, cos, tan, log and exp (the steps
-// and constants of gp_math.cuh, so results are the same bits).  It stops
-// at the first word it does not run (END, the extended functions, a
-// trigonometric or exponential argument outside the fast path in any row
-// of the warp, and whatever XREG or DIVS leave out), hands that word and
-// its constant back to the switch below and leaves pa just past it.  DIVS
-// is off in the instances with the extended functions: there the division
-// set in the loop cost the extended-set population 23% (their out-of-line
-// calls and the division's own slow-path call do not mix well).
-template <int RPT, bool DIVS, bool XREG>
+// pushes and stack moves, add/sub/mul with every operand form, abs, neg, the
+// protected divisions, square root, reciprocal, sin, cos, log and exp (the
+// steps and constants of gp_math.cuh, so results are the same bits), column
+// reads from registers (XREG) or one ahead from memory, and, with EXT, sq,
+// cube, max and min.  It stops at the first word it does not run (END, tan,
+// the other extended functions, arguments outside a fast path in any row of
+// the warp, column reads of a ragged sub-tile), hands that word and its
+// constant back to the switch below and leaves pa just past it.
+template <int RPT, bool EXT, bool XREG>
 __device__ __forceinline__ void run_fast(uint32_t &pa, uint64_t (&t)[RPT / 2],
                                          uint64_t (&x0)[RPT / 2], const uint64_t (&x1)[RPT / 2],
                                          const float *xc, uint32_t unit, uint32_t mode, uint32_t &sp,
                                          uint32_t &hw, float &hc) {
     if constexpr (RPT == 4) {
-        if constexpr (DIVS && XREG) fast_r4_divs_x(pa, t, x0, x1, sp, hw, hc);
-        else if constexpr (DIVS) fast_r4_divs_nox(pa, t, x0, xc, unit, mode, sp, hw, hc);
-        else if constexpr (XREG) fast_r4_nodivs_x(pa, t, x0, x1, sp, hw, hc);
-        else fast_r4_nodivs_nox(pa, t, x0, x1, sp, hw, hc);
+        if constexpr (!EXT && XREG) fast_r4_divs_x(pa, t, x0, x1, sp, hw, hc);
+        else if constexpr (!EXT) fast_r4_divs_nox(pa, t, x0, xc, unit, mode, sp, hw, hc);
+        else if constexpr (XREG) fast_r4_ext_x(pa, t, x0, x1, sp, hw, hc);
+        else fast_r4_ext_nox(pa, t, x0, xc, unit, mode, sp, hw, hc);
     } else {
-        if constexpr (DIVS && XREG) fast_r8_divs_x(pa, t, x0, x1, sp, hw, hc);
-        else if constexpr (DIVS) fast_r8_divs_nox(pa, t, x0, xc, unit, mode, sp, hw, hc);
-        else if constexpr (XREG) fast_r8_nodivs_x(pa, t, x0, x1, sp, hw, hc);
-        else fast_r8_nodivs_nox(pa, t, x0, x1, sp, hw, hc);
+        if constexpr (!EXT && XREG) fast_r8_divs_x(pa, t, x0, x1, sp, hw, hc);
+        else if constexpr (!EXT) fast_r8_divs_nox(pa, t, x0, xc, unit, mode, sp, hw, hc);
+        else if constexpr (XREG) fast_r8_ext_x(pa, t, x0, x1, sp, hw, hc);
+        else fast_r8_ext_nox(pa, t, x0, xc, unit, mode, sp, hw, hc);
     }
 }
 
@@ -352,7 +349,7 @@ __device__ __forceinline__ void interpret(uint64_t (&tp)[RPT / 2], const uint2 *
         uint2 ins;
         if constexpr (kFast) {
             float hc;
-            run_fast<RPT, !EXT, FMODE == 2>(pa, tp, x0p, x1p, xc, unit, mode, sp, ins.x, hc);
+            run_fast<RPT, EXT, FMODE == 2>(pa, tp, x0p, x1p, xc, unit, mode, sp, ins.x, hc);
             ins.y = __float_as_uint(hc);
         } else {
             asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];"
@@ -415,7 +412,7 @@ __device__ __forceinline__ void interpret(uint64_t (&tp)[RPT / 2], const uint2 *
             case OP_SUB_S: GP_POP(u) GP_T(f_sub(t[j], u[j])) break;
             case OP_MUL_S: GP_POP(u) GP_T(f_mul(t[j], u[j])) break;
             case OP_DIV_S:  // (the loop has moved sp for a division that it hands back)
-                if (kFast && !EXT) GP_SLOT_LOAD(u) else GP_POP(u)
+                if (kFast) GP_SLOT_LOAD(u) else GP_POP(u)
                 goto div_tu;
             case OP_ADD_X: GP_X_LOAD(u) GP_T(f_add(t[j], u[j])) break;
             case OP_ADD_C: GP_T(f_add(t[j], c)) break;
@@ -451,15 +448,7 @@ __device__ __forceinline__ void interpret(uint64_t (&tp)[RPT / 2], const uint2 *
                 } else {
                     goto done;
                 }
-            case OP_EXT2:  // max / min, right operand in a stack slot
-                if constexpr (kExt) {
-                    GP_POP(u)
-                    if (GP_HI == EXT_MAX) { GP_T(f_max(t[j], u[j])) }
-                    else { GP_T(f_min(t[j], u[j])) }
-                    break;
-                } else {
-                    goto done;
-                }
+            case OP_EXT2:  // max and min run in the loop
             case OP_END:
                 goto done;
             default:  // every value of w & 31 has a case above
@@ -505,7 +494,7 @@ constexpr int kEpiLoss = 0, kEpiPred = 1, kEpiMom = 2;
 
 template <int RPT, int NSLOT, int FMODE, int EPI, bool EXT>
 __global__ void __launch_bounds__(eval_warps<RPT>() * 32,
-                                  RPT == 8 ? (EPI == kEpiMom ? 3 : 4)
+                                  RPT == 8 ? (EPI == kEpiMom || EXT ? 3 : 4)
                                            : (EPI == kEpiMom && RPT == 4 ? 5 : 0))
     eval_kernel(const EvalArgs a) {
     constexpr bool PRED = EPI == kEpiPred;
@@ -575,9 +564,13 @@ __global__ void __launch_bounds__(eval_warps<RPT>() * 32,
                 uint2 v = src[i];
                 aux[i] = (uint16_t)(v.x >> 16);
                 // a column read's constant: the next column read, as an offset
-                if (FMODE == 0 && !EXT && (kColumnOps >> (v.x & 31u) & 1u))
+                if (FMODE == 0 && (kColumnOps >> (v.x & 31u) & 1u))
                     v.y = (uint32_t)((uint64_t)v.y * (uint64_t)(a.x_unit == 16 ? a.ld >> 2 : a.ld));
-                cbuf[i] = make_uint2(v.x & 63u, v.y);
+                const uint32_t op = v.x & 31u, fn = v.x >> 16;
+                uint32_t index = v.x & 63u;
+                if (EXT && op == OP_EXT2) index = fn == EXT_MAX ? kIndexMax : kIndexMin;
+                if (EXT && op == OP_EXT1 && fn <= EXT_CUBE) index = fn == EXT_SQ ? kIndexSq : kIndexCube;
+                cbuf[i] = make_uint2(index, v.y);
             }
         }
         __syncthreads();  // the words are there
@@ -599,7 +592,7 @@ __global__ void __launch_bounds__(eval_warps<RPT>() * 32,
             load_pairs<RPT, FMODE>(x0, a.X + (feat * a.ld + (int64_t)it->x * a.chunk_rows + o), pk,
                             n_in - 1 - o);
         };
-        constexpr bool kAhead = FMODE == 0 && !EXT;  // the loop reads columns ahead
+        constexpr bool kAhead = FMODE == 0;  // the loop reads columns ahead
         if (kAhead && ok && warp * 32 * RPT < n_in) first_column(warp * 32 * RPT);
         for (int base = warp * 32 * RPT; base < n_in && ok; base += kEvalWarps * 32 * RPT) {
             // whole: every row of the sub-tile is in the chunk; packed: and
