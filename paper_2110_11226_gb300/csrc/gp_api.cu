@@ -20,8 +20,6 @@ __device__ unsigned int g_gp_status_word;
 
 namespace {
 
-constexpr int kMaxDevices = 64;
-
 struct ShapeKey {
     int n_progs;
     int64_t n_rows;
@@ -273,10 +271,14 @@ int run_evaluate(const gp_node *progs, const int32_t *offsets, int n_progs, cons
         tev = timing_pair();
         GP_CUDA(cudaEventRecord(tev.first, st));
     }
-    // launches: class 0 (or, split by length, its long then its short
-    // programs), classes 1, 2 and 3
-    for (int launch = split ? -1 : 0; launch < kNumClasses; ++launch) {
-        const int cls = launch < 0 ? 0 : launch;
+    // launches: the deep programs and class 3, rare and slow, first, so that
+    // they run beside the others; then class 2, then class 0 (split by length:
+    // its long programs, then the rest)
+    constexpr int kLaunches[] = {kClassDeep, kClassShallow8, kClassShallowExt, -1, kClassShallow};
+    for (int i = 0; i < 5; ++i) {
+        const int launch = kLaunches[i];
+        if (launch < 0 && !split) continue;
+        const int cls = launch < 0 ? kClassShallow : launch;
         EvalArgs ea{};
         ea.code = W.code;
         ea.meta = W.meta;
@@ -293,6 +295,7 @@ int run_evaluate(const gp_node *progs, const int32_t *offsets, int n_progs, cons
         ea.chunk_rows = pl.o.chunk_rows;
         ea.n_chunks = pl.n_chunks;
         ea.sub = split && cls == kClassShallow ? (launch < 0 ? 1 : 2) : 0;
+        ea.follows = i > 0;
         ea.counter = W.counters + (ea.sub == 1 ? kNumClasses : cls);
         ea.part = W.part;
         ea.dev_status = c->status;
@@ -374,8 +377,9 @@ int run_predict_compiled(const Workspace &W, int p0, int b, const float *X, int6
     GP_CUDA(launch_order(W.meta + p0, b, W.order, W.class_count, st, W.counters));
     const bool vec = aligned16(X) && aligned16(out_pred) && (n_rows % 4 == 0);
     const int fmode = (n_feat <= 2) ? 2 : 0;
-    for (int cls = 0; cls < kNumClasses; ++cls) {
+    for (int cls : {kClassDeep, kClassShallow8, kClassShallowExt, kClassShallow}) {
         EvalArgs ea{};
+        ea.follows = cls != kClassDeep;
         ea.code = W.code + (size_t)p0 * kCodeStride;
         ea.meta = W.meta + p0;
         ea.order = W.order;

@@ -144,6 +144,8 @@ struct CompileScratch {    // of one warp
 
 __global__ void __launch_bounds__(kCompileWarps * 32) compile_kernel(CompileArgs a) {
     __shared__ CompileScratch scratch[kCompileWarps];
+    griddep_wait();
+    griddep_launch();
     const int lane = threadIdx.x & 31;
     const int p = blockIdx.x * kCompileWarps + (threadIdx.x >> 5);
     if (p >= a.n_progs) return;  // the whole warp
@@ -448,8 +450,7 @@ __global__ void __launch_bounds__(kCompileWarps * 32) compile_kernel(CompileArgs
 cudaError_t launch_compile(const CompileArgs &a, cudaStream_t st) {
     if (a.n_progs <= 0) return cudaSuccess;
     const int grid = (a.n_progs + kCompileWarps - 1) / kCompileWarps;
-    compile_kernel<<<grid, kCompileWarps * 32, 0, st>>>(a);
-    return cudaGetLastError();
+    return launch_chained(compile_kernel, grid, kCompileWarps * 32, 0, st, a);
 }
 
 // Counting sort of program ids: key = class * 256 + (256 - n_ins), so the
@@ -480,6 +481,8 @@ __global__ void __launch_bounds__(kOrderThreads) order_kernel(const ProgMeta *me
                                                               double *sumw, int64_t n_rows) {
     __shared__ int cursor[kOrderThreads * kBinsPerThread + 1];  // counts, then first positions
     __shared__ int warp_sum[kOrderThreads / 32];
+    griddep_wait();
+    griddep_launch();
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     if (t < 8 && counters) counters[t] = 0ull;
     if (t == 0 && sumw) *sumw = (double)n_rows;
@@ -525,9 +528,8 @@ __global__ void __launch_bounds__(kOrderThreads) order_kernel(const ProgMeta *me
 cudaError_t launch_order(const ProgMeta *meta, int n_progs, int32_t *order, int32_t *class_count,
                          cudaStream_t st, unsigned long long *counters, int mode, int edge,
                          double *sumw, int64_t n_rows) {
-    order_kernel<<<1, kOrderThreads, 0, st>>>(meta, n_progs, order, class_count, mode, edge, counters,
-                                              sumw, n_rows);
-    return cudaGetLastError();
+    return launch_chained(order_kernel, 1, kOrderThreads, 0, st, meta, n_progs, order, class_count, mode,
+                          edge, counters, sumw, n_rows);
 }
 
 // FP64 sums over the rows with a fixed partition: block b sums rows
@@ -591,6 +593,8 @@ __global__ void __launch_bounds__(kSumThreads) sumw_kernel(const float *__restri
                                                            double *part, double *sumw,
                                                            unsigned long long *ticket) {
     __shared__ double red[1][kSumThreads];
+    griddep_wait();
+    griddep_launch();
     const int64_t span = (n_rows + gridDim.x - 1) / gridDim.x;
     const int64_t r0 = (int64_t)blockIdx.x * span;
     const int64_t r1 = min(n_rows, r0 + span);
@@ -602,8 +606,8 @@ __global__ void __launch_bounds__(kSumThreads) sumw_kernel(const float *__restri
 
 cudaError_t launch_sumw(const float *w, int64_t n_rows, double *part, double *sumw,
                         unsigned long long *ticket, cudaStream_t st) {
-    sumw_kernel<<<sum_blocks(n_rows), kSumThreads, 0, st>>>(w, n_rows, part, sumw, ticket);
-    return cudaGetLastError();
+    return launch_chained(sumw_kernel, sum_blocks(n_rows), kSumThreads, 0, st, w, n_rows, part, sumw,
+                          ticket);
 }
 
 // Statistics of y for the correlation fitness: phase 0 sums w y and sets
@@ -618,6 +622,8 @@ __global__ void __launch_bounds__(kSumThreads) ystats_kernel(const float *__rest
                                                              unsigned long long *ticket) {
     constexpr int K = PHASE + 1;
     __shared__ double red[K][kSumThreads];
+    griddep_wait();
+    griddep_launch();
     const int64_t span = (n_rows + gridDim.x - 1) / gridDim.x;
     const int64_t r0 = (int64_t)blockIdx.x * span;
     const int64_t r1 = min(n_rows, r0 + span);
@@ -651,9 +657,11 @@ __global__ void __launch_bounds__(kSumThreads) ystats_kernel(const float *__rest
 cudaError_t launch_ystats(const float *y, const float *w, int64_t n_rows, const double *sumw,
                           double *part, double *ystat, unsigned long long *ticket, cudaStream_t st) {
     const int grid = sum_blocks(n_rows);
-    ystats_kernel<0><<<grid, kSumThreads, 0, st>>>(y, w, n_rows, sumw, ystat, part, ticket);
-    ystats_kernel<1><<<grid, kSumThreads, 0, st>>>(y, w, n_rows, sumw, ystat, part, ticket);
-    return cudaGetLastError();
+    const cudaError_t e =
+        launch_chained(ystats_kernel<0>, grid, kSumThreads, 0, st, y, w, n_rows, sumw, ystat, part, ticket);
+    if (e != cudaSuccess) return e;
+    return launch_chained(ystats_kernel<1>, grid, kSumThreads, 0, st, y, w, n_rows, sumw, ystat, part,
+                          ticket);
 }
 
 }  // namespace gpk

@@ -31,6 +31,7 @@
 
 namespace gpk {
 
+constexpr int kMaxDevices = 64;
 constexpr int kCodeStride = 256;   // instructions per program (255 + END)
 constexpr int kEvalBlockThreads = 256;  // threads per block of the evaluator
 constexpr int kDeepSlots = GP_MAX_STACK - 1;  // s[0..18]
@@ -198,6 +199,34 @@ void static_scratch_forget();
 size_t workspace_bytes_for(int n_progs, int64_t n_rows, int n_feat, const gp_eval_opts *opts,
                            int metric);
 
+// ---- chained launches ----------------------------------------------------
+// The kernels of an evaluation follow one another closely: each is launched
+// with programmatic stream serialization, so that its blocks may be set up
+// while the one before still runs, and waits for that one's completion
+// (griddep_wait) before it touches memory.  griddep_launch lets the next
+// kernel's set-up begin.  Every chained kernel waits, so the completion of the
+// last one is the completion of all.  512 programs x 4096 rows: 62 -> 52 us, with the
+// host call 44 -> 34 us (also fewer runtime calls, see info_t).
+__device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void griddep_launch() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+template <class... P, class... A>
+cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                           A &&...args) {
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // ---- kernels / launchers (defined in the .cu files) --------------------
 struct CompileArgs {
     const gp_node *progs;
@@ -272,6 +301,9 @@ struct EvalArgs {
     // 0: the programs of class cls; k + 1: those of order class k (the
     // constant gradient's buckets: its constant-free programs)
     int qcls;
+    // 1: launched right after another launch of the same evaluation, on whose
+    // results it does not depend: it runs beside that one
+    int follows;
 };
 // One launcher per (rows per thread, feature mode) instance; a.cls picks
 // the program class (stack slots, extended functions).  fmode 2: columns 0 and 1 held in

@@ -44,6 +44,8 @@
 // 16.3 ms).
 #pragma once
 
+#include <atomic>
+
 #include "gp_internal.cuh"
 #include "gp_math.cuh"
 #include "gp_fast.cuh"
@@ -513,7 +515,6 @@ __global__ void __launch_bounds__(eval_warps<RPT>() * 32,
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     float4 *stk = stack_all + (size_t)warp * NSLOT * (RPT / 4) * 32 + lane;
-    const float ybar = MOM ? (float)a.ystat[3] : 0.0f;
 
     // Thread 0 takes the next item while the block works on this one: it
     // alone waits for the counter and splits the number into (chunk, rank).
@@ -531,6 +532,13 @@ __global__ void __launch_bounds__(eval_warps<RPT>() * 32,
         }
         s_item[slot] = it;
     };
+    // a launch that follows starts once every block of the first has passed its
+    // wait here, so what the kernels before that one wrote is in the L2 by
+    // then; the fence keeps this block's loads from older lines in its L1
+    if (a.follows) __threadfence();
+    else griddep_wait();
+    griddep_launch();
+    const float ybar = MOM ? (float)a.ystat[3] : 0.0f;
     if (threadIdx.x == 0) {
         const int qc = a.qcls ? a.qcls - 1 : a.cls;  // the span of the program order
         int begin = 0, n = a.class_count[qc];
@@ -700,33 +708,44 @@ __global__ void __launch_bounds__(eval_warps<RPT>() * 32,
             a.part[(size_t)p * a.n_chunks + chunk] = ok ? v : __int_as_float(0x7fc00000);
         }
     }
+    // complete only after the launch that this one follows
+    if (a.follows && blockIdx.x == 0) griddep_wait();
+}
+
+// Resident blocks per SM, after making the instance's shared memory
+// available; asked for once per device (the two runtime calls took 3 us of
+// each of an evaluation's four launches)
+template <int RPT, int NSLOT, int FMODE, int EPI, bool EXT>
+int info_t(int block, int *regs) {
+    (void)block;
+    static std::atomic<int> known[kMaxDevices];  // blocks + 1
+    constexpr size_t smem = eval_smem_bytes<RPT, NSLOT>();
+    auto k = eval_kernel<RPT, NSLOT, FMODE, EPI, EXT>;
+    if (regs) {
+        cudaFuncAttributes fa{};
+        if (cudaFuncGetAttributes(&fa, k) != cudaSuccess) return 0;
+        *regs = fa.numRegs;
+    }
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return 0;
+    int n = known[dev].load(std::memory_order_acquire) - 1;
+    if (n >= 0) return n;
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, eval_warps<RPT>() * 32, smem) != cudaSuccess)
+        return 0;
+    known[dev].store(n + 1, std::memory_order_release);
+    return n;
 }
 
 template <int RPT, int NSLOT, int FMODE, int EPI, bool EXT>
 cudaError_t launch_eval_t(const EvalArgs &a, int grid, int block, cudaStream_t st) {
-    (void)block;
     constexpr size_t smem = eval_smem_bytes<RPT, NSLOT>();
-    auto k = eval_kernel<RPT, NSLOT, FMODE, EPI, EXT>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    k<<<grid, eval_warps<RPT>() * 32, smem, st>>>(a);
-    return cudaGetLastError();
-}
-
-template <int RPT, int NSLOT, int FMODE, int EPI, bool EXT>
-int info_t(int block, int *regs) {
-    (void)block;
-    constexpr size_t smem = eval_smem_bytes<RPT, NSLOT>();
-    auto k = eval_kernel<RPT, NSLOT, FMODE, EPI, EXT>;
-    cudaFuncAttributes fa{};
-    if (cudaFuncGetAttributes(&fa, k) != cudaSuccess) return 0;
-    if (regs) *regs = fa.numRegs;
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-        return 0;
-    int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, eval_warps<RPT>() * 32, smem) != cudaSuccess)
-        return 0;
-    return n;
+    if (info_t<RPT, NSLOT, FMODE, EPI, EXT>(block, nullptr) < 1) {
+        const cudaError_t e = cudaGetLastError();
+        return e != cudaSuccess ? e : cudaErrorInvalidConfiguration;
+    }
+    return launch_chained(eval_kernel<RPT, NSLOT, FMODE, EPI, EXT>, grid, eval_warps<RPT>() * 32, smem, st,
+                          a);
 }
 
 }  // namespace gpk

@@ -36,9 +36,19 @@ __device__ double pearson_from_moments(double s1, double s2, double s12, double 
     return fabs(cov) / sqrt(vp * vy);
 }
 
+// the 32 lanes' sums by a fixed butterfly, the same value in every lane (one
+// lane after the other, they were 32 dependent FP64 additions)
+__device__ __forceinline__ double warp_sum(double s) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    return s;
+}
+
 // warp w handles program w; lane l adds chunks l, l+32, ... in order, then
-// the 32 lane sums are combined by lane 0 in lane order.
+// the 32 lane sums are combined by a fixed butterfly.
 __global__ void __launch_bounds__(256) finalize_kernel(FinalizeArgs a) {
+    griddep_wait();
+    griddep_launch();
     const int lane = threadIdx.x & 31;
     const int p = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
     if (p >= a.n_progs) return;
@@ -52,10 +62,8 @@ __global__ void __launch_bounds__(256) finalize_kernel(FinalizeArgs a) {
         double s[3] = {0.0, 0.0, 0.0};
         for (int i = lane; i < a.n_chunks; i += 32)
             for (int k = 0; k < 3; ++k) s[k] += mp[(size_t)i * 3 + k];
-        double S[3] = {0.0, 0.0, 0.0};
-        for (int l = 0; l < 32; ++l)
-            for (int k = 0; k < 3; ++k) S[k] += __shfl_sync(0xffffffffu, s[k], l);
-        f = pearson_from_moments(S[0], S[1], S[2], *a.sumw, a.ystat[1], a.ystat[2]);
+        for (int k = 0; k < 3; ++k) s[k] = warp_sum(s[k]);
+        f = pearson_from_moments(s[0], s[1], s[2], *a.sumw, a.ystat[1], a.ystat[2]);
     } else if (a.accum == GP_ACCUM_KAHAN32) {
         float s = 0.0f, c = 0.0f;
         for (int i = lane; i < a.n_chunks; i += 32) kahan32(s, c, part[i]);
@@ -70,9 +78,7 @@ __global__ void __launch_bounds__(256) finalize_kernel(FinalizeArgs a) {
     } else {
         double s = 0.0;
         for (int i = lane; i < a.n_chunks; i += 32) s += (double)part[i];
-        double S = 0.0;
-        for (int l = 0; l < 32; ++l) S += __shfl_sync(0xffffffffu, s, l);
-        f = finish_metric(a.metric, S, *a.sumw);
+        f = finish_metric(a.metric, warp_sum(s), *a.sumw);
     }
     if (m.status != GP_PROG_OK) f = __longlong_as_double(0x7ff8000000000000LL);
     if (lane == 0) {
@@ -86,8 +92,7 @@ cudaError_t launch_finalize(const FinalizeArgs &a, cudaStream_t st) {
     if (a.n_progs <= 0) return cudaSuccess;
     const int warps = 8;
     const int grid = (a.n_progs + warps - 1) / warps;
-    finalize_kernel<<<grid, warps * 32, 0, st>>>(a);
-    return cudaGetLastError();
+    return launch_chained(finalize_kernel, grid, warps * 32, 0, st, a);
 }
 
 // constant gradients: same order; grad = S_g / S_w, RMSE scaled by 1/(2 RMSE)
@@ -99,9 +104,7 @@ __global__ void __launch_bounds__(256) grad_finalize_kernel(GradFinalizeArgs a) 
     const double sw = *a.sumw;
     double s = 0.0;
     for (int i = lane; i < a.n_chunks; i += 32) s += (double)a.part[(size_t)p * a.n_chunks + i];
-    double S = 0.0;
-    for (int l = 0; l < 32; ++l) S += __shfl_sync(0xffffffffu, s, l);
-    double f = finish_metric(a.metric, S, sw);
+    double f = finish_metric(a.metric, warp_sum(s), sw);
     const bool bad = (m.status != GP_PROG_OK) || (m.n_consts > GP_MAX_CONSTS);
     const double nan = __longlong_as_double(0x7ff8000000000000LL);
     double scale = 1.0 / sw;
