@@ -31,8 +31,7 @@ slots and marker shapes.
 
 Variants: RPT in {4, 8} x ext (tan, sq, cube, max and min run here too) x XREG
 (columns 0 and 1 held in registers; without it a column read takes the rows
-that were prefetched for it and prefetches the next one's; in the gradient
-variant it is handed back).  A word the loop does not run -- END, the other
+that were prefetched for it and prefetches the next one's).  A word the loop does not run -- END, the other
 extended functions, the trigonometric and exponential arguments outside
 their fast paths, and whatever the variant leaves out -- is handed back to
 the caller's switch with its constant, the address just past it, and the rows
@@ -88,7 +87,7 @@ class Gen:
     def __init__(self, rpt, xreg, ext=False, grad=False):
         self.rpt, self.xreg, self.ext, self.grad = rpt, xreg, ext, grad
         # columns in memory: the next column read is prefetched into XB
-        self.xmem = not xreg and not grad
+        self.xmem = not xreg
         self.np = rpt // 2               # pairs per lane
         p = self.np
         names = ["pa"] + [f"T{i}" for i in range(p)]
@@ -97,22 +96,22 @@ class Gen:
         # the evaluator's words are the dispatch index and a constant, and the
         # stack has a pointer; the gradient's carry slots and markers
         self.plain = not grad
-        names += ["SP", "HW", "HC"] if self.plain else ["HW", "HC", "SB", "NSM1"]
+        names += ["SP", "HW", "HC"] if self.plain else ["HW", "HC", "SB"]
         self.I = "%%w" if self.plain else "%%i"   # the dispatch index
         if self.xmem:
             names += ["XC", "UNIT", "MODE"]
         else:
             names += [f"X{c}_{i}" for c in (0, 1) for i in range(p)]
-        # gradient variant: the lane's tangent slot 0 and the tangent slots
-        names += ["THR", "DB", "KT"]
+        # gradient variant: the lane's tangent slot 0
+        names += ["THR", "DB"]
         at = {n: f"%{k}" for k, n in enumerate(names)}
         self.T = [at[f"T{i}"] for i in range(p)]
         self.HW, self.HC = at["HW"], at["HC"]
         if self.plain:
             self.SP = at["SP"]
         else:
-            self.SB, self.NSM1 = at["SB"], at["NSM1"]
-        self.THR, self.DB, self.KT = at["THR"], at["DB"], at["KT"]
+            self.SB = at["SB"]
+        self.THR, self.DB = at["THR"], at["DB"]
         if self.xmem:
             xb = [at[f"XB{i}"] for i in range(p)]
             self.X, self.XC, self.UNIT, self.MODE = [xb, xb], at["XC"], at["UNIT"], at["MODE"]
@@ -120,6 +119,7 @@ class Gen:
             self.X = [[at[f"X{c}_{i}"] for i in range(p)] for c in (0, 1)]
         self.slot_bytes = (rpt // 4) * 512
         self.lines = []
+        self.resumes = {}     # marked column reads: their index in TD
         # the special-value paths (4 rows per lane only: at 8 the loop's
         # larger code made the evaluator 2.3% slower on Pagie-1 16M x 4096)
         self.special = rpt == 4
@@ -145,8 +145,7 @@ class Gen:
         self.e(f"mov.b64 {dst or self.T[i]}, {{{a}, {b}}};")
 
     def slot_addr(self):
-        self.e("bfe.u32 %%a, %%w, 8, 8;")
-        self.e(f"min.u32 %%a, %%a, {self.NSM1};")
+        self.e("bfe.u32 %%a, %%w, 8, 8;")   # (below the program's depth - 1)
         self.e(f"mad.lo.u32 %%a, %%a, {self.slot_bytes}, {self.SB};")
 
     def slot_load(self):
@@ -608,10 +607,12 @@ class Gen:
         den = lambda i: f"%%U{i}"
         for i in range(self.np):
             # y = 1 / b, q = a y, then q + (a - b q) y
-            self.rcp_pair(den(i), "%%JJ")
-            self.e(f"mul.rn.f32x2 %%JM, {num(i)}, %%JJ;")
+            # (the gradient keeps y for the partial derivatives)
+            y = f"%%A{i}" if self.grad else "%%JJ"
+            self.rcp_pair(den(i), y)
+            self.e(f"mul.rn.f32x2 %%JM, {num(i)}, {y};")
             self.e(f"fma.rn.f32x2 %%R, %%F, %%JM, {num(i)};")  # a - b q
-            self.e("fma.rn.f32x2 %%JM, %%R, %%JJ, %%JM;")
+            self.e(f"fma.rn.f32x2 %%JM, %%R, {y}, %%JM;")
             self.e(f"mov.b64 {{%%s0, %%s1}}, {den(i)};")
             self.e("mov.b64 {%%c0, %%c1}, %%JM;")
             if fix:
@@ -646,12 +647,15 @@ class Gen:
     # scales the tangents of the two ranges.  Marked words the loop does
     # not run, and those whose value body gives up, are handed back as
     # their marker with the address at the marked word.
-    PARTIAL = dict(PC="PONE", PCS="PONE", AC="PONE", AS="PONE", SS="PSUB", SC="PSUB",
-                   RC="PRSUB", MS="PMS", MC="PMC", DS="PDIV", DC="PDIV", RDC="PRDIV",
-                   SQ="PSQ", IV="PIV", LG="PLG", XP="PXP", AB="PAB", NG="PNG",
-                   PX0="PONE", PX1="PONE", PXS0="PONE", PXS1="PONE", AX0="PONE", AX1="PONE",
-                   SX0="PSUB", SX1="PSUB", RX0="PRSUB", RX1="PRSUB", MX0="PMX0", MX1="PMX1",
-                   DX0="PDIV", DX1="PDIV", RDX0="PRDIV", RDX1="PRDIV")
+    # (pushes of a column, additions but for a constant, and subtractions of a
+    # column are never marked: the pre-pass knows that their partials are 1)
+    PARTIAL = dict(PC="ONE", PCS="ONE", AC="ONE", SC="MONE", SS="PSUB", RC="PRSUB", MS="PMS",
+                   MC="PMC", DS="PDIV", DC="PDIV", RDC="PRDIV", SQ="PSQ", IV="PIV", LG="PLG",
+                   XP="PXP", AB="PAB", NG="PNG", RX0="PRSUB", RX1="PRSUB", MX0="PMX0", MX1="PMX1",
+                   DX0="PDIV", DX1="PDIV", RDX0="PRDIV", RDX1="PRDIV",
+                   # columns in memory (the factor of MX is left in U; marked
+                   # divisions are handed back)
+                   RX="PRSUB", MX="PMS")
 
     def partial_labels(self, ent):
         """per dispatch index: the partial-derivative body, or EX where the
@@ -698,7 +702,15 @@ class Gen:
     def partial_code(self, lab):
         e, p = self.e, self.np
         ONES, MONES = "0x3F8000003F800000", "0xBF800000BF800000"
-        if lab in ("PONE", "PSUB", "PRSUB", "PNG"):
+        if lab in ("ONE", "MONE"):
+            # a fresh constant alone (shape 2 always): its tangent starts at +-1
+            one = ONES if lab == "ONE" else MONES
+            e("bfe.u32 %%lo, %%mk, 10, 5;")
+            e(f"mad.lo.u32 %%da, %%lo, 512, {self.DB};")
+            e(f"mov.b64 %%A0, {one};")
+            e("st.shared.v2.b64 [%%da], {%%A0, %%A0};")
+            e("bra.uni N%=;")
+        elif lab in ("PSUB", "PRSUB", "PNG"):
             pt = MONES if lab in ("PRSUB", "PNG") else ONES
             po = MONES if lab == "PSUB" else ONES
             for i in range(p):
@@ -710,10 +722,9 @@ class Gen:
                 e(f"mov.b64 %%PT{i}, {src};")
                 e(f"mov.b64 %%PO{i}, %%TO{i};")
         elif lab in ("PDIV", "PRDIV"):
-            # divisor b in U, quotient v in the rows: r = 1/b, -v r; both 0
-            # where |b| < thr (the protected branch is constant)
+            # divisor b in U, quotient v in the rows, r = 1/b in A: r, -v r;
+            # both 0 where |b| < thr (the protected branch is constant)
             for i in range(p):
-                self.rcp_pair(f"%%U{i}", f"%%A{i}")
                 e(f"mov.b64 %%K0, {MONES};")
                 e(f"mul.rn.f32x2 %%S, {self.T[i]}, %%K0;")
                 e(f"mul.rn.f32x2 %%S, %%S, %%A{i};")
@@ -788,7 +799,7 @@ class Gen:
 
     def tangent_tail(self):
         """dt[k] *= pt for k in [tlo, thi); dt[k] = (fresh ? 1 : dt[k]) * po
-        for k in [olo, ohi); both ranges clamped to the KT slots"""
+        for k in [olo, ohi) (the bucket has a slot for every constant)"""
         e, p = self.e, self.np
         assert p == 2, "one float4 of tangents per (constant, lane): 4 rows"
 
@@ -805,7 +816,6 @@ class Gen:
         def bounds(lo_bit, hi_bit, skip):
             e(f"bfe.u32 %%lo, %%mk, {lo_bit}, 5;")
             e(f"bfe.u32 %%hi, %%mk, {hi_bit}, 5;")
-            e(f"min.u32 %%hi, %%hi, {self.KT};")
             e("setp.ge.u32 %%p, %%lo, %%hi;")
             e(f"@%%p bra {skip}%=;")
             e(f"mad.lo.u32 %%da, %%lo, 512, {self.DB};")
@@ -829,11 +839,9 @@ class Gen:
         self.label("TTE")
         e("mov.u32 %%ret, 0;")
         e("bra.uni N%=;")
-        # shape 1: dt[tlo] *= pt; shape 2: dt[olo] = po (fresh); the index
-        # clamped to the KT slots like the ranges above
+        # shape 1: dt[tlo] *= pt; shape 2: dt[olo] = po (fresh)
         self.label("TT1")
         e("and.b32 %%lo, %%mk, 31;")
-        e(f"min.u32 %%lo, %%lo, {self.KT} - 1;")
         e(f"mad.lo.u32 %%da, %%lo, 512, {self.DB};")
         e("ld.shared.v2.b64 {%%A0, %%A1}, [%%da];")
         for i in range(p):
@@ -843,7 +851,6 @@ class Gen:
         e("bra.uni N%=;")
         self.label("TTF1")
         e("bfe.u32 %%lo, %%mk, 10, 5;")
-        e(f"min.u32 %%lo, %%lo, {self.KT} - 1;")
         e(f"mad.lo.u32 %%da, %%lo, 512, {self.DB};")
         e("st.shared.v2.b64 [%%da], {%%PO0, %%PO1};")
         e("mov.u32 %%ret, 0;")
@@ -874,23 +881,31 @@ class Gen:
     def strided_columns(self):
         e, xb = self.e, self.X[0]
         self.label("NS")
+        step = 4 if self.grad else 128   # (the gradient's rows are always consecutive)
         for i in range(self.np):
-            e(f"ld.global.nc.f32 %%v0, [%%xa+{256 * i}];")
-            e(f"ld.global.nc.f32 %%v1, [%%xa+{256 * i + 128}];")
+            e(f"ld.global.nc.f32 %%v0, [%%xa+{2 * step * i}];")
+            e(f"ld.global.nc.f32 %%v1, [%%xa+{2 * step * i + step}];")
             e(f"mov.b64 {xb[i]}, {{%%v0, %%v1}};")
         e("brx.idx.uni %%dv, TD%=;")
 
-    def xmem_body(self, stem):
+    def xmem_body(self, stem, marked=False):
         """the body of a column-reading word: its operation on XB, then the
         next loads, then (dv) the next word or a division with its operand in
-        U (which, handed back, reads the column again)"""
+        U (which, handed back, reads the column again).  In the gradient's
+        copy for a marked word the partial derivatives follow instead"""
         to = dict(DX=1, RDX=2).get(stem, 0)
-        self.e("@%%pb bra EX%=;")
+        if marked:
+            to = self.resumes.setdefault(stem, 3 + len(self.resumes))
+        self.e(f"@%%pb bra {'MKX' if marked else 'EX'}%=;")
         if stem == "PXS":
             self.spill()
         if stem in ("PX", "PXS"):
             for i in range(self.np):
                 self.e(f"mov.b64 {self.T[i]}, {self.X[0][i]};")
+        elif stem == "MX" and marked:
+            for i in range(self.np):
+                self.e(f"mov.b64 %%U{i}, {self.X[0][i]};")
+            self.pairwise("mul", lambda i: (self.T[i], f"%%U{i}"))
         elif stem in ("AX", "SX", "MX"):
             self.pairwise(dict(AX="add", SX="sub", MX="mul")[stem],
                           lambda i: (self.T[i], self.X[0][i]))
@@ -901,7 +916,10 @@ class Gen:
                 self.e(f"mov.b64 %%U{i}, {self.X[0][i]};")
         self.e(f"mov.u32 %%dv, {to};")
         self.next_column()
-        self.e("bra.uni " + ("N", "DTU", "RDU")[to] + "%=;")
+        if marked:
+            self.label("C" + stem)
+        else:
+            self.e("bra.uni " + ("N", "DTU", "RDU")[to] + "%=;")
 
     # cheap bodies (no range test, a handful of instructions) end with a
     # plain branch to the next word; in the gradient variant the others
@@ -915,13 +933,13 @@ class Gen:
         col = int(name[-1]) if name[-1] in "01" and name not in ("PC",) else None
         return (name[:-1] if col is not None else name), col
 
-    def body(self, name):
+    def body(self, name, marked=False):
         """the value body of one dispatch label; True when it ends with its
         own branch (the divisions go on to the shared division body)"""
         e, p, X = self.e, self.np, self.X
         stem, col = self.stem(name)
         if self.xmem and stem in ("PX", "PXS", "AX", "SX", "MX", "RX", "DX", "RDX"):
-            self.xmem_body(stem)
+            self.xmem_body(stem, marked)
             return True
         if stem == "PX" or stem == "PXS":
             if stem == "PXS":
@@ -1074,7 +1092,7 @@ class Gen:
             e(".reg .pred %%pm, %%pb;")
             e(".reg .b64 %%xa;")
             e(".reg .b32 %%dv;")
-            e("TD%=: .branchtargets N%=, DTU%=, RDU%=;")
+            e("@TD@")
             e(f"setp.ne.u32 %%pm, {self.MODE}, 0;")
             e(f"setp.eq.u32 %%pb, {self.MODE}, 2;")
         e("T%=: .branchtargets " + ", ".join(f"{x}%=" for x in ent) + ";")
@@ -1089,6 +1107,10 @@ class Gen:
             # returns through ret into the partial-derivative body
             tv = [("V" + lab if cheap[i] else "S" + lab) if part[i] != "EX" else "MKX"
                   for i, lab in enumerate(ent)]
+            if self.xmem:
+                # a marked division by or of a column: handed back, after the
+                # loads of the column read next
+                tv = ["MKD" if lab in ("DX", "RDX") else tv[i] for i, lab in enumerate(ent)]
             e("TV%=: .branchtargets " + ", ".join(f"{x}%=" for x in tv) + ";")
             tr = ["N"] + [("EX" if cheap[i] else part[i]) for i in range(64)]
             e("TR%=: .branchtargets " + ", ".join(f"{x}%=" for x in tr) + ";")
@@ -1117,9 +1139,17 @@ class Gen:
                 if self.stem(name)[0] in self.CHEAP and self.PARTIAL.get(name, "EX") != "EX":
                     self.label("V" + name)
                     self.save_rows(self.PARTIAL[name])
-                    self.body(name)
+                    self.body(name, marked=True)
                     self.partial_code(self.PARTIAL[name])
-                    e("brx.idx.uni %%tl, TQ%=;")
+                    if self.PARTIAL[name] not in ("ONE", "MONE"):
+                        e("brx.idx.uni %%tl, TQ%=;")
+            if self.xmem:
+                self.label("MKD")
+                e("@%%pb bra MKX%=;")
+                e(f"mov.u32 %%dv, {self.resumes.setdefault('MKD', 3 + len(self.resumes))};")
+                self.next_column()
+                self.label("CMKD")
+                e("bra.uni MKX%=;")
         # t = t / u with the protection, the divisor pairs in U
         self.label("DTU")
         self.div_body()
@@ -1164,7 +1194,10 @@ class Gen:
         e(f"mov.b32 {self.HW}, %%w;")
         e(f"mov.f32 {self.HC}, %%cf;")
         e("}")
-        return self.lines
+        # where the shared column loads go on
+        on = ["N", "DTU", "RDU"] + ["C" + stem for stem in self.resumes]
+        table = "TD%=: .branchtargets " + ", ".join(x + "%=" for x in on) + ";"
+        return [table if line == "@TD@" else line for line in self.lines]
 
 
 
@@ -1179,14 +1212,13 @@ def function(rpt, xreg, ext=False, grad=False):
     outs = ", ".join(['"+r"(pa)'] + [f'"+l"(t[{i}])' for i in range(p)]
                      + ([f'"+l"(xb[{i}])' for i in range(p)] if xmem else [])
                      + ([] if grad else ['"+r"(sp)']) + ['"=r"(hw)', '"=f"(hc)'])
-    ins = ", ".join((['"r"(sb)', '"n"(NSLOT - 1)'] if grad else [])
+    ins = ", ".join((['"r"(sb)'] if grad else [])
                     + (['"l"(xc)', '"r"(unit)', '"r"(mode)'] if xmem else
                        [f'"l"(x0[{i}])' for i in range(p)] + [f'"l"(x1[{i}])' for i in range(p)])
-                    + ['"f"(kThr)'] + (['"r"(db)', '"n"(KT)'] if grad else []))
+                    + ['"f"(kThr)'] + (['"r"(db)'] if grad else []))
     args = (f"uint64_t (&xb)[{p}], const float *xc, uint32_t unit,\n        uint32_t mode"
             if xmem else f"const uint64_t (&x0)[{p}], const uint64_t (&x1)[{p}]")
-    return (("template <int NSLOT, int KT>\n" if grad else "") +
-            f"__device__ __forceinline__ void {name}(uint32_t &pa, uint64_t (&t)[{p}],\n"
+    return (f"__device__ __forceinline__ void {name}(uint32_t &pa, uint64_t (&t)[{p}],\n"
             f"        {args}, {'uint32_t sb' if grad else 'uint32_t &sp'},\n"
             f"        {'uint32_t db, ' if grad else ''}uint32_t &hw, float &hc) {{\n"
             f"    asm volatile(\n{body}\n"
@@ -1208,8 +1240,7 @@ HEADER = '''// gp_fast.cuh -- the evaluator's indexed-branch fast loop in inline
 // and 1 of the lane's rows in x0 and x1; the _nox ones read columns from
 // memory: xb holds the rows of the column that the program reads next, xc
 // is column 0 at the lane's first row, a word's constant times unit the bytes
-// from there to the next column, mode how the lane's rows lie (in the gradient's
-// variant column reads are handed back).  Every one of the 64
+// from there to the next column, mode how the lane's rows lie.  Every one of the 64
 // values of the six-bit dispatch index has a table entry.  The statement
 // declares no memory clobber: the shared memory it reads and writes (the
 // code buffer, written before a barrier, and the stack, touched elsewhere

@@ -751,8 +751,10 @@ int gp_const_grad(const gp_node *progs, const int32_t *offsets, int n_progs, con
     // one launch per bucket (constants, stack depth) of the compiled programs
     const bool vec = aligned16(X) && aligned16(y) && (!w || aligned16(w)) && (n_rows % 4 == 0) &&
                      (chunk % 4 == 0);
-    for (int bucket = 0; bucket < kGradBuckets; ++bucket) {
+    for (int bucket = kGradBuckets - 1; bucket >= 0; --bucket) {
         GradArgs ga{};
+        ga.follows = bucket < kGradBuckets - 1;
+        ga.x_unit = x_unit(n_feat, n_rows, vec);
         ga.code = W.code;
         ga.meta = W.meta;
         ga.order = W.order;
@@ -786,6 +788,7 @@ int gp_const_grad(const gp_node *progs, const int32_t *offsets, int n_progs, con
         // compiled stacks of up to kSmallDepth values: the 7-slot instance
         ea.cls = kClassShallow8;
         ea.qcls = kGradBuckets + 1;
+        ea.follows = 1;
         ea.X = X;
         ea.ld = n_rows;
         ea.n_rows = n_rows;

@@ -19,12 +19,28 @@
 // A block takes one (program, row chunk) item; its warps run the program
 // over their own sub-tiles of 128 rows (4 per lane) with the evaluator's
 // fast loop (the same FP32 operations, so the fitness equals
-// gp_evaluate's), which hands each marked word back to grad_word.  The
-// loss derivative per row times the tangents gives each constant's share.
-// Programs are bucketed by their number of constants (the tangent slots
-// per row) and stack depth, one launch per bucket.  Per-lane sums are FP32
-// (the loss Kahan-compensated), warp sums fixed-order, chunk sums FP64 in
-// order (gp_reduce.cu).
+// gp_evaluate's) in its gradient variant, which hands the words it does not
+// run back to grad_word.  The loss derivative per row times the tangents
+// gives each constant's share.  Programs are bucketed by what their stack and
+// constants need of shared memory (grad_bucket), one launch per bucket.
+// Per-lane sums are FP32 (the loss Kahan-compensated), warp sums
+// fixed-order, chunk sums FP64 in a fixed order (gp_reduce.cu).
+//
+// Bound by instruction issue and by fetching 130 KB of code a word here and a
+// word there (61% of the issue slots taken at 32 warps per SM, 1 cycle in 5
+// of a warp waiting for instructions), hence as many warps per SM as 64
+// registers allow: with all of a Pagie-1 population's programs at 16
+// warps the gradient takes 10.9 ms, at 24 warps 9.3 and as it is 8.3 ms (2048
+// programs, depth 4-10, 262144 rows).  What the packed shared memory, column
+// reads in the loop (with more than two columns; the next column's rows are
+// prefetched as in the evaluator) and launches that overlap at their
+// edges gave: those 2048 programs 9.18 -> 8.27 ms; 1024 programs, depth 3-7, 28
+// columns x 200000 rows 1.17 -> 1.10 ms; 512 programs x 1000 rows 94 -> 60 us.
+// The rows of a lane, the order of its sums and which words run where are part
+// of the results: a gradient that cancels out is rounding alone, and Adam's
+// first steps divide it by its own size.
+#include <atomic>
+
 #include "gp_internal.cuh"
 #include "gp_interp.cuh"
 
@@ -119,44 +135,70 @@ __device__ __forceinline__ void tan_store(uint32_t a, float4 d) {
 // the constants under each (kGradMark).  Four rows per lane; the stack
 // slot of this lane's rows is one float4 (sb + slot * 512 bytes), the
 // tangent of constant k one float4 at db + k * 512.
-template <int NSLOT, int KT, bool XREG>
-__device__ __forceinline__ void grad_word(uint32_t w, float c, uint32_t mk, float (&t)[4],
-                                          const float (&x0)[4], const float (&x1)[4],
-                                          const float *__restrict__ X, int64_t ld, int64_t r0,
-                                          int64_t re, bool vec, uint32_t sb, uint32_t db) {
+// The gradient's four rows of a lane as pairs: always consecutive, so that
+// which rows a lane's sums hold does not depend on the alignment (the
+// gradient of a constant that cancels out is rounding alone, and an Adam
+// step divides it by its own size); with vec 16-byte loads, else 4-byte ones,
+// rows past p[last] 0.
+__device__ __forceinline__ void load_quad(uint64_t (&v)[2], const float *__restrict__ p, bool vec,
+                                          int last) {
+    if (vec) {
+        const ulonglong2 f = __ldg(reinterpret_cast<const ulonglong2 *>(p));
+        v[0] = f.x;
+        v[1] = f.y;
+    } else {
+        float f[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) f[j] = (j <= last) ? __ldg(p + j) : 0.0f;
+        v[0] = pack2(f[0], f[1]);
+        v[1] = pack2(f[2], f[3]);
+    }
+}
+
+template <bool XREG>
+__device__ __forceinline__ void grad_word(uint32_t w, float c, uint32_t mk, uint64_t (&tp)[2],
+                                          const uint64_t (&x0)[2], const uint64_t (&x1)[2],
+                                          const float *__restrict__ xc, int64_t ld, bool packed,
+                                          int last, uint32_t sb, uint32_t db) {
     constexpr int R = 4;
-    const uint32_t op = w & 31u;
+    float t[R];
+    unpack2(tp[0], t[0], t[1]);
+    unpack2(tp[1], t[2], t[3]);
+    const uint32_t opc = w & 31u;
     const uint32_t fn = (w >> 16) & 7u;
-    const uint32_t sa = sb + min((w >> 8) & 255u, (uint32_t)NSLOT - 1u) * 32u * 16u;
+    const uint32_t sa = sb + ((w >> 8) & 255u) * 512u;
     // the other operand: a stack slot (S forms, EXT2), a column (X forms,
     // PUSH_X), else the word's constant
     float o[R];
-    const bool from_slot = (op >= OP_ADD_S && op <= OP_DIV_S) || op == OP_EXT2;
-    const bool from_col = op == OP_PUSH_X || op == OP_PUSH_X_SP ||
-                          (op >= OP_ADD_X && op <= OP_RDIV_X && ((op - OP_ADD_X) & 1u) == 0u);
+    const bool from_slot = (opc >= OP_ADD_S && opc <= OP_DIV_S) || opc == OP_EXT2;
+    const bool from_col = opc == OP_PUSH_X || opc == OP_PUSH_X_SP ||
+                          (opc >= OP_ADD_X && opc <= OP_RDIV_X && ((opc - OP_ADD_X) & 1u) == 0u);
     if (from_slot) {
         asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
                      : "=f"(o[0]), "=f"(o[1]), "=f"(o[2]), "=f"(o[3])
                      : "r"(sa));
     } else if (from_col) {
         const int feat = (int)(w >> 16);
+        uint64_t op[2];
         if (XREG) {
-#pragma unroll
-            for (int j = 0; j < R; ++j) o[j] = feat ? x1[j] : x0[j];
+            op[0] = feat ? x1[0] : x0[0];
+            op[1] = feat ? x1[1] : x0[1];
         } else {
-            load_rows<R>(o, X + (int64_t)feat * ld, r0, re, vec);
+            load_quad(op, xc + (int64_t)feat * ld, packed, last);
         }
+        unpack2(op[0], o[0], o[1]);
+        unpack2(op[1], o[2], o[3]);
     } else {
 #pragma unroll
         for (int j = 0; j < R; ++j) o[j] = c;
     }
-    if (op == OP_PUSH_X_SP || op == OP_PUSH_C_SP)
+    if (opc == OP_PUSH_X_SP || opc == OP_PUSH_C_SP)
         asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(sa), "f"(t[0]), "f"(t[1]),
                      "f"(t[2]), "f"(t[3])
                      : "memory");
     float v[R];
 #define GP_ROWS(stmt) _Pragma("unroll") for (int j = 0; j < R; ++j) { stmt; }
-    switch (op) {
+    switch (opc) {
     case OP_ADD_S: case OP_ADD_X: case OP_ADD_C: GP_ROWS(v[j] = f_add(t[j], o[j])) break;
     case OP_SUB_S: case OP_SUB_X: case OP_SUB_C: GP_ROWS(v[j] = f_sub(t[j], o[j])) break;
     case OP_RSUB_X: case OP_RSUB_C: GP_ROWS(v[j] = f_sub(o[j], t[j])) break;
@@ -168,7 +210,7 @@ __device__ __forceinline__ void grad_word(uint32_t w, float c, uint32_t mk, floa
     case OP_EXP: GP_ROWS(v[j] = f_exp(t[j])) break;
     case OP_SIN: case OP_COS: case OP_TAN:
         GP_ROWS(v[j] = t[j])
-        trig_rows<R>(v, (int)(op - OP_SIN));
+        trig_rows<R>(v, (int)(opc - OP_SIN));
         break;
     case OP_ABS: GP_ROWS(v[j] = f_abs(t[j])) break;
     case OP_NEG: GP_ROWS(v[j] = f_neg(t[j])) break;
@@ -183,7 +225,7 @@ __device__ __forceinline__ void grad_word(uint32_t w, float c, uint32_t mk, floa
     if (mk != 0u) {
         float pt[R], po[R];
         GP_ROWS(pt[j] = 1.0f; po[j] = 1.0f)
-        switch (op) {
+        switch (opc) {
         case OP_SUB_S: case OP_SUB_X: case OP_SUB_C: GP_ROWS(po[j] = -1.0f) break;
         case OP_RSUB_X: case OP_RSUB_C: GP_ROWS(pt[j] = -1.0f) break;
         case OP_MUL_S: case OP_MUL_X: case OP_MUL_C: GP_ROWS(pt[j] = o[j]; po[j] = t[j]) break;
@@ -204,12 +246,12 @@ __device__ __forceinline__ void grad_word(uint32_t w, float c, uint32_t mk, floa
             break;
         case OP_SQRT: case OP_LOG: case OP_EXP: case OP_SIN: case OP_COS: case OP_TAN:
         case OP_ABS: case OP_NEG: case OP_INV: case OP_EXT1:
-            GP_ROWS(pt[j] = d_unary(op, fn, t[j], v[j]))
+            GP_ROWS(pt[j] = d_unary(opc, fn, t[j], v[j]))
             break;
         default: break;  // add and the pushes: both partials 1
         }
-        const int tlo = (int)(mk & 31u), thi = min((int)((mk >> 5) & 31u), KT);
-        const int olo = (int)((mk >> 10) & 31u), ohi = min((int)((mk >> 15) & 31u), KT);
+        const int tlo = (int)(mk & 31u), thi = (int)((mk >> 5) & 31u);
+        const int olo = (int)((mk >> 10) & 31u), ohi = (int)((mk >> 15) & 31u);
         const bool fresh = ((mk >> 20) & 1u) != 0u;
         for (int k = tlo; k < thi; ++k) {
             float4 d = tan_load(db + (uint32_t)k * 512u);
@@ -228,7 +270,8 @@ __device__ __forceinline__ void grad_word(uint32_t w, float c, uint32_t mk, floa
             tan_store(db + (uint32_t)k * 512u, d);
         }
     }
-    GP_ROWS(t[j] = v[j])
+    tp[0] = pack2(v[0], v[1]);
+    tp[1] = pack2(v[2], v[3]);
 #undef GP_ROWS
 }
 
@@ -236,28 +279,21 @@ __device__ __forceinline__ void grad_word(uint32_t w, float c, uint32_t mk, floa
 // gradient variant of the fast loop runs the words it can, marked ones
 // with their tangent updates, and each word it hands back -- a marker with
 // the word after it, or a word it does not run -- runs in grad_word.
-// Returns the prediction in t and leaves each constant's tangent
-// d(prediction)/d(c_k) at db + k * 512.
-template <int NSLOT, int KT, bool XREG>
-__device__ __forceinline__ void grad_run(float (&t)[4], const uint2 *cbuf, const float (&x0)[4],
-                                         const float (&x1)[4], const float *__restrict__ X,
-                                         int64_t ld, int64_t r0, int64_t re, bool vec,
-                                         float4 *stk, uint32_t db) {
-#pragma unroll
-    for (int j = 0; j < 4; ++j) t[j] = 0.0f;
+// Returns the prediction in tp and leaves each constant's tangent
+// d(prediction)/d(c_k) at db + k * 512.  The columns as in interpret().
+template <bool XREG>
+__device__ __forceinline__ void grad_run(uint64_t (&tp)[2], const uint2 *cbuf, uint64_t (&x0)[2],
+                                         const uint64_t (&x1)[2], const float *__restrict__ xc,
+                                         int64_t ld, uint32_t unit, uint32_t mode, bool packed, int last,
+                                         uint32_t sb, uint32_t db) {
+    asm volatile("" : "=l"(tp[0]), "=l"(tp[1]));  // (the first word is a push)
     uint32_t pa = (uint32_t)__cvta_generic_to_shared(cbuf);
-    const uint32_t sb = (uint32_t)__cvta_generic_to_shared(stk);
-    const uint64_t x0p[2] = {pack2(x0[0], x0[1]), pack2(x0[2], x0[3])};
-    const uint64_t x1p[2] = {pack2(x1[0], x1[1]), pack2(x1[2], x1[3])};
 #pragma unroll 1
     for (;;) {
-        uint64_t tp[2] = {pack2(t[0], t[1]), pack2(t[2], t[3])};
         uint32_t hw;
         float hc;
-        if constexpr (XREG) fast_r4_divs_x_grad<NSLOT, KT>(pa, tp, x0p, x1p, sb, db, hw, hc);
-        else fast_r4_divs_nox_grad<NSLOT, KT>(pa, tp, x0p, x1p, sb, db, hw, hc);
-        unpack2(tp[0], t[0], t[1]);
-        unpack2(tp[1], t[2], t[3]);
+        if constexpr (XREG) fast_r4_divs_x_grad(pa, tp, x0, x1, sb, db, hw, hc);
+        else fast_r4_divs_nox_grad(pa, tp, x0, xc, unit, mode, sb, db, hw, hc);
         uint32_t w = __shfl_sync(0xffffffffu, hw, 0);
         float c = hc;
         uint32_t mk = 0u;
@@ -270,188 +306,254 @@ __device__ __forceinline__ void grad_run(float (&t)[4], const uint2 *cbuf, const
             c = __uint_as_float(c2);
         }
         if ((w & 31u) == OP_END) break;
-        grad_word<NSLOT, KT, XREG>(w, c, mk, t, x0, x1, X, ld, r0, re, vec, sb, db);
+        grad_word<XREG>(w, c, mk, tp, x0, x1, xc, ld, packed, last, sb, db);
     }
 }
 
 // shared memory of one block: the program's words (through the buffer's
-// end OP_END), then per warp the value stack [NSLOT][32 lanes] and the
-// tangents [KT][32 lanes], one float4 (four rows) per entry
-template <int WARPS, int NSLOT, int KT>
+// end OP_END), then per warp UNITS x 128 bytes: the value stack [depth - 1][32
+// lanes] and the tangents [constants][32 lanes], one float4 (four rows) per
+// entry, and (without GREG) the constants' sums [constants][32 lanes]
+template <int WARPS, int UNITS>
 constexpr size_t grad_smem_bytes() {
-    return (size_t)(kGradCodeStride + 2) * sizeof(uint2) +
-           (size_t)WARPS * (NSLOT + KT) * 32 * sizeof(float4);
+    return (size_t)(kGradCodeStride + 2) * sizeof(uint2) + (size_t)WARPS * UNITS * 128;
 }
 
-template <int WARPS, int NSLOT, int KT, int MINB, bool XREG>
+// GREG: the constants' sums in registers (unrolled over GP_MAX_CONSTS), else in
+// shared memory, so that a bucket's limit need not be a number of constants
+template <int WARPS, int UNITS, int MINB, bool GREG, bool XREG>
 __global__ void __launch_bounds__(WARPS * 32, MINB) grad_kernel(const GradArgs a) {
-    constexpr int R = 4;
+    constexpr int R = 4, KT = GREG ? GP_MAX_CONSTS : 1;
+    static_assert(GP_MAX_CONSTS <= 32 && WARPS >= 2, "one thread per constant in warp 1");
     static_assert((kGradCodeStride + 2) * sizeof(uint2) % 16 == 0, "stack alignment");
     extern __shared__ float4 smem_grad[];
     uint2 *cbuf = reinterpret_cast<uint2 *>(smem_grad);
-    float4 *stack_all = smem_grad + (kGradCodeStride + 2) * sizeof(uint2) / 16;
-    float4 *tan_all = stack_all + (size_t)WARPS * NSLOT * 32;
+    float4 *const mine_all = smem_grad + (kGradCodeStride + 2) * sizeof(uint2) / 16;
     __shared__ float wsum[WARPS];
     __shared__ float wgrad[WARPS][GP_MAX_CONSTS];
-    __shared__ unsigned long long s_item;
+    __shared__ int4 s_item[2];  // chunk (-1: the queue is empty), program, words, constants | stack slots << 8 (-1: none to run)
+    __shared__ unsigned long long s_total;
+    __shared__ int s_begin, s_n;
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
-    float4 *stk = stack_all + (size_t)warp * NSLOT * 32 + lane;
-    const uint32_t db = (uint32_t)__cvta_generic_to_shared(tan_all + (size_t)warp * KT * 32 + lane);
-    int cls_begin = 0;
-    for (int b = 0; b < a.bucket; ++b) cls_begin += a.class_count[b];
-    const int n_cls = a.class_count[a.bucket];
-    const unsigned long long total = (unsigned long long)n_cls * (unsigned long long)a.n_chunks;
-    const bool vec = a.vec_ok != 0;
-    const bool two_feat = XREG && a.n_feat == 2;
-
-    for (unsigned long long it = 0; it <= total; ++it) {
-        if (threadIdx.x == 0) s_item = atomicAdd(a.counter + a.bucket, 1ULL);
-        __syncthreads();
-        const unsigned long long item = s_item;
-        if (item >= total || it == total) {  // the cap cannot trigger: one item per pass
-            if (it == total && threadIdx.x == 0) atomicOr(a.dev_status, GP_DEV_QUEUE_CAP);
-            break;
-        }
-        const int chunk = (int)(item / (unsigned long long)n_cls);
-        const int rank = (int)(item - (unsigned long long)chunk * n_cls);
-        const int p = a.order[cls_begin + rank];
-        const ProgMeta m = a.meta[p];
-        float *gp = a.gpart + ((size_t)p * a.n_chunks + chunk) * GP_MAX_CONSTS;
-        if (m.status != GP_PROG_OK || m.n_consts > KT || m.n_ins > kGradCodeStride) {
-            if (threadIdx.x == 0) {
-                a.part[(size_t)p * a.n_chunks + chunk] = __int_as_float(0x7fc00000);
+    float4 *const mine = mine_all + (size_t)warp * UNITS * 8;  // the warp's units
+    const uint32_t sb = (uint32_t)__cvta_generic_to_shared(mine + lane);
+    // thread 0 takes the next item while the block works on this one (as in
+    // the evaluator)
+    auto take = [&](unsigned long long item, int slot) {
+        int4 it = make_int4(-1, 0, 0, 0);
+        if (item < s_total) {
+            const uint32_t n = (uint32_t)s_n;
+            it.x = (int)((s_total >> 32) ? item / n : (uint32_t)item / n);
+            it.y = a.order[s_begin + (int)(item - (unsigned long long)it.x * n)];
+            const ProgMeta m = a.meta[it.y];
+            it.z = m.n_ins;
+            it.w = m.n_consts | (m.depth - 1) << 8;
+            if (m.status != GP_PROG_OK || m.n_consts > GP_MAX_CONSTS || m.n_ins > kGradCodeStride) {
+                it.w = -1;
                 if (m.n_consts > GP_MAX_CONSTS) atomicOr(a.dev_status, GP_DEV_TOO_MANY_CONSTS);
             }
-            if (threadIdx.x < GP_MAX_CONSTS) gp[threadIdx.x] = __int_as_float(0x7fc00000);
-            __syncthreads();  // s_item is rewritten at the top
-            continue;
         }
-        const int n_ins = m.n_ins;
-        const uint2 *src = a.code + (size_t)p * kGradCodeStride;
-        for (int i = threadIdx.x; i < kGradCodeStride + 2; i += WARPS * 32)
-            cbuf[i] = (i < n_ins) ? src[i] : make_uint2(make_ins(OP_END, 0, 0), 0u);
-        __syncthreads();
+        s_item[slot] = it;
+    };
+    if (a.follows) __threadfence();  // see eval_kernel
+    else griddep_wait();
+    griddep_launch();
+    if (threadIdx.x == 0) {
+        int begin = 0;
+        for (int b = 0; b < a.bucket; ++b) begin += a.class_count[b];
+        s_begin = begin;
+        s_n = a.class_count[a.bucket];
+        s_total = (unsigned long long)s_n * (unsigned long long)a.n_chunks;
+        take(blockIdx.x, 0);  // the counter hands out the items from gridDim.x on
+    }
+    __syncthreads();
 
-        const int nc = m.n_consts;
-        const int64_t rb = (int64_t)chunk * a.chunk_rows;
-        const int64_t re = min(a.n_rows, rb + a.chunk_rows);
-        const int n_in = (int)(re - rb);
+    for (int cur = 0;; cur ^= 1) {
+        // (read again where it is needed: held across the interpreter the
+        // item's numbers would spill)
+        const volatile int4 *it = &s_item[cur];
+        if (it->x < 0) break;
+        const bool ok = it->w >= 0;
+        if (ok) {
+            const uint2 *src = a.code + (size_t)it->y * kGradCodeStride;
+            const int n_ins = it->z;
+            for (int i = threadIdx.x; i < n_ins; i += WARPS * 32) {
+                uint2 v = src[i];
+                // a column read's constant: the next column read, as an offset
+                if (!XREG && (kColumnOps >> (v.x & 31u) & 1u))
+                    v.y = (uint32_t)((uint64_t)v.y * (uint64_t)(a.x_unit == 16 ? a.ld >> 2 : a.ld));
+                cbuf[i] = v;
+            }
+        }
+        __syncthreads();  // the words are there
+        unsigned long long next = 0;
+        if (threadIdx.x == 0) next = gridDim.x + atomicAdd(a.counter + a.bucket, 1ULL);
+
+        const int n_in = (int)min(a.n_rows - (int64_t)it->x * a.chunk_rows, a.chunk_rows);
+        // the tangents lie past the stack, the sums past the tangents
+        const uint32_t db = sb + (uint32_t)(it->w >> 8) * 512u;
+        float *const gm = reinterpret_cast<float *>(mine + ((it->w >> 8) + (it->w & 255)) * 32) + lane;
         float gs[KT];
 #pragma unroll
         for (int k = 0; k < KT; ++k) gs[k] = 0.0f;
+        if (!GREG && ok)
+            for (int k = 0; k < (it->w & 255); ++k) gm[k * 32] = 0.0f;
         float ls = 0.0f, lc = 0.0f;
-        for (int base = warp * 32 * R; base < n_in; base += WARPS * 32 * R) {
+        uint64_t x0[2], x1[2];
+        auto first_column = [&](int base) {
+            const bool pk = __all_sync(0xffffffffu, base + 32 * R <= n_in) && a.vec_ok;
             const int o = base + lane * R;
-            const bool full = __all_sync(0xffffffffu, o + R <= n_in);
-            const int nv = full ? R : n_in - o;
-            float x0[R], x1[R];
-            if (XREG) {
-                load_chunk_rows<R>(x0, a.X + (rb + o), full && vec, nv);
-                if (two_feat) load_chunk_rows<R>(x1, a.X + (a.ld + rb + o), full && vec, nv);
-                else {
-#pragma unroll
-                    for (int j = 0; j < R; ++j) x1[j] = x0[j];
+            const int64_t feat = cbuf[it->z - 1].y;
+            load_quad(x0, a.X + (feat * a.ld + (int64_t)it->x * a.chunk_rows + o), pk, n_in - 1 - o);
+        };
+        if (!XREG && ok && warp * 32 * R < n_in) first_column(warp * 32 * R);
+        for (int base = warp * 32 * R; base < n_in && ok; base += WARPS * 32 * R) {
+            const bool whole = __all_sync(0xffffffffu, base + 32 * R <= n_in);
+            const bool packed = whole && a.vec_ok;
+            const int o = base + lane * R;
+            const int last = n_in - 1 - o;
+            uint64_t t[2];
+            {
+                const float *xr = a.X + ((int64_t)it->x * a.chunk_rows + o);
+                if (XREG) {
+                    load_quad(x0, xr, packed, last);
+                    load_quad(x1, xr + (a.n_feat == 2 ? a.ld : 0), packed, last);
                 }
-            } else {
-#pragma unroll
-                for (int j = 0; j < R; ++j) x0[j] = x1[j] = 0.0f;
+                const uint32_t mode = a.x_unit == 0 || !whole ? 2u : packed ? 0u : 1u;
+                grad_run<XREG>(t, cbuf, x0, x1, xr, a.ld, (uint32_t)a.x_unit, mode, packed,
+                                          last, sb, db);
             }
-            float t[R];
-            grad_run<NSLOT, KT, XREG>(t, cbuf, x0, x1, a.X, a.ld, rb + o, re, vec, stk, db);
+            const int64_t r = (int64_t)it->x * a.chunk_rows + o;
+            const int nc = it->w & 255;
+            if (!XREG && base + WARPS * 32 * R < n_in) first_column(base + WARPS * 32 * R);
             // the loss and its derivative per row
-            float yv[R], wv[R];
-            load_chunk_rows<R>(yv, a.y + (rb + o), full && vec, nv);
-            if (a.w) load_chunk_rows<R>(wv, a.w + (rb + o), full && vec, nv);
-            else {
+            const int nv = whole ? R : last + 1;  // rows of the lane that count
+            uint64_t yv[2], wv[2];
+            load_quad(yv, a.y + r, packed, last);
+            if (a.w) load_quad(wv, a.w + r, packed, last);
+            kahan_add(ls, lc, loss_sum<R>(a.metric, t, yv, wv, a.w != nullptr, whole, nv));
+            float at[R];
+            {
+                float tv[R], yy[R], ww[R];
 #pragma unroll
-                for (int j = 0; j < R; ++j) wv[j] = 1.0f;
-            }
-            float e = 0.0f, at[R];
-#pragma unroll
-            for (int j = 0; j < R; ++j) {
-                const bool in = j < nv;
-                float l = row_loss(a.metric, t[j], yv[j]);
-                if (a.w) l = __fmul_rn(wv[j], l);
-                e = in ? __fadd_rn(e, l) : e;
-                at[j] = in ? __fmul_rn(wv[j], g_dloss(a.metric, t[j], yv[j])) : 0.0f;
-            }
-            kahan_add(ls, lc, e);
-            // each constant's share: the rows' loss derivatives times its tangents
-#pragma unroll
-            for (int k = 0; k < KT; ++k) {
-                if (k < nc) {
-                    const float4 d = tan_load(db + (uint32_t)k * 512u);
-                    const float dd[R] = {d.x, d.y, d.z, d.w};
-                    float s = 0.0f;
-#pragma unroll
-                    for (int j = 0; j < R; ++j) s = (j < nv) ? __fadd_rn(s, __fmul_rn(at[j], dd[j])) : s;
-                    gs[k] = __fadd_rn(gs[k], s);
+                for (int i = 0; i < 2; ++i) {
+                    unpack2(t[i], tv[2 * i], tv[2 * i + 1]);
+                    unpack2(yv[i], yy[2 * i], yy[2 * i + 1]);
+                    if (a.w) unpack2(wv[i], ww[2 * i], ww[2 * i + 1]);
                 }
+                if (a.metric == GP_MAE) {
+#pragma unroll
+                    for (int j = 0; j < R; ++j) at[j] = g_dloss(GP_MAE, tv[j], yy[j]);
+                } else if (a.metric == GP_LOGLOSS) {
+#pragma unroll
+                    for (int j = 0; j < R; ++j) at[j] = g_dloss(GP_LOGLOSS, tv[j], yy[j]);
+                } else {
+#pragma unroll
+                    for (int j = 0; j < R; ++j) at[j] = g_dloss(GP_MSE, tv[j], yy[j]);
+                }
+                if (a.w) {
+#pragma unroll
+                    for (int j = 0; j < R; ++j) at[j] = __fmul_rn(ww[j], at[j]);
+                }
+            }
+            // each constant's share: the rows' loss derivatives times its
+            // tangents (rows past the end do not count, whatever they hold)
+            auto share = [&](const float4 d) {
+                float q = __fmul_rn(at[0], d.x);
+                if (whole) {
+                    q = __fadd_rn(q, __fmul_rn(at[1], d.y));
+                    q = __fadd_rn(q, __fmul_rn(at[2], d.z));
+                    return __fadd_rn(q, __fmul_rn(at[3], d.w));
+                }
+                q = nv > 0 ? q : 0.0f;
+                q = nv > 1 ? __fadd_rn(q, __fmul_rn(at[1], d.y)) : q;
+                q = nv > 2 ? __fadd_rn(q, __fmul_rn(at[2], d.z)) : q;
+                return nv > 3 ? __fadd_rn(q, __fmul_rn(at[3], d.w)) : q;
+            };
+            if (GREG) {
+#pragma unroll
+                for (int k = 0; k < KT; ++k)
+                    if (k < nc) gs[k] = __fadd_rn(gs[k], share(tan_load(db + (uint32_t)k * 512u)));
+            } else {
+#pragma unroll 1
+                for (int k = 0; k < nc; ++k)
+                    gm[k * 32] = __fadd_rn(gm[k * 32], share(tan_load(db + (uint32_t)k * 512u)));
             }
         }
+        if (threadIdx.x == 0) take(next, cur ^ 1);
+        const int nc = ok ? it->w & 255 : 0;
         // fixed butterfly per warp, then the warps in order
         float lv = __fsub_rn(ls, lc);
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) lv = __fadd_rn(lv, __shfl_xor_sync(0xffffffffu, lv, off));
         if (lane == 0) wsum[warp] = lv;
+        auto total = [&](int k, float v) {
 #pragma unroll
-        for (int k = 0; k < GP_MAX_CONSTS; ++k) {
-            float v = 0.0f;
-            if (k < KT) {
-                v = gs[k < KT ? k : 0];
-#pragma unroll
-                for (int off = 16; off > 0; off >>= 1)
-                    v = __fadd_rn(v, __shfl_xor_sync(0xffffffffu, v, off));
-            }
+            for (int off = 16; off > 0; off >>= 1) v = __fadd_rn(v, __shfl_xor_sync(0xffffffffu, v, off));
             if (lane == 0) wgrad[warp][k] = v;
+        };
+        if (GREG) {
+#pragma unroll
+            for (int k = 0; k < KT; ++k)
+                if (k < nc) total(k, gs[k]);
+        } else {
+            for (int k = 0; k < nc; ++k) total(k, gm[k * 32]);
         }
-        __syncthreads();
+        __syncthreads();  // the sums and the next item complete; everyone is done with cbuf
         if (threadIdx.x == 0) {
             float v = 0.0f;
             for (int q = 0; q < WARPS; ++q) v = __fadd_rn(v, wsum[q]);
-            a.part[(size_t)p * a.n_chunks + chunk] = v;
+            a.part[(size_t)it->y * a.n_chunks + it->x] = ok ? v : __int_as_float(0x7fc00000);
         } else if (threadIdx.x >= 32 && threadIdx.x < 32 + GP_MAX_CONSTS) {
             const int k = threadIdx.x - 32;
             float v = 0.0f;
-            for (int q = 0; q < WARPS; ++q) v = __fadd_rn(v, wgrad[q][k]);
-            gp[k] = v;
+            if (k < nc)
+                for (int q = 0; q < WARPS; ++q) v = __fadd_rn(v, wgrad[q][k]);
+            a.gpart[((size_t)it->y * a.n_chunks + it->x) * GP_MAX_CONSTS + k] =
+                ok ? v : __int_as_float(0x7fc00000);
         }
-        __syncthreads();  // wsum, wgrad, cbuf and s_item are reused
     }
+    if (a.follows && blockIdx.x == 0) griddep_wait();  // see eval_kernel
 }
 
-template <int WARPS, int NSLOT, int KT, int MINB, bool XREG>
+template <int WARPS, int UNITS, int MINB, bool GREG, bool XREG>
 cudaError_t launch_grad_t(const GradArgs &a, int sms, cudaStream_t st, int *occ_out) {
-    constexpr size_t smem = grad_smem_bytes<WARPS, NSLOT, KT>();
-    auto k = grad_kernel<WARPS, NSLOT, KT, MINB, XREG>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    static std::atomic<int> known[kMaxDevices];  // resident blocks, asked for once per device
+    constexpr size_t smem = grad_smem_bytes<WARPS, UNITS>();
+    auto k = grad_kernel<WARPS, UNITS, MINB, GREG, XREG>;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    int occ = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, WARPS * 32, smem);
-    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+    int occ = known[dev].load(std::memory_order_acquire);
+    if (occ == 0) {
+        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, WARPS * 32, smem);
+        if (e != cudaSuccess) return e;
+        occ = occ > 0 ? occ : 1;
+        known[dev].store(occ, std::memory_order_release);
+    }
     if (occ_out) {
         *occ_out = occ;
         return cudaSuccess;
     }
-    k<<<sms * (occ > 0 ? occ : 1), WARPS * 32, smem, st>>>(a);
-    return cudaGetLastError();
+    return launch_chained(k, sms * occ, WARPS * 32, smem, st, a);
 }
 
-// Four rows per lane.  Buckets 0-2 (compiled depth <= 8, 7 stack slots):
-// 8 warps with 4, 8 or 16 tangent slots per row, 4, 3 or 2 blocks per SM
-// (shared memory allows no more); bucket 3 (deeper stacks): 4 warps, 19
-// slots, 3 blocks.
-#define GP_GRAD_LAUNCH(W, S, K, M) \
-    (xreg ? launch_grad_t<W, S, K, M, true>(a, sms, st, occ) \
-          : launch_grad_t<W, S, K, M, false>(a, sms, st, occ))
+// Four rows per lane, 8 warps and 4, 3 or 2 blocks per SM by what the bucket's
+// programs need of shared memory (grad_bucket); bucket 3: 4 warps, 3 blocks.
+#define GP_GRAD_LAUNCH(W, U, M, G) \
+    (xreg ? launch_grad_t<W, U, M, G, true>(a, sms, st, occ) \
+          : launch_grad_t<W, U, M, G, false>(a, sms, st, occ))
 cudaError_t launch_grad(const GradArgs &a, int sms, cudaStream_t st, int *occ) {
     const bool xreg = a.n_feat <= 2;
     switch (a.bucket) {
-    case 0: return GP_GRAD_LAUNCH(8, kSmallDepth - 1, kGradTan0, 4);
-    case 1: return GP_GRAD_LAUNCH(8, kSmallDepth - 1, kGradTan1, 3);
-    case 2: return GP_GRAD_LAUNCH(8, kSmallDepth - 1, GP_MAX_CONSTS, 2);
-    default: return GP_GRAD_LAUNCH(4, kDeepSlots, GP_MAX_CONSTS, 3);
+    case 0: return GP_GRAD_LAUNCH(8, kGradUnits0, 4, false);
+    case 1: return GP_GRAD_LAUNCH(8, kGradUnits1, 3, false);
+    case 2: return GP_GRAD_LAUNCH(8, grad_units(GP_MAX_CONSTS, kSmallDepth), 2, false);
+    default: return GP_GRAD_LAUNCH(4, 4 * (kDeepSlots + GP_MAX_CONSTS), 3, true);
     }
 }
 #undef GP_GRAD_LAUNCH

@@ -140,20 +140,29 @@ __host__ __device__ inline int prog_class(int depth, int ext) {
     return depth > kShallowDepth ? kClassShallow8 : kClassShallow;
 }
 
-// Buckets of the constant gradient, one launch each: the tangents of a
-// warp's rows take kGradTan0 (bucket 0), kGradTan1 (bucket 1) or
-// GP_MAX_CONSTS (buckets 2, 3) shared-memory slots per row, the value
-// stack 7 (buckets 0-2) or 19 (bucket 3); fewer tangent slots leave room
-// for more resident warps.
+// Buckets of the constant gradient, one launch each.  A warp's shared
+// memory holds, in units of 128 bytes, the value stack (4 units a slot), the
+// tangents (4 a constant) and the constants' sums (1 a constant) of the program
+// at hand, packed; what a program needs of it decides the bucket, and with it
+// how many blocks of 8 warps an SM holds: 4 up to kGradUnits0, 3 up to
+// kGradUnits1, else 2 (buckets 0-2).  With a fixed stack of 7 slots and buckets
+// of 4, 8 and 16 constants 59, 28 and 13% of the words of a Pagie-1 population
+// (depth 4-10) ran at 32, 24 and 16 warps per SM, now 80, 14 and 6%.  Stacks of
+// more than kSmallDepth values (bucket 3): 4 warps, 19 slots and 16 constants,
+// the sums in registers.
 // Programs without constants (and without the extended functions, stack
 // depth <= 8) need no tangents: they form order class kGradBuckets and
 // run through the evaluator, which writes their loss partials.
 constexpr int kGradBuckets = 4;
-constexpr int kGradTan0 = 4, kGradTan1 = 8;
+constexpr int kGradUnits0 = 51, kGradUnits1 = 70;
+__host__ __device__ constexpr int grad_units(int n_consts, int depth) {
+    return 4 * (depth - 1) + 5 * n_consts;
+}
 __host__ __device__ inline int grad_bucket(int n_consts, int depth, int ext) {
     if (depth > kSmallDepth) return 3;
     if (n_consts == 0 && !ext) return kGradBuckets;
-    return n_consts <= kGradTan0 ? 0 : (n_consts <= kGradTan1 ? 1 : 2);
+    const int u = grad_units(n_consts, depth);
+    return u <= kGradUnits0 ? 0 : (u <= kGradUnits1 ? 1 : 2);
 }
 // classes of the program order (evaluator classes or gradient buckets)
 constexpr int kOrderClasses = 5;
@@ -392,6 +401,7 @@ struct GradArgs {
     int n_chunks;
     unsigned long long *counter;  // [kGradBuckets] work-queue counters, one per bucket
     int vec_ok;                   // X, y, w and the row counts allow 16-byte row loads
+    int x_unit, follows;          // as in EvalArgs
     float *part;   // [P][n_chunks] loss sums
     float *gpart;  // [P][n_chunks][16]
     unsigned int *dev_status;

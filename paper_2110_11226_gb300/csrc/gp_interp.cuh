@@ -111,46 +111,7 @@ __device__ __forceinline__ void unpack2(uint64_t r, float &a, float &b) {
     asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(r));
 }
 
-// RPT consecutive rows starting at r0 of one column; rows >= re read 0.
-template <int RPT>
-__device__ __forceinline__ void load_rows(float (&v)[RPT], const float *__restrict__ col,
-                                          int64_t r0, int64_t re, bool vec) {
-    if (vec && r0 + RPT <= re) {
-#pragma unroll
-        for (int q = 0; q < RPT / 4; ++q) {
-            const float4 f = __ldg(reinterpret_cast<const float4 *>(col + r0) + q);
-            v[4 * q + 0] = f.x;
-            v[4 * q + 1] = f.y;
-            v[4 * q + 2] = f.z;
-            v[4 * q + 3] = f.w;
-        }
-    } else {
-#pragma unroll
-        for (int j = 0; j < RPT; ++j) v[j] = (r0 + j < re) ? __ldg(col + r0 + j) : 0.0f;
-    }
-}
-
-// RPT consecutive rows of one column from p; with vec all of them as
-// 16-byte loads, otherwise the first nv rows one by one and 0 after them
-template <int RPT>
-__device__ __forceinline__ void load_chunk_rows(float (&v)[RPT], const float *__restrict__ p,
-                                                bool vec, int nv) {
-    if (vec) {
-#pragma unroll
-        for (int q = 0; q < RPT / 4; ++q) {
-            const float4 f = __ldg(reinterpret_cast<const float4 *>(p) + q);
-            v[4 * q + 0] = f.x;
-            v[4 * q + 1] = f.y;
-            v[4 * q + 2] = f.z;
-            v[4 * q + 3] = f.w;
-        }
-    } else {
-#pragma unroll
-        for (int j = 0; j < RPT; ++j) v[j] = (j < nv) ? __ldg(p + j) : 0.0f;
-    }
-}
-
-// The evaluator's rows of a lane as pairs.  packed: RPT consecutive rows
+// A lane's rows as pairs.  packed: RPT consecutive rows
 // from p, 16-byte loads; else rows p[0], p[32], p[64], ..., the last of them
 // at most p[last] (a ragged sub-tile reads its last row again; those rows
 // do not count).

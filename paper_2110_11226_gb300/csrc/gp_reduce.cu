@@ -95,8 +95,10 @@ cudaError_t launch_finalize(const FinalizeArgs &a, cudaStream_t st) {
     return launch_chained(finalize_kernel, grid, warps * 32, 0, st, a);
 }
 
-// constant gradients: same order; grad = S_g / S_w, RMSE scaled by 1/(2 RMSE)
+// constant gradients: a slot's even and odd chunks by two lanes; grad = S_g / S_w, RMSE scaled by 1/(2 RMSE)
 __global__ void __launch_bounds__(256) grad_finalize_kernel(GradFinalizeArgs a) {
+    griddep_wait();
+    griddep_launch();
     const int lane = threadIdx.x & 31;
     const int p = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
     if (p >= a.n_progs) return;
@@ -109,11 +111,17 @@ __global__ void __launch_bounds__(256) grad_finalize_kernel(GradFinalizeArgs a) 
     const double nan = __longlong_as_double(0x7ff8000000000000LL);
     double scale = 1.0 / sw;
     if (a.metric == GP_RMSE) scale = (f > 0.0) ? scale / (2.0 * f) : 0.0;
-    // lanes 0..15 each finish one constant slot
+    // lanes l and l + 16 add constant slot l's even and odd chunks, lane l
+    // finishes it
+    static_assert(GP_MAX_CONSTS == 16, "two lanes per slot");
     double g = 0.0;
-    if (lane < GP_MAX_CONSTS) {
+    if ((lane & 15) < m.n_consts) {
         const float *gp = a.gpart + (size_t)p * a.n_chunks * GP_MAX_CONSTS + lane;
-        for (int i = 0; i < a.n_chunks; ++i) g += (double)gp[(size_t)i * GP_MAX_CONSTS];
+#pragma unroll 4
+        for (int i = 0; i < a.n_chunks - (lane >> 4); i += 2) g += (double)gp[(size_t)i * GP_MAX_CONSTS];
+    }
+    g += __shfl_down_sync(0xffffffffu, g, 16);
+    if (lane < GP_MAX_CONSTS) {
         g = (lane < m.n_consts) ? g * scale : 0.0;
         if (bad) g = nan;
         a.grad[(size_t)p * GP_MAX_CONSTS + lane] = (float)g;
@@ -125,8 +133,7 @@ cudaError_t launch_grad_finalize(const GradFinalizeArgs &a, cudaStream_t st) {
     if (a.n_progs <= 0) return cudaSuccess;
     const int warps = 8;
     const int grid = (a.n_progs + warps - 1) / warps;
-    grad_finalize_kernel<<<grid, warps * 32, 0, st>>>(a);
-    return cudaGetLastError();
+    return launch_chained(grad_finalize_kernel, grid, warps * 32, 0, st, a);
 }
 
 }  // namespace gpk
