@@ -670,15 +670,15 @@ def main():
                                 "long_rows_per_thread": used.long_rows_per_thread if used.long_edge > 0 else None,
                                 "long_blocks_per_sm": (used.long_blocks_per_sm or "max resident")
                                 if used.long_edge > 0 else None,
-                                "classes_1_to_3_rows_per_thread": 4, "autotuned": tuned is not None,
+                                "classes_1_and_3_rows_per_thread": 4, "autotuned": tuned is not None,
                                 "autotune_seconds": tune_s, "untuned": untuned}},
             "node_evals_per_s": value * (n_nodes / P),
             "finite_fitness_frac": fin,
             "clocks": clocks,
-            # per step: compile, order, weight sum (+1 with weights), four
-            # evaluator launches (program classes; +1 when the common class is
-            # split by length), finalize, tournament
-            "gpu_launches": (9 + (d.w is not None) + (used.long_edge > 0)) * args.steps,
+            # per step: compile, order, four evaluator launches (program
+            # classes; +1 when the common class is split by length), finalize,
+            # tournament; with weights their sum
+            "gpu_launches": (8 + (d.w is not None) + (used.long_edge > 0)) * args.steps,
             "roofline": roof,
             "pipes": pipes}
 
