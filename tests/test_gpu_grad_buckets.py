@@ -77,3 +77,46 @@ def test_gradient_at_the_bucket_edges(n_feat, n_rows):
     # whole: no cancellation, at most some 60 roundings in a row
     np.testing.assert_allclose(fit.cpu().numpy(), fits, rtol=1e-5)
     np.testing.assert_allclose(grad.cpu().numpy(), want.numpy(), rtol=1e-5, atol=0)
+
+
+def test_back_to_back_gradients():
+    """Gradients, evaluations and Adam steps with nothing waiting between them,
+    and captured, equal each call alone."""
+    import torch
+
+    from paper_2110_11226_gb300 import gp
+    g = torch.Generator(device="cuda").manual_seed(3)
+    n, n_feat = 4099, 5
+    X = torch.randn(n_feat, n, generator=g, device="cuda")
+    y = torch.randn(n, generator=g, device="cuda")
+    w = torch.rand(n, generator=g, device="cuda") + 0.5
+    pops = []
+    for i in range(3):
+        nodes, off = synth.ramped_half_and_half(100 + 150 * i, 2, 7, synth.FULL_SET, n_feat, seed=i, max_consts=16)
+        pops.append((gp.nodes_to_device(nodes), torch.from_numpy(off).cuda()))
+    want = []
+    for nodes, off in pops:
+        for ww in (None, w):
+            torch.cuda.synchronize()
+            grad, fit = gp.gp_const_grad(nodes, off, X, y, ww, "mse")
+            torch.cuda.synchronize()
+            want.append((grad.cpu(), fit.cpu(), gp.gp_evaluate(nodes, off, X, y, ww, "mse").cpu()))
+
+    def run(out):
+        for nodes, off in pops:
+            for ww in (None, w):
+                grad, fit = gp.gp_const_grad(nodes, off, X, y, ww, "mse")
+                out.append((grad, fit, gp.gp_evaluate(nodes, off, X, y, ww, "mse")))
+
+    got = []
+    for _ in range(4):
+        run(got)
+    graph, captured = torch.cuda.CUDAGraph(), []
+    with torch.cuda.graph(graph):
+        run(captured)
+    for _ in range(3):
+        graph.replay()
+    torch.cuda.synchronize()
+    for i, tensors in enumerate(got + captured):
+        for a, b in zip(tensors, want[i % len(want)]):
+            assert torch.equal(a.cpu().nan_to_num(-1.0), b.nan_to_num(-1.0)), i
