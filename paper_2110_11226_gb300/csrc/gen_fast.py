@@ -31,11 +31,11 @@ slots and marker shapes.
 
 Variants: RPT in {4, 8} x ext (tan, sq, cube, max and min run here too) x XREG
 (columns 0 and 1 held in registers; without it a column read takes the rows
-that were prefetched for it and prefetches the next one's).  A word the loop does not run -- END, the other
-extended functions, the trigonometric and exponential arguments outside
-their fast paths, and whatever the variant leaves out -- is handed back to
-the caller's switch with its constant, the address just past it, and the rows
-untouched.
+that were prefetched for it and prefetches the next one's).  A word the loop
+does not run -- END, the other extended functions, the trigonometric and
+exponential arguments outside their fast paths, and whatever the variant
+leaves out -- is handed back to the caller's switch with its constant, the
+address just past it, and the rows untouched.
 
 Run: python paper_2110_11226_gb300/csrc/gen_fast.py  (rewrites gp_fast.cuh)
 """
