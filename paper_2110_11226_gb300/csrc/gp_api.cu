@@ -223,6 +223,17 @@ int x_unit(int n_feat, int64_t ld, bool vec) {
     return n_feat <= 2 || (int64_t)n_feat * ld * 4 / unit >= ((int64_t)1 << 32) ? 0 : (int)unit;
 }
 
+// The table as the evaluator reads it.  Feature mode 2 (at most two columns)
+// holds columns 0 and 1 of a lane's rows in registers, whatever the programs
+// name: it reads X and X + ld, so the stride of a one-column table is 0.
+void set_table(EvalArgs *ea, const float *X, int64_t n_rows, int n_feat, int64_t ld, bool vec) {
+    ea->X = X;
+    ea->ld = n_feat == 1 ? 0 : ld;
+    ea->n_rows = n_rows;
+    ea->vec_ok = vec ? 1 : 0;
+    ea->x_unit = x_unit(n_feat, ld, vec);
+}
+
 struct Plan {
     gp_eval_opts o;
     int n_chunks;
@@ -285,9 +296,7 @@ int run_evaluate(const gp_node *progs, const int32_t *offsets, int n_progs, cons
         ea.order = W.order;
         ea.class_count = W.class_count;
         ea.cls = cls;
-        ea.X = X;
-        ea.ld = (fmode == 2) ? (n_feat == 2 ? ld : 0) : ld;
-        ea.n_rows = n_rows;
+        set_table(&ea, X, n_rows, n_feat, ld, vec);
         ea.y = y;
         ea.w = w;
         ea.n_progs = n_progs;
@@ -299,8 +308,6 @@ int run_evaluate(const gp_node *progs, const int32_t *offsets, int n_progs, cons
         ea.counter = W.counters + (ea.sub == 1 ? kNumClasses : cls);
         ea.part = W.part;
         ea.dev_status = c->status;
-        ea.vec_ok = vec ? 1 : 0;
-        ea.x_unit = x_unit(n_feat, ea.ld, vec);
         if (mom) {
             ea.mom = W.mom;
             ea.shift = W.shift;
@@ -385,9 +392,7 @@ int run_predict_compiled(const Workspace &W, int p0, int b, const float *X, int6
         ea.order = W.order;
         ea.class_count = W.class_count;
         ea.cls = cls;
-        ea.X = X;
-        ea.ld = (fmode == 2) ? (n_feat == 2 ? n_rows : 0) : n_rows;
-        ea.n_rows = n_rows;
+        set_table(&ea, X, n_rows, n_feat, n_rows, vec);
         ea.n_progs = b;
         ea.metric = GP_MSE;
         ea.chunk_rows = chunk;
@@ -395,8 +400,6 @@ int run_predict_compiled(const Workspace &W, int p0, int b, const float *X, int6
         ea.counter = W.counters + cls;
         ea.pred = out_pred;
         ea.dev_status = c->status;
-        ea.vec_ok = vec ? 1 : 0;
-        ea.x_unit = x_unit(n_feat, ea.ld, vec);
         if ((cls == kClassShallow || cls == kClassShallowExt) && rpt == 8) {
             // the class-0 instance at 8 rows per thread (its store epilogue)
             const int occ = eval_info(8, fmode, cls, kEvalBlockThreads, nullptr, false, true);
@@ -789,9 +792,7 @@ int gp_const_grad(const gp_node *progs, const int32_t *offsets, int n_progs, con
         ea.cls = kClassShallow8;
         ea.qcls = kGradBuckets + 1;
         ea.follows = 1;
-        ea.X = X;
-        ea.ld = n_rows;
-        ea.n_rows = n_rows;
+        set_table(&ea, X, n_rows, n_feat, n_rows, vec);
         ea.y = y;
         ea.w = w;
         ea.n_progs = n_progs;
@@ -801,8 +802,6 @@ int gp_const_grad(const gp_node *progs, const int32_t *offsets, int n_progs, con
         ea.counter = W.counters + kGradBuckets;
         ea.part = W.part;
         ea.dev_status = c->status;
-        ea.vec_ok = vec ? 1 : 0;
-        ea.x_unit = x_unit(n_feat, ea.ld, vec);
         const int fmode = (n_feat <= 2) ? 2 : 0;
         const int occ = eval_info(4, fmode, kClassShallow8, kEvalBlockThreads, nullptr);
         GP_CUDA(eval_launch(ea, 4, fmode, c->sms * std::max(occ, 1), kEvalBlockThreads, st));
