@@ -24,8 +24,9 @@ def lib(tmp_path):
     if shutil.which("g++") is None or not os.path.exists(os.path.join(cuda, "cuda_runtime.h")):
         pytest.skip("g++ and the CUDA headers are needed")
     so = str(tmp_path / "recorded.so")
-    subprocess.run(["g++", "-std=c++17", "-O1", "-fPIC", "-shared", "-I" + build.INCLUDE, "-I" + build.CSRC,
-                    "-I" + cuda, os.path.join(HERE, "recorded_launches.cpp"), "-o", so], check=True)
+    # (-Bsymbolic: its own stand-ins, whatever else the process has loaded)
+    subprocess.run(["g++", "-std=c++17", "-O1", "-fPIC", "-shared", "-Wl,-Bsymbolic", "-I" + build.INCLUDE,
+                    "-I" + build.CSRC, "-I" + cuda, os.path.join(HERE, "recorded_launches.cpp"), "-o", so], check=True)
     lib = C.CDLL(so)
     lib.recorded.restype = C.c_char_p
     lib.memory_limit.argtypes = [C.c_size_t]
