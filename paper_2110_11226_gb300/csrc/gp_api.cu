@@ -282,9 +282,8 @@ int run_evaluate(const gp_node *progs, const int32_t *offsets, int n_progs, cons
         tev = timing_pair();
         GP_CUDA(cudaEventRecord(tev.first, st));
     }
-    // launches: the deep programs and class 3, rare and slow, first, so that
-    // they run beside the others; then class 2, then class 0 (split by length:
-    // its long programs, then the rest)
+    // launches: the deep programs and class 3, then class 2, then class 0
+    // (split by length: its long programs, then the rest)
     constexpr int kLaunches[] = {kClassDeep, kClassShallow8, kClassShallowExt, -1, kClassShallow};
     for (int i = 0; i < 5; ++i) {
         const int launch = kLaunches[i];
@@ -304,7 +303,6 @@ int run_evaluate(const gp_node *progs, const int32_t *offsets, int n_progs, cons
         ea.chunk_rows = pl.o.chunk_rows;
         ea.n_chunks = pl.n_chunks;
         ea.sub = split && cls == kClassShallow ? (launch < 0 ? 1 : 2) : 0;
-        ea.follows = i > 0;
         ea.counter = W.counters + (ea.sub == 1 ? kNumClasses : cls);
         ea.part = W.part;
         ea.dev_status = c->status;
@@ -386,7 +384,6 @@ int run_predict_compiled(const Workspace &W, int p0, int b, const float *X, int6
     const int fmode = (n_feat <= 2) ? 2 : 0;
     for (int cls : {kClassDeep, kClassShallow8, kClassShallowExt, kClassShallow}) {
         EvalArgs ea{};
-        ea.follows = cls != kClassDeep;
         ea.code = W.code + (size_t)p0 * kCodeStride;
         ea.meta = W.meta + p0;
         ea.order = W.order;
@@ -756,7 +753,6 @@ int gp_const_grad(const gp_node *progs, const int32_t *offsets, int n_progs, con
                      (chunk % 4 == 0);
     for (int bucket = kGradBuckets - 1; bucket >= 0; --bucket) {
         GradArgs ga{};
-        ga.follows = bucket < kGradBuckets - 1;
         ga.x_unit = x_unit(n_feat, n_rows, vec);
         ga.code = W.code;
         ga.meta = W.meta;
@@ -791,7 +787,6 @@ int gp_const_grad(const gp_node *progs, const int32_t *offsets, int n_progs, con
         // compiled stacks of up to kSmallDepth values: the 7-slot instance
         ea.cls = kClassShallow8;
         ea.qcls = kGradBuckets + 1;
-        ea.follows = 1;
         set_table(&ea, X, n_rows, n_feat, n_rows, vec);
         ea.y = y;
         ea.w = w;

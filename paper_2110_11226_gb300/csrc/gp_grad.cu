@@ -356,8 +356,7 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) grad_kernel(const GradArgs a
         }
         s_item[slot] = it;
     };
-    if (a.follows) __threadfence();  // see eval_kernel
-    else griddep_wait();
+    griddep_wait();
     griddep_launch();
     if (threadIdx.x == 0) {
         int begin = 0;
@@ -514,7 +513,6 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) grad_kernel(const GradArgs a
                 ok ? v : __int_as_float(0x7fc00000);
         }
     }
-    if (a.follows && blockIdx.x == 0) griddep_wait();  // see eval_kernel
 }
 
 template <int WARPS, int UNITS, int MINB, bool GREG, bool XREG>

@@ -213,8 +213,10 @@ size_t workspace_bytes_for(int n_progs, int64_t n_rows, int n_feat, const gp_eva
 // with programmatic stream serialization, so that its blocks may be set up
 // while the one before still runs, and waits for that one's completion
 // (griddep_wait) before it touches memory.  griddep_launch lets the next
-// kernel's set-up begin.  Every chained kernel waits, so the completion of the
-// last one is the completion of all.  512 programs x 4096 rows: 62 -> 52 us, with the
+// kernel's set-up begin.  Every chained kernel waits, also one that needs nothing
+// from the launch before it: what earlier launches wrote is only certain to be
+// visible after the wait, and the completion of the last one is then the
+// completion of all.  512 programs x 4096 rows: 62 -> 52 us, with the
 // host call 44 -> 34 us (also fewer runtime calls, see info_t).
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void griddep_launch() {
@@ -310,9 +312,6 @@ struct EvalArgs {
     // 0: the programs of class cls; k + 1: those of order class k (the
     // constant gradient's buckets: its constant-free programs)
     int qcls;
-    // 1: launched right after another launch of the same evaluation, on whose
-    // results it does not depend: it runs beside that one
-    int follows;
 };
 // One launcher per (rows per thread, feature mode) instance; a.cls picks
 // the program class (stack slots, extended functions).  fmode 2: columns 0 and 1 held in
@@ -401,7 +400,7 @@ struct GradArgs {
     int n_chunks;
     unsigned long long *counter;  // [kGradBuckets] work-queue counters, one per bucket
     int vec_ok;                   // X, y, w and the row counts allow 16-byte row loads
-    int x_unit, follows;          // as in EvalArgs
+    int x_unit;                   // as in EvalArgs
     float *part;   // [P][n_chunks] loss sums
     float *gpart;  // [P][n_chunks][16]
     unsigned int *dev_status;

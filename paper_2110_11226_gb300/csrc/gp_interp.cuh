@@ -493,11 +493,7 @@ __global__ void __launch_bounds__(eval_warps<RPT>() * 32,
         }
         s_item[slot] = it;
     };
-    // a launch that follows starts once every block of the first has passed its
-    // wait here, so what the kernels before that one wrote is in the L2 by
-    // then; the fence keeps this block's loads from older lines in its L1
-    if (a.follows) __threadfence();
-    else griddep_wait();
+    griddep_wait();
     griddep_launch();
     const float ybar = MOM ? (float)a.ystat[3] : 0.0f;
     if (threadIdx.x == 0) {
@@ -669,8 +665,6 @@ __global__ void __launch_bounds__(eval_warps<RPT>() * 32,
             a.part[(size_t)p * a.n_chunks + chunk] = ok ? v : __int_as_float(0x7fc00000);
         }
     }
-    // complete only after the launch that this one follows
-    if (a.follows && blockIdx.x == 0) griddep_wait();
 }
 
 // Resident blocks per SM, after making the instance's shared memory
