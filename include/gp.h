@@ -27,8 +27,11 @@
  *     the device (a malformed program) never trap: they set bits of a
  *     device status word (gp_last_device_status) and NaN results.
  *   - Floating point: evaluation in FP32 (IEEE +,-,*,/ and sqrt, CUDA's
- *     accurate libm functions, no contraction into FMA); the cross-block
- *     fitness sum in FP64.
+ *     accurate libm functions, no contraction of a program's operations into
+ *     FMA); a row's squared error is rounded, then multiplied by its weight
+ *     (a square past the float range is infinite, and NaN under a zero
+ *     weight), and such a term may join its sum in one rounding; the
+ *     cross-block fitness sum in FP64.
  */
 #ifndef GP_H_
 #define GP_H_

@@ -154,8 +154,11 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
 
 // the weighted losses of a lane's rows added up (the first nv rows count);
 // the metric and the weights are tested once, not per row.  The squares of
-// whole sub-tiles are added as they are formed, without a rounding of their
-// own, even and odd rows apart (9 instructions for 8 rows instead of 24)
+// whole sub-tiles (their products with the weights) are added as they are
+// formed, without a rounding of their own, even and odd rows apart (9
+// instructions for 8 rows instead of 24).  A weight multiplies the square, as
+// in the other branch: w d first would stay finite for some errors whose
+// square does not, in whole sub-tiles alone
 template <int RPT>
 __device__ __forceinline__ float loss_sum(int metric, const uint64_t (&tp)[RPT / 2],
                                           const uint64_t (&yp)[RPT / 2],
@@ -166,7 +169,7 @@ __device__ __forceinline__ float loss_sum(int metric, const uint64_t (&tp)[RPT /
 #pragma unroll
         for (int i = 0; i < RPT / 2; ++i) {
             const uint64_t d = sub2(tp[i], yp[i]);
-            e2 = fma2(has_w ? mul2(wp[i], d) : d, d, e2);
+            e2 = has_w ? fma2(wp[i], mul2(d, d), e2) : fma2(d, d, e2);
         }
         float lo, hi;
         unpack2(e2, lo, hi);
