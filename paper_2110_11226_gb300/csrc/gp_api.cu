@@ -39,6 +39,7 @@ struct DevCtx {
     size_t stage_bytes = 0;
     void *rank = nullptr;  // Spearman: predictions, sort buffers, target ranks
     size_t rank_bytes = 0;
+    size_t rank_refused = SIZE_MAX;  // the smallest `rank` that the device did not give
     std::map<ShapeKey, gp_eval_opts> tuned;
 };
 
@@ -98,6 +99,21 @@ int grow(void **ptr, size_t *cap, size_t need) {
     }
     *cap = want;
     return GP_OK;
+}
+
+// as grow, but what is there stays there until the larger buffer is: for a size
+// that the caller can do without
+bool try_grow(void **ptr, size_t *cap, size_t need) {
+    if (*cap >= need && *ptr) return true;
+    void *p = nullptr;
+    if (cudaMalloc(&p, need) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    if (*ptr) cudaFree(*ptr);
+    *ptr = p;
+    *cap = need;
+    return true;
 }
 
 inline cudaStream_t S(void *s) { return static_cast<cudaStream_t>(s); }
@@ -440,10 +456,11 @@ int run_predict(const gp_node *progs, const int32_t *offsets, int n_progs, const
 }
 
 // Spearman: the target's ranks once, then batches of programs predicted
-// into [B][N], ranked and reduced.  A batch takes up to 4.5 GB (at 1M rows
-// 160 programs, whose splitters are then sorted on every SM at once), or 2 GB
-// when the device has no room for that
-constexpr size_t kRankBudgets[] = {4608ull << 20, 2ull << 30};
+// into [B][N], ranked and reduced.  A batch takes up to 4.5 GB (at 2^20 rows
+// 164 programs, whose splitters are then sorted on every SM at once), or 2 GB
+// where the device does not give that; a size once refused is not asked for
+// again, so that a call of a shape that ran before allocates nothing
+constexpr size_t kRankBudget = 4608ull << 20, kRankBudgetSmall = 2ull << 30;
 
 int run_spearman(const gp_node *progs, const int32_t *offsets, int n_progs, const float *X,
                  int64_t n_rows, int n_feat, const float *y, const float *w, float *out,
@@ -453,19 +470,28 @@ int run_spearman(const gp_node *progs, const int32_t *offsets, int n_progs, cons
     const int64_t per_prog = n_rows * 4 + (int64_t)rank_scratch_bytes(1, n_rows, w != nullptr);
     const size_t b_r2y = (size_t)round_up(n_rows * 4, 256);
     const size_t b_tp = (size_t)round_up((int64_t)target_part_bytes(n_rows), 256);
-    int rc = GP_ERR_NOMEM, B = 0;
+    int B = 0;
     size_t b_pred = 0;
-    char *base = nullptr;
-    for (size_t budget : kRankBudgets) {
+    // programs per batch within the budget; the bytes that they take
+    auto plan = [&](size_t budget) {
         B = (int)std::max<int64_t>(1, std::min<int64_t>(n_progs, (int64_t)budget / per_prog));
         b_pred = (size_t)round_up((int64_t)B * n_rows * 4, 256);
-        const size_t b_scr = rank_scratch_bytes(B, n_rows, w != nullptr);
+        return b_pred + b_r2y + b_tp + rank_scratch_bytes(B, n_rows, w != nullptr);
+    };
+    int rc;
+    char *base = nullptr;
+    {
         std::lock_guard<std::mutex> g(g_mu);
-        rc = grow(&c->rank, &c->rank_bytes, b_pred + b_r2y + b_tp + b_scr);
+        const size_t least = plan(kRankBudgetSmall);
+        size_t need = plan(kRankBudget);
+        if (need > least && need > c->rank_bytes &&
+            (need >= c->rank_refused || !try_grow(&c->rank, &c->rank_bytes, need))) {
+            c->rank_refused = std::min(c->rank_refused, need);
+            need = plan(kRankBudgetSmall);
+        }
+        if ((rc = grow(&c->rank, &c->rank_bytes, need))) return rc;
         base = static_cast<char *>(c->rank);
-        if (rc == GP_OK) break;
     }
-    if (rc) return rc;
     float *pred = reinterpret_cast<float *>(base);
     uint32_t *r2y = reinterpret_cast<uint32_t *>(base + b_pred);
     double *tpart = reinterpret_cast<double *>(base + b_pred + b_r2y);
@@ -1098,6 +1124,7 @@ void gp_shutdown(void) {
         if (c.rank) cudaFree(c.rank);
         c.ws = c.stage = c.rank = nullptr;
         c.ws_bytes = c.stage_bytes = c.rank_bytes = 0;
+        c.rank_refused = SIZE_MAX;
         c.tuned.clear();
     }
     cudaSetDevice(cur);

@@ -66,3 +66,39 @@ def test_column_stride_of_every_evaluator_launch(lib, n_feat, n_rows):
         for a in launches:
             assert a["fmode"] == (2 if n_feat <= 2 else 0) and a["rows"] == n_rows
             assert a["ld"] == (0 if n_feat == 1 else n_rows), a
+
+
+@pytest.mark.parametrize("limit", [1 << 40, 7 << 29], ids=["room", "3.5 GB"])
+def test_rank_scratch_is_allocated_once(lib, limit):
+    """A population of several batches: where the device gives no 4.5 GB the
+    smaller batch runs, and the next call of the shape neither frees nor
+    allocates (it may be captured in a graph)."""
+    lib.memory_limit(limit)
+    for call in range(3):
+        assert _evaluate(lib, 512, 1_000_000, 2, SPEARMAN) == 0
+        lines = _lines(lib, "malloc", "free", "rank")
+        memory = [a for a in lines if a["kind"] != "rank"]
+        batches = [a["segments"] for a in lines if a["kind"] == "rank"]
+        assert sum(batches) == 512 and len(set(batches[:-1])) == 1
+        if call == 0:
+            big = [a for a in memory if a["bytes"] > 1 << 30]
+            assert [a["ok"] for a in big] == ([1] if limit > 1 << 33 else [0, 1])
+            first = batches
+        else:
+            assert memory == []
+            assert batches == first
+
+
+def test_refused_rank_scratch_leaves_what_is_held(lib):
+    """The larger batch is asked for beside the buffer that is there: when it
+    is refused and the buffer serves the smaller batch, nothing moves."""
+    lib.memory_limit(7 << 29)
+    assert _evaluate(lib, 512, 1_000_000, 2, SPEARMAN) == 0
+    small = max(a["segments"] for a in _lines(lib, "rank"))
+    lib.gp_shutdown()
+    lib.record_anew()
+    assert _evaluate(lib, small, 1_000_000, 2, SPEARMAN) == 0   # one batch, within the smaller budget
+    assert [a["ok"] for a in _lines(lib, "malloc") if a["bytes"] > 1 << 30] == [1]
+    assert _evaluate(lib, 512, 1_000_000, 2, SPEARMAN) == 0
+    lines = _lines(lib, "malloc", "free")
+    assert [(a["kind"], a.get("ok")) for a in lines if a["bytes"] > 1 << 30] == [("malloc", 0)]
