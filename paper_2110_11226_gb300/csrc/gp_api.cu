@@ -461,6 +461,7 @@ int run_predict(const gp_node *progs, const int32_t *offsets, int n_progs, const
 // where the device does not give that; a size once refused is not asked for
 // again, so that a call of a shape that ran before allocates nothing
 constexpr size_t kRankBudget = 4608ull << 20, kRankBudgetSmall = 2ull << 30;
+constexpr int64_t kRankBatch = 65535;  // a segment of the sort is a row of the grid
 
 int run_spearman(const gp_node *progs, const int32_t *offsets, int n_progs, const float *X,
                  int64_t n_rows, int n_feat, const float *y, const float *w, float *out,
@@ -474,7 +475,8 @@ int run_spearman(const gp_node *progs, const int32_t *offsets, int n_progs, cons
     size_t b_pred = 0;
     // programs per batch within the budget; the bytes that they take
     auto plan = [&](size_t budget) {
-        B = (int)std::max<int64_t>(1, std::min<int64_t>(n_progs, (int64_t)budget / per_prog));
+        B = (int)std::max<int64_t>(
+            1, std::min<int64_t>({(int64_t)n_progs, kRankBatch, (int64_t)budget / per_prog}));
         b_pred = (size_t)round_up((int64_t)B * n_rows * 4, 256);
         return b_pred + b_r2y + b_tp + rank_scratch_bytes(B, n_rows, w != nullptr);
     };

@@ -102,3 +102,12 @@ def test_refused_rank_scratch_leaves_what_is_held(lib):
     assert _evaluate(lib, 512, 1_000_000, 2, SPEARMAN) == 0
     lines = _lines(lib, "malloc", "free")
     assert [(a["kind"], a.get("ok")) for a in lines if a["bytes"] > 1 << 30] == [("malloc", 0)]
+
+
+@pytest.mark.parametrize("w", [None, P], ids=["unweighted", "weighted"])
+@pytest.mark.parametrize("n_rows", [1, 500, 2000, 3000])
+def test_rank_batch_fits_a_grid(lib, w, n_rows):
+    """A segment is a row of the sort's grid: at most 65535 of them."""
+    assert _evaluate(lib, 200_000, n_rows, 2, SPEARMAN, w) == 0
+    batches = [a["segments"] for a in _lines(lib, "rank")]
+    assert sum(batches) == 200_000 and max(batches) <= 65535
