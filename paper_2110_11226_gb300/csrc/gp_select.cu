@@ -1,6 +1,8 @@
 // gp_select.cu -- tournament selection on the device (Sec. III-C1): one
 // thread per tournament, k draws from Philox4x32-10, the best adjusted
 // fitness wins (Eqs. parsimony and fitness).
+#include <climits>
+
 #include <math_constants.h>
 
 #include "gp_internal.cuh"
@@ -13,14 +15,21 @@ namespace gpk {
 // 9.2 us now.
 constexpr int kTournThreads = 64;
 
+// groups of four draws of a tournament of k >= 1.  Counted without a sign: a
+// signed draw number in steps of four passes INT_MAX for the last three
+// values of k and would never end
+__host__ __device__ constexpr uint32_t draw_groups(int k) { return ((uint32_t)k + 3u) / 4u; }
+static_assert(draw_groups(1) == 1u && draw_groups(4) == 1u && draw_groups(5) == 2u, "groups of four");
+static_assert(draw_groups(INT_MAX) == 1u << 29 && draw_groups(INT_MAX - 2) == 1u << 29, "the largest k");
+
 __global__ void __launch_bounds__(kTournThreads) tournament_kernel(TournArgs a) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= a.n_tourn) return;
     const uint2 key = make_uint2((uint32_t)a.seed, (uint32_t)(a.seed >> 32));
     int best = -1;
     double best_adj = 0.0;
-    for (int j = 0; j < a.k; j += 4) {
-        const uint4 r = philox4x32_10(make_uint4((uint32_t)(j >> 2), (uint32_t)t, (uint32_t)a.offset,
+    for (uint32_t g = 0; g < draw_groups(a.k); ++g) {
+        const uint4 r = philox4x32_10(make_uint4(g, (uint32_t)t, (uint32_t)a.offset,
                                                  (uint32_t)(a.offset >> 32)),
                                       key);
         const uint32_t u[4] = {r.x, r.y, r.z, r.w};
@@ -49,7 +58,7 @@ __global__ void __launch_bounds__(kTournThreads) tournament_kernel(TournArgs a) 
                 if (isnan(adj)) adj = CUDART_INF;
                 better = best < 0 || adj < best_adj;
             }
-            if (better && j + q < a.k) {
+            if (better && 4u * g + q < (uint32_t)a.k) {
                 best = i[q];
                 best_adj = adj;
             }
