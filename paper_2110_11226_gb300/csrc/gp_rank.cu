@@ -16,6 +16,7 @@
 #include <type_traits>
 
 #include "gp_internal.cuh"
+#include "gp_rank_sample.cuh"
 
 namespace gpk {
 namespace {
@@ -623,24 +624,11 @@ cudaError_t radix_sort_values(const float *v, uint32_t *keys, uint32_t *vals, ui
 // programs takes 0.50 ms of predictions, 0.12 of splitters, 1.34 of
 // partition (tiles of 4096 keys or other block sizes: 1.42 to 1.65) and 1.42
 // of local ranks.
-constexpr int kBucketCap = 6144;
-constexpr int kBucketAim = kBucketCap / 3;
-constexpr int kMaxBuckets = 2048;
-constexpr int kOversample = 16;  // sampled keys per bucket
 constexpr int kPartThreads = 512, kPartItems = 16, kPartTile = kPartThreads * kPartItems;
 constexpr int kLocThreads = 512, kLocItems = kBucketCap / kLocThreads, kLocBins = 4096;
 constexpr int kLocKeys = 8192;   // kBucketCap to a power of two, for the bitonic sort
 constexpr int kCrowded = 128;  // keys in one bin that make the bucket sort
 
-static inline int pow2_at_least(int v) {
-    int p = 1;
-    while (p < v) p *= 2;
-    return p;
-}
-// a few thousand rows are one bucket, taken straight from the predictions
-static inline int bucket_count(int64_t n) {
-    return n <= kBucketCap ? 1 : (int)std::min<int64_t>((n + kBucketAim - 1) / kBucketAim, kMaxBuckets + 1);
-}
 // weighted sums are FP64 and need a fixed order; beyond kMaxBuckets the
 // partition's runs get too short
 static inline bool bucket_path(const float *w, int64_t n) {
@@ -681,8 +669,8 @@ __global__ void __launch_bounds__(1024) splitter_kernel(const float *__restrict_
     extern __shared__ uint32_t sample[];
     const int seg = blockIdx.x, t = threadIdx.x;
     const float *v = pred + (int64_t)seg * n;
-    for (int i = t; i < samples; i += blockDim.x)
-        sample[i] = float_key(v[((int64_t)(2 * i + 1) * n) / (2 * (int64_t)samples)]);
+    const int log2_samples = 31 - __clz(samples);
+    for (int i = t; i < samples; i += blockDim.x) sample[i] = float_key(v[sample_row(i, n, log2_samples)]);
     for (int j = t; j < B.nb; j += blockDim.x) {
         const int64_t q = (int64_t)seg * B.nb + j;
         B.cnt[q] = 0;
