@@ -628,7 +628,8 @@ constexpr int kPartThreads = 512, kPartItems = 16, kPartTile = kPartThreads * kP
 constexpr int kLocThreads = 512, kLocItems = kBucketCap / kLocThreads, kLocBins = 4096;
 constexpr int kLocKeys = 8192;   // kBucketCap to a power of two, for the bitonic sort
 constexpr int kTogether = 4;   // lanes with one key that add their sum at once
-constexpr int kCrowded = 128;  // keys in one bin that make the bucket sort
+constexpr int kBusy = 32;      // keys in one bin that make a look for bins of one value worth it
+constexpr int kCrowded = 128;  // keys in one bin of several values that make the bucket sort
 
 // weighted sums are FP64 and need a fixed order; beyond kMaxBuckets the
 // partition's runs get too short
@@ -884,6 +885,7 @@ __global__ void __launch_bounds__(kLocThreads, 3) local_kernel(
     extern __shared__ uint32_t keys[];  // [kLocKeys]
     __shared__ int32_t wsum[kLocThreads / 32];
     __shared__ uint32_t s_lo, s_hi;
+    __shared__ __align__(8) uint8_t mixed[kLocBins];  // 1: the bin holds several values
     __shared__ long long red[3][kLocThreads / 32];
     const int seg = DIRECT ? blockIdx.x : blockIdx.y, t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int64_t q = DIRECT ? 0 : (int64_t)seg * B.nb + blockIdx.x;
@@ -922,6 +924,7 @@ __global__ void __launch_bounds__(kLocThreads, 3) local_kernel(
     uint4 *bins4 = reinterpret_cast<uint4 *>(bins);
     static_assert(kLocBins == 8 * kLocThreads, "two uint4 of bins per thread");
     bins4[t] = bins4[kLocThreads + t] = make_uint4(0u, 0u, 0u, 0u);
+    reinterpret_cast<uint2 *>(mixed)[t] = make_uint2(0u, 0u);
     if (t == 0) {
         s_lo = 0xffffffffu;
         s_hi = 0u;
@@ -972,12 +975,33 @@ __global__ void __launch_bounds__(kLocThreads, 3) local_kernel(
         bins4[2 * t + 1] = make_uint4(at + x[4], at + x[5], at + x[6], at + x[7]);
         if (t == kLocThreads - 1) bins[kLocBins] = at + run;
     }
-    // a bin with many keys of one value is fine only where one value fills it
-    const bool crowded = __syncthreads_or(most > kCrowded && mult != 0u);
+    const bool busy = __syncthreads_or(most > kBusy && mult != 0u);
 #pragma unroll
     for (int r = 0; r < kLocItems; ++r) {
         if (r * kLocThreads >= m) break;
         if (r * kLocThreads + t < m) keys[bins[bin_of(key[r])] + off[r]] = key[r];
+    }
+    // Well-filled bins mostly hold one value that repeats, whose keys need no
+    // look at the others of the bin and make no bucket sort.  512 columns of
+    // 100003 values of two decimals took 2.9 ms with both, the plain sort 2.1,
+    // now 1.1; 2000 columns of 6000 distinct values 0.46 -> 0.48 (0.93)
+    bool crowded = false;
+    if (busy) {
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < kLocItems; ++r) {
+            if (r * kLocThreads >= m) break;
+            if (r * kLocThreads + t >= m) continue;
+            const uint32_t bin = bin_of(key[r]);
+            if (keys[bins[bin]] != key[r]) mixed[bin] = 1;
+        }
+        __syncthreads();
+        // the thread's 8 bins: one that is mixed and long?
+        bool many = false;
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            many |= mixed[8 * t + i] && bins[8 * t + i + 1] - bins[8 * t + i] > kCrowded;
+        crowded = __syncthreads_or(many);
     }
     if (crowded) {
         const int p2 = 1 << (32 - __clz(max(m - 1, 1)));
@@ -1014,10 +1038,13 @@ __global__ void __launch_bounds__(kLocThreads, 3) local_kernel(
             const uint32_t bin = bin_of(k);
             const int b0 = (int)bins[bin], b1 = (int)bins[bin + 1];
             less = b0;
-            same = 0;
-            for (int x = b0; x < b1; ++x) {
-                less += keys[x] < k;
-                same += keys[x] == k;
+            same = b1 - b0;
+            if (!busy || mixed[bin]) {
+                same = 0;
+                for (int x = b0; x < b1; ++x) {
+                    less += keys[x] < k;
+                    same += keys[x] == k;
+                }
             }
         }
         const long long a = 2ll * (base + less) + same + 1 - (n + 1);

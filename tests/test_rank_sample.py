@@ -93,3 +93,30 @@ def test_every_program_misjudged(lib, n, n_progs):
     want = np.where(np.arange(n_progs) == n_progs // 2, want[1], want[0])
     # the rounding of the FP32 result and of two FP64 evaluations
     np.testing.assert_allclose(got, want, rtol=1e-6, atol=1e-9)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n", [100, 4096, 6144, 16384, 200_003, 1_000_000])
+def test_repeated_values(n):
+    """Values that repeat (integers, decimals, a grid's axes), alone and among
+    others so close that they fall into the same bin; in each the ranks are
+    the definition's."""
+    import torch
+
+    from paper_2110_11226_gb300 import gp
+    rng = np.random.default_rng(n)
+    r, side = np.arange(n), int(n ** 0.5)
+    z = rng.standard_normal(n)
+    near = 1.0 + rng.integers(0, 40, n) * 2.0 ** -23
+    cols = [np.round(z, 2), rng.integers(0, 10000, n), rng.integers(0, 30, n), r % side, r // side,
+            np.where(rng.random(n) < 0.9, 0.0, z), np.where(rng.random(n) < 0.5, near, 1000.0 * z),
+            np.where(rng.random(n) < 0.02, 1.0 + 1e-5 * rng.random(n), np.round(1000.0 * z, 0)),
+            np.round(rng.standard_normal(n) ** 5, 1)]
+    X = np.stack(cols).astype(np.float32)
+    y = np.round(rng.standard_normal(n) + 0.2 * X[0], 2).astype(np.float32)
+    nodes, off = synth.pack([[(synth.OP["var"], f, 0.0)] for f in range(len(X))])
+    got = gp.gp_evaluate(gp.nodes_to_device(nodes), torch.from_numpy(off).cuda(), torch.from_numpy(X).cuda(),
+                         torch.from_numpy(y).cuda(), None, "spearman").cpu().numpy()
+    want = [oracle.spearman_of(c.astype(np.float64), y.astype(np.float64)) for c in X]
+    # the rounding of the FP32 result and of two FP64 evaluations
+    np.testing.assert_allclose(got, want, rtol=1e-6, atol=1e-9)
