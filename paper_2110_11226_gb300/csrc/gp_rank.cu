@@ -53,12 +53,13 @@ __device__ __forceinline__ uint32_t load_key(const void *src, int64_t m) {
 }
 
 // The segments that a kernel's blocks work on: all of them, one per
-// blockIdx.y, or, with a list on the device, the *count listed ones, taken
-// in turn by the gridDim.y rows of blocks.
+// blockIdx.y, or, with a list on the device, the *count listed ones of them,
+// taken in turn by the gridDim.y rows of blocks.
 struct Segs {
     const int32_t *list;
     const int32_t *count;
     int all;
+    unsigned rows(int64_t x) const { return (unsigned)(list ? listed_rows(all, x) : all); }
 };
 template <class F>
 __device__ __forceinline__ void each_segment(const Segs &sg, F body) {
@@ -573,9 +574,9 @@ __global__ void __launch_bounds__(32) target_total_kernel(const double *tpart, i
 cudaError_t radix_sort_values(const float *v, uint32_t *keys, uint32_t *vals, uint32_t *keys2,
                               uint32_t *vals2, int64_t n, int32_t *hist, int32_t *tot,
                               uint32_t *nan_flag, const uint32_t *payload, const Segs &sg,
-                              int rows_of_blocks, cudaStream_t st) {
+                              cudaStream_t st) {
     const int n_tiles = (int)((n + kSortTile - 1) / kSortTile);
-    const dim3 grid(n_tiles, rows_of_blocks), scan_grid(kBins / 8, rows_of_blocks);
+    const dim3 grid(n_tiles, sg.rows(n_tiles)), scan_grid(kBins / 8, sg.rows(kBins / 8));
     for (int pass = 0; pass < kPasses; ++pass) {
         const int shift = pass * kRadixBits;
         // pass 0: values -> keys2; then keys2 -> keys -> keys2 -> keys
@@ -1171,14 +1172,14 @@ RankScratch carve_rank(void *scratch, int n_seg, int64_t n, bool buckets, Bucket
 // the radix path's sort, tie groups and rank sums for the segments sg
 cudaError_t radix_ranks(const float *v, int64_t n, const RankScratch &r, const uint32_t *payload,
                         int mode, uint32_t *r2, const uint32_t *r2y, const float *w, double *part,
-                        uint32_t *nan_flag, const Segs &sg, int rows_of_blocks, cudaStream_t st) {
+                        uint32_t *nan_flag, const Segs &sg, cudaStream_t st) {
     const int64_t n_tiles = (n + kTile - 1) / kTile;
     cudaError_t e = radix_sort_values(v, r.keys, r.vals, r.keys2, r.vals2, n, r.hist, r.tot, nan_flag,
-                                      payload, sg, rows_of_blocks, st);
+                                      payload, sg, st);
     if (e != cudaSuccess) return e;
-    edges_kernel<<<dim3((unsigned)((n_tiles + 255) / 256), rows_of_blocks), 256, 0, st>>>(
-        r.keys, n, (int)n_tiles, r.edge, sg);
-    rank_kernel<<<dim3((unsigned)n_tiles, rows_of_blocks), kTileThreads, 0, st>>>(
+    const unsigned edge_blocks = (unsigned)((n_tiles + 255) / 256);
+    edges_kernel<<<dim3(edge_blocks, sg.rows(edge_blocks)), 256, 0, st>>>(r.keys, n, (int)n_tiles, r.edge, sg);
+    rank_kernel<<<dim3((unsigned)n_tiles, sg.rows(n_tiles)), kTileThreads, 0, st>>>(
         r.keys, r.vals, n, (int)n_tiles, mode, r.edge, r2, r2y, w, part, payload ? 1 : 0, sg);
     return cudaGetLastError();
 }
@@ -1201,7 +1202,7 @@ cudaError_t target_ranks(const float *y, const float *w, int64_t n, void *scratc
     const RankScratch r = carve_rank(scratch, 1, n, false, &B);
     cudaError_t e = cudaMemsetAsync(r.nan_flag, 0, 4, st);
     if (e != cudaSuccess) return e;
-    e = radix_ranks(y, n, r, nullptr, 0, r2y, nullptr, w, tpart, r.nan_flag, Segs{nullptr, nullptr, 1}, 1, st);
+    e = radix_ranks(y, n, r, nullptr, 0, r2y, nullptr, w, tpart, r.nan_flag, Segs{nullptr, nullptr, 1}, st);
     if (e != cudaSuccess) return e;
     target_total_kernel<<<1, 32, 0, st>>>(tpart, (int)n_tiles, tpart + 3 * n_tiles);
     return cudaGetLastError();
@@ -1225,9 +1226,8 @@ cudaError_t spearman_batch(const float *pred, int n_seg, int64_t n, const uint32
     // instead of gathering it by row
     const uint32_t *payload = w == nullptr ? r2y : nullptr;
     if (!buckets || B.nb > 1) {
-        const Segs sg = buckets ? Segs{B.list, B.count, 0} : Segs{nullptr, nullptr, n_seg};
-        e = radix_ranks(pred, n, r, payload, 1, nullptr, r2y, w, r.part, r.nan_flag, sg,
-                        buckets ? std::min(n_seg, 4) : n_seg, st);
+        const Segs sg = buckets ? Segs{B.list, B.count, n_seg} : Segs{nullptr, nullptr, n_seg};
+        e = radix_ranks(pred, n, r, payload, 1, nullptr, r2y, w, r.part, r.nan_flag, sg, st);
         if (e != cudaSuccess) return e;
     }
     spearman_final_kernel<<<(n_seg + 7) / 8, 256, 0, st>>>(r.part, buckets ? B.sums : nullptr, B.listed,

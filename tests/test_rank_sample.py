@@ -68,6 +68,16 @@ def test_no_bucket_overflows_on_structured_rows(lib, n):
         assert fullest <= lib.capacity(), name
 
 
+@pytest.mark.parametrize("n_seg", [1, 3, 600, 65535])
+@pytest.mark.parametrize("x", [1, 2, 4, 32, 245, 1024])
+def test_listed_segments_fill_the_device(lib, n_seg, x):
+    """blocks for every SM, or for every segment, and few that read a zero"""
+    rows = lib.listed_rows(C.c_int64(n_seg), C.c_int64(x))
+    assert 1 <= rows <= n_seg
+    assert rows * x >= min(n_seg * x, 4 * 152)
+    assert rows * x < max(4 * x, 4 * 152 + x) + 1
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("n,n_progs", [(8192, 700), (16384, 600), (200_003, 12), (1_000_000, 9)])
 def test_every_program_misjudged(lib, n, n_progs):
