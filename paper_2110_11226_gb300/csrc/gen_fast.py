@@ -84,7 +84,7 @@ def kp(name, neg=False):
 
 
 class Gen:
-    def __init__(self, rpt, xreg, ext=False, grad=False):
+    def __init__(self, rpt, xreg, ext=False, grad=False, special=True):
         self.rpt, self.xreg, self.ext, self.grad = rpt, xreg, ext, grad
         # columns in memory: the next column read is prefetched into XB
         self.xmem = not xreg
@@ -120,9 +120,8 @@ class Gen:
         self.slot_bytes = (rpt // 4) * 512
         self.lines = []
         self.resumes = {}     # marked column reads: their index in TD
-        # the special-value paths (4 rows per lane only: at 8 the loop's
-        # larger code made the evaluator 2.3% slower on Pagie-1 16M x 4096)
-        self.special = rpt == 4
+        # the special-value paths
+        self.special = special
         self.nsv = 0          # special-value paths emitted so far
         self.deferred = []    # their blocks, emitted after the bodies
 
@@ -318,7 +317,12 @@ class Gen:
     # variants only: in the others, wherever it stood, it made populations
     # without tan 1.5-5% slower (code size), so programs with tan run there
     def tan(self):
-        self.range_check("trig_fast", lo="two_m60")
+        def test(v):
+            # (NaN and infinities go through the steps: NaN)
+            self.beyond("trig_fast", v)
+            self.e(f"setp.lt.or.f32 %%p, %%m, {kf('two_m60')}, %%p;")
+        self.range_check("trig_fast", lo="two_m60",
+                         special=lambda: self.rows_test(lambda i: self.T[i], test))
         for i in range(self.np):
             t = self.T[i]
             self.e(f"mov.b64 %%K0, {kp('two_over_pi')};")
@@ -1201,12 +1205,12 @@ class Gen:
 
 
 
-def function(rpt, xreg, ext=False, grad=False):
-    g = Gen(rpt, xreg, ext, grad)
+def function(rpt, xreg, ext=False, grad=False, special=True):
+    g = Gen(rpt, xreg, ext, grad, special)
     lines = g.generate()
     p = rpt // 2
     name = f"fast_r{rpt}_{'ext' if ext else 'divs'}_{'x' if xreg else 'nox'}" + \
-        ("_grad" if grad else "")
+        ("_grad" if grad else "") + ("" if special else "_lean")
     body = "\n".join(f'        "{ln}\\n\\t"' for ln in lines)
     xmem = g.xmem
     outs = ", ".join(['"+r"(pa)'] + [f'"+l"(t[{i}])' for i in range(p)]
@@ -1236,7 +1240,8 @@ HEADER = '''// gp_fast.cuh -- the evaluator's indexed-branch fast loop in inline
 // in hw and hc, leaves pa just past it and the rows untouched by it.  sp is the
 // lane's next free slot of the shared-memory stack ([slot][q][lane] float4); a
 // division handed back has taken its operand off.  ext: with tan, sq, cube,
-// max and min.  The _x variants take columns 0
+// max and min.  _lean: without the paths for special values (NaN, infinities,
+// zero), which are handed back.  The _x variants take columns 0
 // and 1 of the lane's rows in x0 and x1; the _nox ones read columns from
 // memory: xb holds the rows of the column that the program reads next, xc
 // is column 0 at the lane's first row, a word's constant times unit the bytes
@@ -1263,6 +1268,10 @@ def main():
             for xreg in (True, False):
                 parts.append(function(rpt, xreg, ext))
                 parts.append("\n")
+    # the fitness of the common class at 8 rows
+    for xreg in (True, False):
+        parts.append(function(8, xreg, special=False))
+        parts.append("\n")
     # the constant gradient's loop (4 rows per lane, the division set)
     for xreg in (True, False):
         parts.append(function(4, xreg, grad=True))

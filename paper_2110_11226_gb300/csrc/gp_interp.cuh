@@ -249,7 +249,7 @@ static __device__ __noinline__ float4 ext_rows4(float4 v, uint32_t f) {
 // the other extended functions, arguments outside a fast path in any row of
 // the warp, column reads of a ragged sub-tile), hands that word and its
 // constant back to the switch below and leaves pa just past it.
-template <int RPT, bool EXT, bool XREG>
+template <int RPT, bool EXT, bool XREG, bool LEAN>
 __device__ __forceinline__ void run_fast(uint32_t &pa, uint64_t (&t)[RPT / 2],
                                          uint64_t (&x0)[RPT / 2], const uint64_t (&x1)[RPT / 2],
                                          const float *xc, uint32_t unit, uint32_t mode, uint32_t &sp,
@@ -260,7 +260,9 @@ __device__ __forceinline__ void run_fast(uint32_t &pa, uint64_t (&t)[RPT / 2],
         else if constexpr (XREG) fast_r4_ext_x(pa, t, x0, x1, sp, hw, hc);
         else fast_r4_ext_nox(pa, t, x0, xc, unit, mode, sp, hw, hc);
     } else {
-        if constexpr (!EXT && XREG) fast_r8_divs_x(pa, t, x0, x1, sp, hw, hc);
+        if constexpr (LEAN && XREG) fast_r8_divs_x_lean(pa, t, x0, x1, sp, hw, hc);
+        else if constexpr (LEAN) fast_r8_divs_nox_lean(pa, t, x0, xc, unit, mode, sp, hw, hc);
+        else if constexpr (!EXT && XREG) fast_r8_divs_x(pa, t, x0, x1, sp, hw, hc);
         else if constexpr (!EXT) fast_r8_divs_nox(pa, t, x0, xc, unit, mode, sp, hw, hc);
         else if constexpr (XREG) fast_r8_ext_x(pa, t, x0, x1, sp, hw, hc);
         else fast_r8_ext_nox(pa, t, x0, xc, unit, mode, sp, hw, hc);
@@ -288,7 +290,7 @@ __device__ __forceinline__ void run_fast(uint32_t &pa, uint64_t (&t)[RPT / 2],
 // covers all 32 values of its 5-bit operand, so it needs no range test;
 // and the word is loaded when it is needed rather than one ahead, which
 // saves the register copies of a prefetch.
-template <int RPT, int NSLOT, int FMODE, bool EXT>
+template <int RPT, int NSLOT, int FMODE, bool EXT, bool LEAN>
 __device__ __forceinline__ void interpret(uint64_t (&tp)[RPT / 2], const uint2 *__restrict__ cbuf,
                                           uint64_t (&x0p)[RPT / 2],
                                           const uint64_t (&x1p)[RPT / 2],
@@ -315,7 +317,7 @@ __device__ __forceinline__ void interpret(uint64_t (&tp)[RPT / 2], const uint2 *
         uint2 ins;
         if constexpr (kFast) {
             float hc;
-            run_fast<RPT, EXT, FMODE == 2>(pa, tp, x0p, x1p, xc, unit, mode, sp, ins.x, hc);
+            run_fast<RPT, EXT, FMODE == 2, LEAN>(pa, tp, x0p, x1p, xc, unit, mode, sp, ins.x, hc);
             ins.y = __float_as_uint(hc);
         } else {
             asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];"
@@ -465,6 +467,13 @@ __global__ void __launch_bounds__(eval_warps<RPT>() * 32,
     eval_kernel(const EvalArgs a) {
     constexpr bool PRED = EPI == kEpiPred;
     constexpr bool MOM = EPI == kEpiMom;
+    // Special values (NaN, infinities, zero) run in the loop, except for the
+    // fitness of class 0 at 8 rows, where the paths' code cost 2.3% (Pagie-1 16M
+    // x 4096) and a program that meets many has no fitness.  Handed back,
+    // they took most words of a table with 1% of NaN out of the loop:
+    // predictions of 512 programs, 200000 rows x 5 columns, 1.14 -> 0.46 ms, over
+    // the paper's set 2.23 -> 0.66; without NaN no difference
+    constexpr bool kLean = RPT == 8 && !EXT && !PRED;
     constexpr int kEvalWarps = eval_warps<RPT>();
     constexpr int kEvalBlock = kEvalWarps * 32;
     extern __shared__ float4 smem_eval[];
@@ -579,7 +588,7 @@ __global__ void __launch_bounds__(eval_warps<RPT>() * 32,
                     load_pairs<RPT, FMODE>(x1, xr + a.ld, packed, last);
                 }
                 const uint32_t mode = a.x_unit == 0 || !whole ? 2u : packed ? 0u : 1u;
-                interpret<RPT, NSLOT, FMODE, EXT>(t, cbuf, x0, x1, xr, a.ld, (uint32_t)a.x_unit, mode,
+                interpret<RPT, NSLOT, FMODE, EXT, kLean>(t, cbuf, x0, x1, xr, a.ld, (uint32_t)a.x_unit, mode,
                                                   packed, last, stk, aux);
             }
             // the lane's first row again; in feature mode 0 from the item, as held
