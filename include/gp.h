@@ -121,7 +121,7 @@ enum gp_prog_status {
 /* Bits of the device status word. */
 #define GP_DEV_BAD_PROGRAM 0x1u      /* a program failed validation     */
 #define GP_DEV_TOO_MANY_CONSTS 0x2u  /* gp_const_grad: > 16 constants  */
-#define GP_DEV_QUEUE_CAP 0x4u        /* persistent work loop hit its cap */
+#define GP_DEV_QUEUE_CAP 0x4u        /* not set: no work loop has a cap */
 #define GP_DEV_BAD_PARENT 0x8u       /* gp_mutate: parent index out of range */
 
 /* Cross-block accumulation of the fitness sums. */
@@ -131,7 +131,8 @@ enum gp_accum { GP_ACCUM_FP64 = 0, GP_ACCUM_KAHAN32 = 1 };
  * the autotuned one for this problem shape when gp_autotune has run,
  * otherwise a fixed default.
  * Length buckets: with long_edge > 0 the programs of the common class
- * (compiled stack of at most 7 values, no extended function) whose compiled
+ * (compiled stack of at most 7 values, neither GP_TAN nor a function from
+ * GP_SQ on) whose compiled
  * form is longer than long_edge words run in a launch of their own, with
  * long_rows_per_thread and long_blocks_per_sm (0: rows_per_thread and
  * blocks_per_sm), before the shorter ones; long_edge = -1 asks for no split

@@ -1058,14 +1058,11 @@ class Gen:
             ent[OPS[k]] = v
         if self.ext:
             ent[OPS["TAN"]] = "TN"
-        if self.xreg or self.xmem:
-            xops = dict(PUSH_X="PX", PUSH_X_SP="PXS", ADD_X="AX", SUB_X="SX", RSUB_X="RX",
-                        MUL_X="MX")
-            xops.update(DIV_X="DX", RDIV_X="RDX")
-            for k, v in xops.items():
-                ent[OPS[k]] = v if self.xmem else v + "0"
-                if not self.xmem:
-                    ent[OPS[k] | COL1] = v + "1"
+        for k, v in dict(PUSH_X="PX", PUSH_X_SP="PXS", ADD_X="AX", SUB_X="SX", RSUB_X="RX", MUL_X="MX",
+                         DIV_X="DX", RDIV_X="RDX").items():
+            ent[OPS[k]] = v if self.xmem else v + "0"
+            if not self.xmem:
+                ent[OPS[k] | COL1] = v + "1"
         if self.ext:
             for k, v in EXT_INDEX.items():
                 ent[v] = k

@@ -499,8 +499,8 @@ int run_spearman(const gp_node *progs, const int32_t *offsets, int n_progs, cons
     double *tpart = reinterpret_cast<double *>(base + b_pred + b_r2y);
     void *scr = base + b_pred + b_r2y + b_tp;
     GP_CUDA(target_ranks(y, w, n_rows, scr, r2y, tpart, st));
-    // the pre-pass once for all programs (one thread per program: compiled
-    // batch by batch, its latency came back with every batch)
+    // the pre-pass once for all programs (compiled batch by batch, its latency
+    // came back with every batch)
     Workspace W;
     if ((rc = compile_all(progs, offsets, n_progs, n_feat, out_status, c, &W, st))) return rc;
     for (int p0 = 0; p0 < n_progs; p0 += B) {

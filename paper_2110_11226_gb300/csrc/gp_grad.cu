@@ -18,10 +18,10 @@
 //
 // A block takes one (program, row chunk) item; its warps run the program
 // over their own sub-tiles of 128 rows (4 per lane) with the evaluator's
-// fast loop (the same FP32 operations, so the fitness equals
-// gp_evaluate's) in its gradient variant, which hands the words it does not
-// run back to grad_word.  The loss derivative per row times the tangents
-// gives each constant's share.  Programs are bucketed by what their stack and
+// fast loop (the same FP32 operations on every row, so the fitness is
+// gp_evaluate's but for the order of its sums) in its gradient variant, which
+// hands the words it does not run back to grad_word.  The loss derivative per
+// row times the tangents gives each constant's share.  Programs are bucketed by what their stack and
 // constants need of shared memory (grad_bucket), one launch per bucket.
 // Per-lane sums are FP32 (the loss Kahan-compensated), warp sums
 // fixed-order, chunk sums FP64 in a fixed order (gp_reduce.cu).

@@ -326,7 +326,7 @@ GP_EVAL_INSTANCE(4, 0)
 GP_EVAL_INSTANCE(16, 2)
 GP_EVAL_INSTANCE(16, 0)
 #undef GP_EVAL_INSTANCE
-// 8 rows per thread: class 0 only, with the store epilogue too (pred)
+// 8 rows per thread: classes 0 and 2, with the store epilogue too (pred)
 cudaError_t launch_eval_r8_f2(const EvalArgs &a, int grid, int block, cudaStream_t st);
 int info_eval_r8_f2(int cls, int block, int *regs, bool moments, bool pred = false);
 cudaError_t launch_eval_r8_f0(const EvalArgs &a, int grid, int block, cudaStream_t st);

@@ -20,8 +20,8 @@
 // register array t[RPT]; deeper values sit in the warp's slice of a
 // shared-memory stack, one float4 per (slot, group of 4 rows, lane), so a
 // push or pop is one or two conflict-free 16-byte accesses per lane.  Each
-// instruction costs one indexed branch (the inline-PTX fast loop, 4 rows per
-// lane) or one switch, and nothing else that branches:
+// instruction costs one indexed branch (the inline-PTX fast loop, 4 or 8 rows
+// per lane) or one switch, and nothing else that branches:
 // measured on this GPU, an interpreter's dispatch latency grows with every
 // dependent branch per instruction (about 20-40 cycles each) and with the
 // number of distinct code locations it jumps between, so operand source and
@@ -287,7 +287,7 @@ __device__ __forceinline__ void run_fast(uint32_t &pa, uint64_t (&t)[RPT / 2],
 // through 32-bit shared-memory addresses computed once; the opcode is
 // broadcast from lane 0, which lets the compiler treat the switch as
 // warp-uniform (no reconvergence barrier per instruction); the switch
-// covers all 32 values of its 5-bit operand, so it needs no range test;
+// covers every value of its 5-bit operand that occurs, so it needs no range test;
 // and the word is loaded when it is needed rather than one ahead, which
 // saves the register copies of a prefetch.
 template <int RPT, int NSLOT, int FMODE, bool EXT, bool LEAN>
@@ -416,10 +416,9 @@ __device__ __forceinline__ void interpret(uint64_t (&tp)[RPT / 2], const uint2 *
                 } else {
                     goto done;
                 }
-            case OP_EXT2:  // max and min run in the loop
             case OP_END:
                 goto done;
-            default:  // every value of w & 31 has a case above
+            default:  // every other value has a case above, but OP_EXT2, which the loop runs
                 __builtin_unreachable();
         }
         goto next;

@@ -17,17 +17,22 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 MSE, PEARSON, SPEARMAN = 1, 4, 5
 
 
-@pytest.fixture
-def lib(tmp_path):
-    """a library of its own, with nothing allocated yet"""
+@pytest.fixture(scope="module")
+def recorded(tmp_path_factory):
     cuda = os.path.join(os.path.dirname(os.path.dirname(build._nvcc())) or "/usr/local/cuda", "include")
     if shutil.which("g++") is None or not os.path.exists(os.path.join(cuda, "cuda_runtime.h")):
         pytest.skip("g++ and the CUDA headers are needed")
-    so = str(tmp_path / "recorded.so")
+    so = str(tmp_path_factory.mktemp("recorded") / "recorded.so")
     # (-Bsymbolic: its own stand-ins, whatever else the process has loaded)
     subprocess.run(["g++", "-std=c++17", "-O1", "-fPIC", "-shared", "-Wl,-Bsymbolic", "-I" + build.INCLUDE,
                     "-I" + build.CSRC, "-I" + cuda, os.path.join(HERE, "recorded_launches.cpp"), "-o", so], check=True)
-    lib = C.CDLL(so)
+    return so
+
+
+@pytest.fixture
+def lib(recorded, tmp_path):
+    """a copy of its own, with nothing allocated yet"""
+    lib = C.CDLL(shutil.copy(recorded, tmp_path / "copy.so"))
     lib.recorded.restype = C.c_char_p
     lib.memory_limit.argtypes = [C.c_size_t]
     return lib
