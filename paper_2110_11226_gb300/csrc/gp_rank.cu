@@ -604,27 +604,28 @@ cudaError_t radix_sort_values(const float *v, uint32_t *keys, uint32_t *vals, ui
 // ---- ranks by buckets --------------------------------------------------
 // Without weights the coefficient needs each value's rank only next to the
 // target's rank of its row, so no segment has to be sorted as a whole:
-//   splitter_kernel   a sorted sample of the segment's keys gives splitters
-//                     for buckets of about kBucketAim keys
+//   splitter_kernel   a sorted sample of the segment's keys (sample_row) gives
+//                     splitters for buckets of about kBucketAim keys
 //   partition_kernel  every key goes, with the target's rank of its row, to
 //                     its bucket (of at most kBucketCap places).  Keys equal
 //                     to a splitter -- every value frequent enough to fill a
 //                     bucket is one -- need no place: they share one rank, so
-//                     their number and the sum of their targets' ranks do
+//                     their number and the sum of their targets' ranks do,
+//                     counted per tile in shared memory
 //   base_kernel       first position of every bucket; the splitters' shares
 //   local_kernel      a bucket in shared memory: 4096 equal bins over its key
 //                     range, about one key each, then a key's rank is the
-//                     bin's start plus the smaller keys in the bin
+//                     bin's start plus the smaller keys in the bin (a bin
+//                     of one value that repeats: the bin's start)
 // The sums are integers and exact, so no order shows in them.  A segment
 // with an overfull bucket (the sample misjudged it) is listed, and the radix
 // sort below runs for the listed segments alone.
 // Bound by the global traffic of the partition (4 B read, 8 B written as runs
 // of about 6 keys, 8 B read) and shared-memory atomics; the radix sort moves
-// 84 B a key and spends about 800 instructions on it, these 158 and 208 in
-// the last two steps.  512 programs x 1M rows: 20.4 -> 10.9 ms; a batch of 156
-// programs takes 0.50 ms of predictions, 0.12 of splitters, 1.34 of
-// partition (tiles of 4096 keys or other block sizes: 1.42 to 1.65) and 1.42
-// of local ranks.
+// 84 B a key and spends about 800 instructions on it.  512 programs x 1M rows:
+// 20.5 -> 9.75 ms; a batch of 164 programs x 2^20 rows takes 0.71 ms of
+// predictions, 0.12 of splitters, 1.09 of partition (tiles of 4096 keys or
+// other block sizes: 6 to 23% more) and 1.43 of local ranks.
 constexpr int kPartThreads = 512, kPartItems = 16, kPartTile = kPartThreads * kPartItems;
 constexpr int kLocThreads = 512, kLocItems = kBucketCap / kLocThreads, kLocBins = 4096;
 constexpr int kLocKeys = 8192;   // kBucketCap to a power of two, for the bitonic sort
