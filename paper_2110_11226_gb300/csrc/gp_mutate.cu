@@ -277,6 +277,7 @@ __global__ void __launch_bounds__(kPlanWarps * 32) mutate_plan_kernel(const MutA
                 const int idx = pick(s, ns);
                 nd.op = ar == 1 ? a.unary[idx] : a.binary[idx];
             }
+            __syncwarp();  // every lane has read node m
             if (lane == 0) par.node[m] = bits_of(nd);
         }
         __syncwarp();
